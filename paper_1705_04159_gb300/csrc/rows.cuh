@@ -43,7 +43,6 @@ struct SweepArgs {
   int64_t n_other;      // rows of the other side (of Vo and its shadow)
   // per slot of the degree order: (row, first rating, one past the last, 0)
   const int4* work;
-  float* wsbase;        // base tiles of the persistent kernel (rows_ws.cu)
 };
 
 SweepArgs make_sweep_args(Handle* h, int s);

@@ -23,8 +23,9 @@
 //     accumulators instead, and the drain adds hi.lo and its transpose (two
 //     products per step);
 //   drain (warps 4-7, thread m = tensor-memory lane m = matrix row m):
-//     forms A = base + alpha G (base = bordered [[Lambda_s, b0], [b0^T, 0]])
-//     and writes its lower triangle as 8 x 8 FP32 tiles into a free
+//     forms A = base + alpha G (base = bordered [[Lambda_s, b0], [b0^T, 0]],
+//     kept in tensor memory, or in shared memory where the accumulators take
+//     all of it) and writes its lower triangle as 8 x 8 FP32 tiles into a free
 //     consumer slot, releasing the accumulator for the next row;
 //   consumers (warps 9.., one row each): blocked right-looking Cholesky of
 //     the slot (per 8-column panel: the diagonal tile in registers by every
@@ -86,6 +87,10 @@ struct WsNb {
 constexpr int64_t kWsCrossRow = 2048;
 template <bool XO>
 __host__ __device__ constexpr uint32_t ws_acc_stride() { return XO ? 256u : 128u; }  // TMEM columns per buffer
+// Tensor memory: two accumulators from column 0; without XO the base matrix
+// follows them (columns 256 .. 383), with XO they fill all 512 columns.
+constexpr uint32_t kWsTmemCols = 512;
+constexpr uint32_t kWsBaseCol = 256;
 __host__ __device__ constexpr int ws_stage_bytes(int nb) { return 2 * 2 * nb * 128; }
 constexpr int kWsMaxStages = 16;
 constexpr int kWsMaxCons = 7;
@@ -154,6 +159,7 @@ struct RowRec {
 struct WsShared {
   uint8_t* stages;
   float* slots;
+  float* base;  // base tiles (with XO only)
   uint16_t* sched;  // [32 * nround] lane units, then [g + 1] first round of each panel
   uint64_t* empty;
   uint64_t* tma;  // the stage's copies have landed (and its metadata and ratings are written)
@@ -182,19 +188,21 @@ __host__ __device__ inline int ws_fixed_bytes(int nb, int S, int C) {
   // barriers, stage meta, row records, ratings, next_row, abort, taddr
   return 8 * ws_nbar(S, C) + 16 * S + 16 * kWsRecs + 4 * S * nb + 32;
 }
-// stages, consumer slots, the trailing-update schedule, then the fixed part;
-// one atom more, to start the stages on a 1024-byte boundary (the swizzle
-// pattern follows address bits 7 .. 9)
-__host__ __device__ inline int ws_smem_bytes(const WsGeom& G, int S, int C, int nb) {
-  return kWsAtom + S * ws_stage_bytes(nb) + C * G.slot_floats() * 4 + G.sched_bytes() +
-         ws_fixed_bytes(nb, S, C);
+// stages, consumer slots, base tiles (with XO), the trailing-update schedule,
+// then the fixed part; one atom more, to start the stages on a 1024-byte
+// boundary (the swizzle pattern follows address bits 7 .. 9)
+__host__ __device__ inline int ws_smem_bytes(const WsGeom& G, int S, int C, int nb, bool cross) {
+  return kWsAtom + S * ws_stage_bytes(nb) + C * G.slot_floats() * 4 +
+         (cross ? G.ntile * kWsTileF * 4 : 0) + G.sched_bytes() + ws_fixed_bytes(nb, S, C);
 }
 
-__device__ __forceinline__ WsShared ws_carve(uint8_t* base, const WsGeom& G, int S, int C, int nb) {
+__device__ __forceinline__ WsShared ws_carve(uint8_t* base, const WsGeom& G, int S, int C, int nb,
+                                             bool cross) {
   WsShared w;
   w.stages = base;
   w.slots = reinterpret_cast<float*>(base + S * ws_stage_bytes(nb));
-  w.sched = reinterpret_cast<uint16_t*>(w.slots + C * G.slot_floats());
+  w.base = w.slots + C * G.slot_floats();
+  w.sched = reinterpret_cast<uint16_t*>(w.base + (cross ? G.ntile * kWsTileF : 0));
   uint8_t* p = reinterpret_cast<uint8_t*>(w.sched) + G.sched_bytes();
   uint64_t* b = reinterpret_cast<uint64_t*>(p);
   w.empty = b;
@@ -586,43 +594,55 @@ __device__ __forceinline__ void st8(float* p, const float (&x)[8]) {
   reinterpret_cast<float4*>(p)[1] = make_float4(x[4], x[5], x[6], x[7]);
 }
 
-// Base tiles (the bordered [[Lambda_s, b0], [b0^T, 0]] as lower 8 x 8 tiles,
-// identity on the padding): row m of tile (m / 8, J) for J <= m / 8, from the
-// FP32 bordered hyper matrix; one CTA writes them to global memory before
-// each launch of the row kernel, whose drain threads add alpha G to them.
-__global__ void ws_base_kernel(const SweepArgs a, float* base) {
-  const WsGeom G(a.K);
-  for (int m = threadIdx.x; m < G.KP; m += blockDim.x) {
-    const int I = m >> 3, p = m & 7;
-    for (int J = 0; J <= I; ++J) {
-      float x[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int n = 8 * J + i;
-        x[i] = (m < G.KA && n < G.KA) ? (n <= m ? __ldg(a.lamaug + m * G.KA + n) : 0.f)
-                                      : (n == m ? 1.f : 0.f);
-      }
-      st8(base + (I * (I + 1) / 2 + J) * kWsTileF + trow(p), x);
-    }
-  }
-}
-
-__device__ __forceinline__ void ldg8(const float* p, float (&x)[8]) {
-  const float4 u = __ldg(reinterpret_cast<const float4*>(p));
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p) + 1);
-  x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
-  x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+// Element (m, n) of the base matrix: the lower triangle of the bordered
+// [[Lambda_s, b0], [b0^T, 0]], identity on the padding past row K.
+__device__ __forceinline__ float ws_base(const SweepArgs& a, const WsGeom& G, int m, int n) {
+  return m < G.KA && n < G.KA ? (n <= m ? __ldg(a.lamaug + m * G.KA + n) : 0.f)
+                              : (n == m ? 1.f : 0.f);
 }
 
 // -------------------------------------------------------------- drain --
 // Thread m (0..127) owns tensor-memory lane m = row m of the accumulator.
+//
+// One row's drain stands between the MMA warp (which waits for the
+// accumulator) and a consumer (which waits for the slot), so it is latency
+// that counts.  The base matrix therefore sits on chip for the whole launch:
+// in tensor memory beside the accumulators, read by the same kind of load in
+// the same batch, or, with XO, in shared memory.  (Read from global memory
+// tile by tile, as it was before, each 16 columns waited for a round trip to
+// the L2: 8.5k cycles per row of K = 100, during which the consumers idled a
+// quarter of their time.  60,000 rows of 188 ratings on average, K = 100:
+// 3.06 -> 2.83 ms; K = 64, 50,000 rows of 45 and 12,000 of 188: 1.5 -> 1.3 ms
+// for both sides.)
 template <bool XO>
 __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, const WsShared& w, int C,
                          uint32_t tmem) {
   const int m = threadIdx.x - kWsGather;
-  const int wq = m >> 5;  // warp quarter: lanes 32 wq .. 32 wq + 31
+  const int wq = m >> 5, lane = m & 31;  // warp quarter: lanes 32 wq .. 32 wq + 31
   const int I = m >> 3, p = m & 7;
   const int slotf = G.slot_floats();
+  const int row_tile = I * (I + 1) / 2;
+  // columns 0 .. 32 wq + 31 cover the lower triangle of this warp's rows
+  const int ncol = 32 * wq + 32 < G.NP ? 32 * wq + 32 : G.NP;
+  const uint32_t quarter = (uint32_t)(32 * wq) << 16;
+  if (XO) {
+    if (m < G.KP) {
+      for (int J = 0; J <= I; ++J) {
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = ws_base(a, G, m, 8 * J + i);
+        st8(w.base + (row_tile + J) * kWsTileF + trow(p), x);
+      }
+    }
+  } else {
+    for (int c0 = 0; c0 < ncol; c0 += 16) {
+      float x[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) x[i] = ws_base(a, G, m, c0 + i);
+      tmem_st16(tmem + kWsBaseCol + quarter + (uint32_t)c0, x);
+    }
+    tmem_wait_st();
+  }
   int q = 0;
   uint32_t nsync = 0;  // completed phases of drain_sync
   for (;;) {
@@ -637,7 +657,8 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
         const int use = (q + i) / C;
         if (!ws_wait_warp(&w.slot_empty[c], ((uint32_t)use & 1u) ^ 1u, w.abort, w.wait_ns)) return;
         if (m == 0) reinterpret_cast<int*>(w.slots + c * slotf)[0] = -1;
-        mbar_arrive(&w.slot_full[c]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&w.slot_full[c]);
       }
       return;
     }
@@ -646,46 +667,45 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
     float* slot = w.slots + c * slotf;
     float* tiles = slot + 4;
     float* diag0 = tiles + G.ntile * kWsTileF;
-    const uint32_t lane_base = tmem + (uint32_t)b * ws_acc_stride<XO>() + ((uint32_t)(32 * wq) << 16);
+    const uint32_t lane_base = tmem + (uint32_t)b * ws_acc_stride<XO>() + quarter;
     const bool gram = r.nst > 0;
-    // columns 0 .. 32 wq + 31 cover the lower triangle of this warp's rows
-    const int ncol = 32 * wq + 32 < G.NP ? 32 * wq + 32 : G.NP;
+    // A = base + alpha G, 16 columns at a time.  Entries past the diagonal in
+    // the last tile are not read; G is zero in the padding rows and columns.
     for (int c0 = 0; c0 < ncol; c0 += 16) {
-      float v[16];
-      if (gram) {
-        tmem_ld16(lane_base + (uint32_t)c0, v);
-        if (XO) {
-          float v2[16];
-          tmem_ld16(lane_base + kWsAccCols + (uint32_t)c0, v2);
-          tmem_wait_ld();
+      float v[16], x[16];
+      tmem_ld16(lane_base + (uint32_t)c0, v);
+      if (XO) {
+        float v2[16];
+        tmem_ld16(lane_base + kWsAccCols + (uint32_t)c0, v2);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) v[i] += v2[i];
-        } else {
-          tmem_wait_ld();
+        for (int h = 0; h < 2; ++h) {
+          const int J = (c0 >> 3) + h;
+          float y[8];
+          ld8(w.base + (m < G.KP && J <= I ? (row_tile + J) * kWsTileF + trow(p) : 0), y);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[8 * h + i] = y[i];
         }
-      } else {
+        tmem_wait_ld(v);
+        tmem_wait_ld(v2);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+        for (int i = 0; i < 16; ++i) v[i] += v2[i];
+      } else {
+        tmem_ld16(tmem + kWsBaseCol + quarter + (uint32_t)c0, x);
+        tmem_wait_ld(v);
+        tmem_wait_ld(x);
+      }
+      if (gram) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = fmaf(a.alpha, v[i], x[i]);
       }
       if (m < G.KP) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int J = (c0 >> 3) + h;
           if (J <= I) {
-            float x[8];
-            float dv = 0.f;
-            const int toff = (I * (I + 1) / 2 + J) * kWsTileF + trow(p);
-            ldg8(a.wsbase + toff, x);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int n = 8 * J + i;
-              if (m < G.KA && n <= m) x[i] = fmaf(a.alpha, v[8 * h + i], x[i]);
-              if (n == m) dv = x[i];
-            }
-            float* dst = tiles + toff;
-            reinterpret_cast<float4*>(dst)[0] = make_float4(x[0], x[1], x[2], x[3]);
-            reinterpret_cast<float4*>(dst)[1] = make_float4(x[4], x[5], x[6], x[7]);
-            if (J == I && m < G.K) diag0[m] = dv;
+            float4* dst = reinterpret_cast<float4*>(tiles + (row_tile + J) * kWsTileF + trow(p));
+            dst[0] = make_float4(x[8 * h], x[8 * h + 1], x[8 * h + 2], x[8 * h + 3]);
+            dst[1] = make_float4(x[8 * h + 4], x[8 * h + 5], x[8 * h + 6], x[8 * h + 7]);
           }
         }
       }
@@ -702,26 +722,35 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
       ++nsync;
       const int n = m;
       for (int c0 = (32 * wq) & ~15; c0 < G.NP; c0 += 16) {
-        float v[16];
+        float v[16], e[16];
         tmem_ld16(lane_base + kWsAccCols + (uint32_t)c0, v);
-        tmem_wait_ld();
-        if (n < G.KA) {
+        // element (c0, n): the 16 rows are two tile rows of eight
+        float* e0 = tiles + ((c0 >> 3) * ((c0 >> 3) + 1) / 2 + (n >> 3)) * kWsTileF + (n & 7);
+        float* e1 = e0 + ((c0 >> 3) + 1) * kWsTileF;
+        // all loads before the first store (the elements are distinct)
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int j = c0 + i;
-            if (j >= n && j < G.KA) {
-              float* e = tiles + ((j >> 3) * ((j >> 3) + 1) / 2 + (n >> 3)) * kWsTileF + trow(j & 7) + (n & 7);
-              *e = fmaf(a.alpha, v[i], *e);
-              if (j == n && n < G.K) diag0[n] = *e;
-            }
-          }
+        for (int i = 0; i < 16; ++i) {
+          const int j = c0 + i;
+          e[i] = j >= n && j < G.KA ? (i < 8 ? e0 : e1)[trow(i & 7)] : 0.f;
+        }
+        tmem_wait_ld(v);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int j = c0 + i;
+          if (j >= n && j < G.KA) (i < 8 ? e0 : e1)[trow(i & 7)] = fmaf(a.alpha, v[i], e[i]);
         }
       }
     }
+    // the row's own diagonal element, after any transposed term (both are
+    // this thread's writes)
+    if (m < G.K) diag0[m] = tiles[(row_tile + I) * kWsTileF + trow(p) + p];
     if (m == 0) reinterpret_cast<int*>(slot)[0] = r.row;
     tc_fence_before();
-    mbar_arrive(&w.acc_empty[b]);
-    mbar_arrive(&w.slot_full[c]);
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(&w.acc_empty[b]);
+      mbar_arrive(&w.slot_full[c]);
+    }
     ++q;
   }
 }
@@ -937,7 +966,7 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
   extern __shared__ __align__(1024) uint8_t smem_ws[];
   const WsGeom G(a.K);
   uint8_t* base = smem_ws + ((kWsAtom - (smem_u32(smem_ws) & (kWsAtom - 1))) & (kWsAtom - 1));
-  WsShared w = ws_carve(base, G, S, C, NB);
+  WsShared w = ws_carve(base, G, S, C, NB, XO);
   w.wait_ns = a.wait_ns;
   const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
@@ -949,10 +978,10 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&w.acc_full[b], 1);
-      mbar_init(&w.acc_empty[b], kWsDrain);
+      mbar_init(&w.acc_empty[b], kWsDrain / 32);  // lane 0 of each drain warp
     }
     for (int c = 0; c < C; ++c) {
-      mbar_init(&w.slot_full[c], kWsDrain);
+      mbar_init(&w.slot_full[c], kWsDrain / 32);
       mbar_init(&w.slot_empty[c], 1);
     }
     mbar_init(w.fin, 1);
@@ -972,7 +1001,7 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
     for (int e = threadIdx.x; e <= G.g; e += blockDim.x) w.sched[32 * G.nround + e] = (uint16_t)(rr[e] - r0);
   }
   if (warp == kWsMmaWarp) {
-    tmem_alloc(w.taddr, 2 * ws_acc_stride<XO>());
+    tmem_alloc(w.taddr, kWsTmemCols);
     tmem_relinquish();
   }
   fence_proxy_async_smem();
@@ -994,7 +1023,7 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
   if (*w.abort && threadIdx.x == 0) atomicOr(status, kStatusTimeout);
   if (warp == kWsMmaWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem, 2 * ws_acc_stride<XO>());
+    tmem_dealloc(tmem, kWsTmemCols);
   }
 }
 
@@ -1031,12 +1060,13 @@ bool ws_supported(int K) {
 }
 
 // Stages (a multiple of 4, one or more ring slots per gather warp) and
-// consumer warps for latent dimension K and nb neighbours per stage.  With
+// consumer warps for latent dimension K and nb neighbours per stage (cross:
+// with the base tiles in shared memory).  With
 // `cons` > 0 that many consumers (as many as fit, if fewer) and the deepest
 // ring up to kWsMaxStages that fits;
 // otherwise 8 stages if at least 3 consumers fit beside them, else 4 stages
 // and as many consumers as fit.
-int ws_config(int K, int cons, int nb, int* S, int* C) {
+int ws_config(int K, int cons, int nb, bool cross, int* S, int* C) {
   const WsGeom G(K);
   int dev = 0, max_smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -1046,15 +1076,15 @@ int ws_config(int K, int cons, int nb, int* S, int* C) {
   }
   auto fit_cons = [&](int s) {
     int c = kWsMaxCons;
-    while (c > 0 && ws_smem_bytes(G, s, c, nb) > max_smem) --c;
+    while (c > 0 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) --c;
     return c;
   };
   int s = 8, c = 0;
   if (cons > 0) {
     c = std::min(cons, kWsMaxCons);
     s = kWsMaxStages;
-    while (s > 4 && ws_smem_bytes(G, s, c, nb) > max_smem) s -= 4;
-    while (c > 1 && ws_smem_bytes(G, s, c, nb) > max_smem) --c;  // more than fit: cut
+    while (s > 4 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) s -= 4;
+    while (c > 1 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) --c;  // more than fit: cut
   } else {
     c = fit_cons(s);
     if (c < 3) {
@@ -1062,7 +1092,7 @@ int ws_config(int K, int cons, int nb, int* S, int* C) {
       c = fit_cons(s);
     }
   }
-  if (c < 1 || ws_smem_bytes(G, s, c, nb) > max_smem) return BPMF_EINVAL;
+  if (c < 1 || ws_smem_bytes(G, s, c, nb, cross) > max_smem) return BPMF_EINVAL;
   *S = s;
   *C = c;
   return BPMF_OK;
@@ -1120,15 +1150,12 @@ int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross
   if (nb != 32 && nb != 64) return BPMF_EINVAL;
   if (cross && nb != 64) return BPMF_EINVAL;
   int S = 0, C = 0;
-  BPMF_TRY(ws_config(a.K, cons, nb, &S, &C));
+  BPMF_TRY(ws_config(a.K, cons, nb, cross, &S, &C));
   const WsGeom G(a.K);
-  const int smem = ws_smem_bytes(G, S, C, nb);
+  const int smem = ws_smem_bytes(G, S, C, nb, cross);
   auto kern = nb == 32 ? row_ws<32, false> : cross ? row_ws<64, true> : row_ws<64, false>;
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   BPMF_CUDA_CHECK(cudaMemsetAsync(counter, 0, sizeof(int), st));
-  ws_base_kernel<<<1, 128, 0, st>>>(a, a.wsbase);
-  BPMF_CUDA_CHECK(cudaGetLastError());
-  if (launches) *launches += 1;
   const int grid = (int)std::min<int64_t>(num_sms, nrows);
   CUtensorMap map_hi, map_lo;
   BPMF_TRY(encode_shadow_map(a.Vhi, a.n_other, a.KS, &map_hi));
