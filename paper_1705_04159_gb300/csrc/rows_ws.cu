@@ -16,7 +16,7 @@
 //     128-byte swizzle, into a ring of stages (64-neighbour stages copy the
 //     features past 64 by 16-byte cp.async instead); the MMA warp patches
 //     the rating in as feature K;
-//   MMA (warp 8, one thread): per 16 neighbours hi.hi + hi.lo + lo.hi into
+//   MMA (warp 8, one elected thread): per 16 neighbours hi.hi + hi.lo + lo.hi into
 //     one of two FP32 accumulators in tensor memory (G = X^T X with X the
 //     stage's neighbours x features; lo.lo, ~2^-16 relative, is dropped); on
 //     sides whose rows average 2048 ratings or more, hi.hi and hi.lo into two
@@ -516,7 +516,7 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
 // ---------------------------------------------------------------- MMA --
 // The whole MMA warp waits for each stage's copies (and with them its
 // metadata and ratings), patches the ratings into their swizzled places,
-// makes them visible to the tensor cores, and lane 0 issues the products.
+// makes them visible to the tensor cores, and one elected lane issues the products.
 // With `hold` (failure-path testing) the first row's accumulator is never
 // handed to the drain, whose bounded wait then runs out.
 template <int NB, bool XO>
@@ -524,7 +524,9 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
                                        int hold) {
   const int lane = threadIdx.x & 31;
   const uint32_t idesc = idesc_bf16_mn(128, G.NP);
-  const uint32_t base = smem_u32(w.stages);
+  // operand tile of the first stage: the leading byte offset steps between
+  // 64-feature blocks, the stride one between atoms
+  const uint64_t desc0 = smem_desc_sw128(smem_u32(w.stages), WsNb<NB>::kBlk, kWsAtom);
   uint32_t n = 0;
   int q = 0;
   for (;;) {
@@ -543,23 +545,25 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
       if (!ws_wait_warp(&w.acc_empty[b], ((uint32_t)(q >> 1) & 1u) ^ 1u, w.abort, w.wait_ns)) break;
     }
     tc_fence_after();
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t acc = tmem + (uint32_t)b * ws_acc_stride<XO>();
-      if (m.cnt > 0) {
-        const uint32_t hi = base + (uint32_t)s * WsNb<NB>::kStageBytes, lo = hi + WsNb<NB>::kOpBytes;
-        // K-steps of 16 neighbours: two atoms apart; the leading byte offset
-        // steps between 64-feature blocks, the stride one between atoms
-        for (int kk = 0; kk < (m.cnt + 15) / 16; ++kk) {
-          const uint64_t dh = smem_desc_sw128(hi + kk * 2 * kWsAtom, WsNb<NB>::kBlk, kWsAtom);
-          const uint64_t dl = smem_desc_sw128(lo + kk * 2 * kWsAtom, WsNb<NB>::kBlk, kWsAtom);
-          const uint32_t first = ((m.flags & 1) && kk == 0) ? 0u : 1u;
+      // K-steps of 16 neighbours: two atoms apart (the descriptors count in
+      // units of 16 bytes)
+      const uint64_t dh = desc0 + (uint64_t)((s * WsNb<NB>::kStageBytes) >> 4);
+      const int steps = (m.cnt + 15) >> 4;
+#pragma unroll
+      for (int kk = 0; kk < NB / 16; ++kk) {
+        if (kk < steps) {
+          const uint64_t h = dh + (uint64_t)((kk * 2 * kWsAtom) >> 4);
+          const uint64_t l = h + (uint64_t)(WsNb<NB>::kOpBytes >> 4);
+          const uint32_t more = kk == 0 ? (m.flags & 1) ^ 1u : 1u;
           if (XO) {
-            tc_mma_bf16(acc, dh, dh, idesc, first);
-            tc_mma_bf16(acc + kWsAccCols, dh, dl, idesc, first);
+            tc_mma_bf16(acc, h, h, idesc, more);
+            tc_mma_bf16(acc + kWsAccCols, h, l, idesc, more);
           } else {
-            tc_mma_bf16(acc, dh, dh, idesc, first);
-            tc_mma_bf16(acc, dh, dl, idesc, 1u);
-            tc_mma_bf16(acc, dl, dh, idesc, 1u);
+            tc_mma_bf16(acc, h, h, idesc, more);
+            tc_mma_bf16(acc, h, l, idesc, 1u);
+            tc_mma_bf16(acc, l, h, idesc, 1u);
           }
         }
       }
@@ -574,7 +578,7 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
     }
   }
   // every MMA issued has completed before the tensor memory is freed
-  if (lane == 0) {
+  if (elect_one()) {
     tc_commit(w.fin);
     uint32_t polls = 0;
     while (!mbar_try_wait_sleep(w.fin, 0, 20000u) && ++polls < kWsPolls) {

@@ -118,6 +118,19 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
+// True in one lane of a converged warp.  The compiler knows that a branch on
+// it runs a single thread, so the operands of tcgen05 instructions inside go
+// to uniform registers directly; under a branch on the lane number each
+// instruction is issued through a loop over the lanes' values instead
+// (measured, M = 128, N = 112, one thread issuing back to back: 157 cycles per
+// tcgen05.mma against 70).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+               : "=r"(p));
+  return p != 0;
+}
+
 // D[tmem] (+)= A[smem] * B[smem]^T; issued by one thread.
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                             uint32_t idesc, uint32_t accumulate) {
