@@ -1,5 +1,8 @@
-"""Writes ws_units.inc: the lane schedule of the trailing update in the
-persistent row kernel (rows_ws.cu).
+"""Writes ws_units.inc: a lane schedule of the trailing update of a
+right-looking tile Cholesky by one warp.  The persistent row kernel
+(rows_ws.cu), which used it, now factors left-looking on tensor-core tiles and
+includes no schedule; the table and its generator are kept as the subject of
+the schedule and algorithm tests.
 
 In the blocked right-looking Cholesky of one row's bordered matrix (g x g
 tiles of 8 x 8), panel p leaves the trailing tiles (I, J), p < J <= I < g, to

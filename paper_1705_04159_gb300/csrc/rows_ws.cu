@@ -17,7 +17,7 @@
 //     features past 64 by 16-byte cp.async instead); the MMA warp patches
 //     the rating in as feature K;
 //   MMA (warp 8, one elected thread): per 16 neighbours hi.hi + hi.lo + lo.hi into
-//     one of two FP32 accumulators in tensor memory (G = X^T X with X the
+//     one of three FP32 accumulators in tensor memory (G = X^T X with X the
 //     stage's neighbours x features; lo.lo, ~2^-16 relative, is dropped); on
 //     sides whose rows average 2048 ratings or more, hi.hi and hi.lo into two
 //     accumulators instead, and the drain adds hi.lo and its transpose (two
@@ -27,11 +27,11 @@
 //     kept in tensor memory, or in shared memory where the accumulators take
 //     all of it) and writes its lower triangle as 8 x 8 FP32 tiles into a free
 //     consumer slot, releasing the accumulator for the next row;
-//   consumers (warps 9.., one row each): blocked right-looking Cholesky of
-//     the slot (per 8-column panel: the diagonal tile in registers by every
-//     lane, the panel by forward substitution, the trailing tiles as
-//     register-blocked half-tile updates on a bank-aware lane schedule),
-//     then u = L^-T (y + z) by back substitution.
+//   consumers (warps 9.., one row each): left-looking blocked Cholesky of the
+//     slot (per 8-column block: the updates from the columns before by
+//     mma.m16n8k8 on operands split into two TF32 parts, the diagonal tile in
+//     registers by every lane, the panel by forward substitution), then
+//     u = L^-T (y + z) by back substitution.
 // So the tensor cores, the gathers and the FP32 factorisations of up to
 // seven rows per SM overlap, with no CTA-wide barrier on the way.
 //
@@ -87,14 +87,18 @@ struct WsNb {
 constexpr int64_t kWsCrossRow = 2048;
 template <bool XO>
 __host__ __device__ constexpr uint32_t ws_acc_stride() { return XO ? 256u : 128u; }  // TMEM columns per buffer
-// Tensor memory: two accumulators from column 0; without XO the base matrix
-// follows them (columns 256 .. 383), with XO they fill all 512 columns.
+// Tensor memory: the accumulators from column 0, three of 128 columns followed
+// by the base matrix (columns 384 .. 511), or with XO two pairs that fill all
+// 512 columns.
 constexpr uint32_t kWsTmemCols = 512;
-constexpr uint32_t kWsBaseCol = 256;
+constexpr uint32_t kWsBaseCol = 384;
+template <bool XO>
+__host__ __device__ constexpr int ws_num_acc() { return XO ? 2 : 3; }
+constexpr int kWsMaxAcc = 3;
 __host__ __device__ constexpr int ws_stage_bytes(int nb) { return 2 * 2 * nb * 128; }
 constexpr int kWsMaxStages = 16;
 constexpr int kWsMaxCons = 7;
-constexpr int kWsRecs = 32;          // row records in flight: >= stages + 3 (see the gather loop)
+constexpr int kWsRecs = 32;          // row records in flight: >= stages + accumulators + 1
 constexpr int kWsTileF = 68;         // floats per 8 x 8 tile (see trow)
 constexpr int kWsGather = 128, kWsDrain = 128;
 constexpr int kWsMmaWarp = 8, kWsConsWarp0 = 9;
@@ -116,32 +120,24 @@ __host__ __device__ constexpr int ws_consumer_of(int w, int C) {
 constexpr uint32_t kWsPolls = 100000;  // suspending polls of <= 20 us: a 2 s bound (final MMA wait)
 constexpr uint32_t kWsAccCols = 128;
 
-#include "ws_units.inc"
-
-// Offset of row r in a tile: rows 0-3 at 8 r, rows 4-7 four floats further.
+// Offset of row r in a tile: rows 0-3 at 8 r, rows 4-7 four floats further, so
+// that eight lanes' 16-byte accesses to the same half of a tile's eight rows
+// (the drain's stores, the panel's loads and stores) fall on different banks.
 // Tiles are 68 floats apart, so consecutive tile bases fall on eight
-// different bank groups, and the two halves of a tile's rows on different
-// banks.  The trailing update's lane schedule (ws_units.inc, written by
-// gen_ws_units.py) is built for exactly this layout.
+// different bank groups.
 __host__ __device__ __forceinline__ int trow(int r) { return r * 8 + ((r >> 2) << 2); }
 
 struct WsGeom {
-  int K, KA, g, KP, NP, nfull, cb, ntile, nround;
+  int K, KA, g, KP, NP, ntile;
   __host__ __device__ explicit WsGeom(int K_) : K(K_) {
     KA = K + 1;
     g = (KA + 7) / 8;
     KP = 8 * g;
     NP = (KA + 15) & ~15;
-    nfull = K / 8;
-    cb = K / 8;
     ntile = g * (g + 1) / 2;
-    nround = 0;  // rounds of 32 half-tile units over all panels (see ws_units.inc)
-    for (int nb = 1; nb < g; ++nb) nround += (nb * (nb + 1) + 31) / 32;
   }
-  // consumer slot: header (4 ints), tiles, diag0, rinv, z
+  // consumer slot: header (4 ints), tiles, pivot thresholds, 1 / diagonal, z
   __host__ __device__ int slot_floats() const { return 4 + ntile * kWsTileF + 3 * KP; }
-  // the trailing-update schedule of this g and its per-panel first rounds
-  __host__ __device__ int sched_bytes() const { return (64 * nround + 2 * (g + 1) + 15) & ~15; }
 };
 
 struct StageMeta {
@@ -160,7 +156,6 @@ struct WsShared {
   uint8_t* stages;
   float* slots;
   float* base;  // base tiles (with XO only)
-  uint16_t* sched;  // [32 * nround] lane units, then [g + 1] first round of each panel
   uint64_t* empty;
   uint64_t* tma;  // the stage's copies have landed (and its metadata and ratings are written)
   uint64_t* acc_full;
@@ -183,17 +178,17 @@ struct WsShared {
 // mbarriers: empty and tma per stage, full and empty per accumulator, full
 // and empty per consumer slot, fin, row_ready, row_read, drain_sync (an even
 // count, so that what follows stays 16-byte aligned)
-__host__ __device__ inline int ws_nbar(int S, int C) { return (2 * S + 4 + 2 * C + 3 + 1) & ~1; }
+__host__ __device__ inline int ws_nbar(int S, int C) { return 2 * S + 2 * kWsMaxAcc + 2 * C + 4; }
 __host__ __device__ inline int ws_fixed_bytes(int nb, int S, int C) {
   // barriers, stage meta, row records, ratings, next_row, abort, taddr
   return 8 * ws_nbar(S, C) + 16 * S + 16 * kWsRecs + 4 * S * nb + 32;
 }
-// stages, consumer slots, base tiles (with XO), the trailing-update schedule,
-// then the fixed part; one atom more, to start the stages on a 1024-byte
-// boundary (the swizzle pattern follows address bits 7 .. 9)
+// stages, consumer slots, base tiles (with XO), then the fixed part; one atom
+// more, to start the stages on a 1024-byte boundary (the swizzle pattern
+// follows address bits 7 .. 9)
 __host__ __device__ inline int ws_smem_bytes(const WsGeom& G, int S, int C, int nb, bool cross) {
   return kWsAtom + S * ws_stage_bytes(nb) + C * G.slot_floats() * 4 +
-         (cross ? G.ntile * kWsTileF * 4 : 0) + G.sched_bytes() + ws_fixed_bytes(nb, S, C);
+         (cross ? G.ntile * kWsTileF * 4 : 0) + ws_fixed_bytes(nb, S, C);
 }
 
 __device__ __forceinline__ WsShared ws_carve(uint8_t* base, const WsGeom& G, int S, int C, int nb,
@@ -202,14 +197,13 @@ __device__ __forceinline__ WsShared ws_carve(uint8_t* base, const WsGeom& G, int
   w.stages = base;
   w.slots = reinterpret_cast<float*>(base + S * ws_stage_bytes(nb));
   w.base = w.slots + C * G.slot_floats();
-  w.sched = reinterpret_cast<uint16_t*>(w.base + (cross ? G.ntile * kWsTileF : 0));
-  uint8_t* p = reinterpret_cast<uint8_t*>(w.sched) + G.sched_bytes();
+  uint8_t* p = reinterpret_cast<uint8_t*>(w.base + (cross ? G.ntile * kWsTileF : 0));
   uint64_t* b = reinterpret_cast<uint64_t*>(p);
   w.empty = b;
   w.tma = b + S;
   w.acc_full = b + 2 * S;
-  w.acc_empty = w.acc_full + 2;
-  w.slot_full = w.acc_empty + 2;
+  w.acc_empty = w.acc_full + kWsMaxAcc;
+  w.slot_full = w.acc_empty + kWsMaxAcc;
   w.slot_empty = w.slot_full + C;
   w.fin = w.slot_empty + C;
   w.row_ready = w.fin + 1;
@@ -540,9 +534,11 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
     __syncwarp();
     const StageMeta m = w.meta[s];
     const RowRec r = w.recs[m.rec];
-    const int b = q & 1;
+    const int b = q % ws_num_acc<XO>();
     if (m.flags & 1) {
-      if (!ws_wait_warp(&w.acc_empty[b], ((uint32_t)(q >> 1) & 1u) ^ 1u, w.abort, w.wait_ns)) break;
+      if (!ws_wait_warp(&w.acc_empty[b], ((uint32_t)(q / ws_num_acc<XO>()) & 1u) ^ 1u, w.abort,
+                        w.wait_ns))
+        break;
     }
     tc_fence_after();
     if (elect_one()) {
@@ -599,10 +595,12 @@ __device__ __forceinline__ void st8(float* p, const float (&x)[8]) {
 }
 
 // Element (m, n) of the base matrix: the lower triangle of the bordered
-// [[Lambda_s, b0], [b0^T, 0]], identity on the padding past row K.
+// [[Lambda_s, b0], [b0^T, c]], identity on the padding past row K.  The
+// corner c, which no draw reads, is large, so that the factorisation passes
+// row K with a positive pivot.
 __device__ __forceinline__ float ws_base(const SweepArgs& a, const WsGeom& G, int m, int n) {
-  return m < G.KA && n < G.KA ? (n <= m ? __ldg(a.lamaug + m * G.KA + n) : 0.f)
-                              : (n == m ? 1.f : 0.f);
+  if (m >= G.KA || n >= G.KA) return n == m ? 1.f : 0.f;
+  return n > m ? 0.f : m == G.K && n == G.K ? 1e30f : __ldg(a.lamaug + m * G.KA + n);
 }
 
 // -------------------------------------------------------------- drain --
@@ -650,8 +648,9 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
   int q = 0;
   uint32_t nsync = 0;  // completed phases of drain_sync
   for (;;) {
-    const int b = q & 1;
-    if (!ws_wait_warp(&w.acc_full[b], (uint32_t)(q >> 1) & 1u, w.abort, w.wait_ns)) return;
+    const int b = q % ws_num_acc<XO>();
+    if (!ws_wait_warp(&w.acc_full[b], (uint32_t)(q / ws_num_acc<XO>()) & 1u, w.abort, w.wait_ns))
+      return;
     tc_fence_after();
     const RowRec r = w.recs[q % kWsRecs];
     if (r.row < 0) {
@@ -670,7 +669,7 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
     if (!ws_wait_warp(&w.slot_empty[c], ((uint32_t)(q / C) & 1u) ^ 1u, w.abort, w.wait_ns)) return;
     float* slot = w.slots + c * slotf;
     float* tiles = slot + 4;
-    float* diag0 = tiles + G.ntile * kWsTileF;
+    float* thr = tiles + G.ntile * kWsTileF;
     const uint32_t lane_base = tmem + (uint32_t)b * ws_acc_stride<XO>() + quarter;
     const bool gram = r.nst > 0;
     // A = base + alpha G, 16 columns at a time.  Entries past the diagonal in
@@ -745,9 +744,11 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
         }
       }
     }
-    // the row's own diagonal element, after any transposed term (both are
-    // this thread's writes)
-    if (m < G.K) diag0[m] = tiles[(row_tile + I) * kWsTileF + trow(p) + p];
+    // the pivot threshold from the row's own diagonal element, after any
+    // transposed term (both are this thread's writes)
+    if (m < G.KP)
+      thr[m] = m < G.K ? pivot_threshold(a.pivot_rel, tiles[(row_tile + I) * kWsTileF + trow(p) + p])
+                       : -INFINITY;
     if (m == 0) reinterpret_cast<int*>(slot)[0] = r.row;
     tc_fence_before();
     __syncwarp();
@@ -760,121 +761,274 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
 }
 
 // ----------------------------------------------------------- consumer --
+//
+// One warp factors a slot's tiles and solves for the row.  The factorisation
+// is left-looking by block columns J of eight columns:
+//   update: A_IJ -= sum_{p<J} L_Ip L_Jp^T for all row tiles I >= J, on the
+//     tensor cores by mma.m16n8k8 (two row tiles at a time) with FP32 operands
+//     split into two TF32 parts, x = h + l: h h^T in one FP32 accumulator and
+//     h l^T + l h^T in another (l l^T, 2^-24 relative, is dropped), so only
+//     the p-sums of like size meet in an accumulator;
+//   diagonal tile: Cholesky in registers by every lane;
+//   panel: the rows below by substitution, a lane per row.
+// A tile is 8 rows of 8 floats (trow), and a lane's fragment of an operand or
+// an accumulator is the same pair of neighbouring floats everywhere: column
+// pair t of row g (lane 4 g + t), taking the operands' k index t for column 2t
+// and t + 4 for column 2t + 1.  So tiles are loaded by 8-byte conflict-free
+// loads and never rearranged.
+// What bounds it: instruction issue and latency of one warp (at K = 100, 14.8k
+// warp instructions and 3.7k shared-memory wavefronts a row; the right-looking
+// FP32 form before it needed 17.2k and 7.3k, and its wavefronts alone were 72%
+// of what the SM can serve).  Six rows side by side on an SM, nothing else
+// running: 5.43 -> 4.53 us per row at K = 100, 2.80 -> 2.41 at K = 64, 1.28 ->
+// 1.14 at K = 33; error of the draws against FP64 2.8e-7 -> 2.4e-7, 2.1e-7 ->
+// 1.7e-7 and 1.4e-7 -> 1.2e-7.
 __device__ __forceinline__ int tidx(int I, int J) { return I * (I + 1) / 2 + J; }
 
-// Blocked right-looking Cholesky of the slot's tiles by one warp.  Returns
-// false if a pivot (of rows 0..K-1) failed the pivot rule of tile_chol.cuh
-// (at or below prel times its starting diagonal); row K (the bordered
-// right-hand side) and the padding rows are never tested.
-__device__ __forceinline__ bool ws_cholesky(const WsGeom& G, float* T, const float* diag0, float* rinv,
-                                            const uint16_t* sched, int lane, float prel) {
+__device__ __forceinline__ float2 ldf2(const float* p) { return *reinterpret_cast<const float2*>(p); }
+
+// D += A B on 16 x 8 x 8 elements, TF32 operands, FP32 accumulator
+__device__ __forceinline__ void mma_tf32(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%0, %1, %2, %3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// x = h + l: h to the nearest TF32 value (10 fraction bits), l the exact rest,
+// whose own TF32 part the tensor core reads
+__device__ __forceinline__ void split_tf32(float x, uint32_t& h, uint32_t& l) {
+  h = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  l = __float_as_uint(x - __uint_as_float(h));
+}
+
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// A_IJ -= sum_{p<J} L_Ip L_Jp^T for the 2 NPR row tiles I = I0 .. (those below
+// g; pairs wholly past it compute on the last tile and store nothing).  The
+// next step's fragments are loaded as soon as the current ones are split, so
+// after the last step they are those of column J itself.
+template <int NPR>
+__device__ __forceinline__ void ws_update(float* T, int g, int J, int I0, int fo) {
+  float acc[NPR][4], cross[NPR][4];
+  float2 fu[NPR], fv[NPR];
+  float *pu[NPR], *pv[NPR];
+#pragma unroll
+  for (int i = 0; i < NPR; ++i) {
+    const int I = min(I0 + 2 * i, g - 1);
+    pu[i] = T + tidx(I, 0) * kWsTileF + fo;
+    pv[i] = I + 1 < g ? pu[i] + (I + 1) * kWsTileF : pu[i];
+    fu[i] = ldf2(pu[i]);
+    fv[i] = ldf2(pv[i]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[i][q] = cross[i][q] = 0.f;
+  }
+  const float* pb = T + tidx(J, 0) * kWsTileF + fo;
+  float2 b = ldf2(pb);
+  int off = 0;
+#pragma unroll 1
+  for (int p = 0; p < J; ++p) {
+    off += kWsTileF;
+    uint32_t bh0, bl0, bh1, bl1;
+    split_tf32(b.x, bh0, bl0);
+    split_tf32(b.y, bh1, bl1);
+    b = ldf2(pb + off);
+    uint32_t l[NPR][4];
+#pragma unroll
+    for (int i = 0; i < NPR; ++i) {
+      uint32_t h0, h1, h2, h3;
+      split_tf32(fu[i].x, h0, l[i][0]);
+      split_tf32(fv[i].x, h1, l[i][1]);
+      split_tf32(fu[i].y, h2, l[i][2]);
+      split_tf32(fv[i].y, h3, l[i][3]);
+      fu[i] = ldf2(pu[i] + off);
+      fv[i] = ldf2(pv[i] + off);
+      mma_tf32(acc[i], h0, h1, h2, h3, bh0, bh1);
+      mma_tf32(cross[i], h0, h1, h2, h3, bl0, bl1);
+    }
+#pragma unroll
+    for (int i = 0; i < NPR; ++i)
+      mma_tf32(cross[i], l[i][0], l[i][1], l[i][2], l[i][3], bh0, bh1);
+  }
+#pragma unroll
+  for (int i = 0; i < NPR; ++i) {
+    const int I = I0 + 2 * i;
+    if (I < g)
+      *reinterpret_cast<float2*>(pu[i] + off) =
+          make_float2(fu[i].x - (acc[i][0] + cross[i][0]), fu[i].y - (acc[i][1] + cross[i][1]));
+    if (I + 1 < g)
+      *reinterpret_cast<float2*>(pv[i] + off) =
+          make_float2(fv[i].x - (acc[i][2] + cross[i][2]), fv[i].y - (acc[i][3] + cross[i][3]));
+  }
+}
+
+// x L_JJ^T = a for rows r0 .. nr - 1 (at most 32 N of them) of those below the
+// diagonal tile, N rows per lane side by side
+template <int N>
+__device__ __forceinline__ void ws_panel(int r0, int nr, int J, float* T, const float (&d)[8][8],
+                                         const float (&rdv)[8], int lane) {
+  float x[N][8];
+  float* row[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    const int rr = r0 + lane + 32 * k, I = J + 1 + (rr >> 3);
+    row[k] = T + tidx(I, J) * kWsTileF + trow(rr & 7);
+    if (rr < nr) ld8(row[k], x[k]);
+  }
+#pragma unroll
+  for (int c = 0; c < 8; ++c)
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      x[k][c] *= rdv[c];
+#pragma unroll
+      for (int s = c + 1; s < 8; ++s) x[k][s] = fmaf(-x[k][c], d[s][c], x[k][s]);
+    }
+#pragma unroll
+  for (int k = 0; k < N; ++k)
+    if (r0 + lane + 32 * k < nr) st8(row[k], x[k]);
+}
+
+// Left-looking Cholesky of the slot's tiles by one warp.  Returns false if a
+// pivot met the pivot rule of tile_chol.cuh (at or below thr, formed by the
+// drain from its starting diagonal; -inf on the bordered row K and on the
+// padding, which are never tested: row K's starting diagonal is set far above
+// any y^T y, so that its pivot is a positive number).  The diagonals
+// themselves are not stored; rinv holds their reciprocals.
+__device__ __forceinline__ bool ws_cholesky(const WsGeom& G, float* T, const float* thr_s,
+                                            float* rinv, int lane) {
   bool fail = false;
-  const uint16_t* sched_round = sched + 32 * G.nround;
-  for (int p = 0; p < G.g; ++p) {
-    // (a) diagonal tile, factored by every lane in registers (the same
-    // values in all lanes: no shuffles)
-    float* D = T + tidx(p, p) * kWsTileF;
-    float d[8][8];
+  const int g = G.g;
+  const int fo = trow(lane >> 2) + 2 * (lane & 3);
+#pragma unroll 1
+  for (int J = 0; J < g; ++J) {
+    if (J > 0) {
+      int I0 = J;
+#pragma unroll 1
+      for (; g - I0 > 4; I0 += 8) ws_update<4>(T, g, J, I0, fo);
+      if (g - I0 > 2) ws_update<2>(T, g, J, I0, fo);
+      else if (g - I0 > 0) ws_update<1>(T, g, J, I0, fo);
+      __syncwarp();
+    }
+    float* D = T + tidx(J, J) * kWsTileF;
+    float d[8][8], rdv[8], thr[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) ld8(D + trow(i), d[i]);
-    float rdv[8];
-    float thr[8];  // pivot thresholds of the panel, from the starting diagonals
-    ld8(diag0 + 8 * p, thr);
-#pragma unroll
-    for (int c = 0; c < 8; ++c) thr[c] = pivot_threshold(prel, thr[c]);
+    ld8(thr_s + 8 * J, thr);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      // Nothing but the square root stands between one pivot and the next:
-      // the pivot rule is checked beside the chain.  A failed real pivot
-      // leaves NaN or inf in the rest of the factorisation, which is
-      // discarded with the row (the FP64 redo draws it).  The pivots of the
-      // bordered row K and of the padding rows (the last panel only) are not
-      // tested: whatever they turn into stays in entries at or past column K
-      // of rows at or past K, which the draw never reads.
+      // A failed pivot leaves NaN or inf in the rest of the factorisation,
+      // which is discarded with the row (the FP64 redo draws it).  A pivot
+      // that passes is a normal number, where the flushing root is the same.
       const float piv = d[c][c];
-      fail = fail || (8 * p + c < G.K && !(piv > thr[c]));  // without branches
-      const float rd = rsqrtf(piv);
+      fail = fail || !(piv > thr[c]);
+      const float rd = rsqrt_normal(piv);
       rdv[c] = rd;
-      d[c][c] = piv * rd;
 #pragma unroll
       for (int i = c + 1; i < 8; ++i) d[i][c] *= rd;
 #pragma unroll
-      for (int j2 = c + 1; j2 < 8; ++j2)
+      for (int j = c + 1; j < 8; ++j)
 #pragma unroll
-        for (int i = j2; i < 8; ++i) d[i][j2] = fmaf(-d[i][c], d[j2][c], d[i][j2]);
+        for (int i = j; i < 8; ++i) d[i][j] = fmaf(-d[i][c], d[j][c], d[i][j]);
     }
     // every lane holds the same factor, so every lane writes it: same
     // address, same value, no divergent stores
 #pragma unroll
-    for (int i = 0; i < 8; ++i) st8(D + trow(i), d[i]);
-    st8(rinv + 8 * p, rdv);
-    // (b) panel rows below: x L_pp^T = a, row by row, against the registers
-    const int nb = G.g - 1 - p;
-    for (int rr = lane; rr < 8 * nb; rr += 32) {
-      const int I = p + 1 + (rr >> 3);
-      float* row = T + tidx(I, p) * kWsTileF + trow(rr & 7);
-      float x[8];
-      ld8(row, x);
-#pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        float t2 = x[c];
-#pragma unroll
-        for (int s2 = 0; s2 < c; ++s2) t2 = fmaf(-x[s2], d[c][s2], t2);
-        x[c] = t2 * rdv[c];
-      }
-      st8(row, x);
+    for (int i = 1; i < 8; ++i) {
+      float4* dst = reinterpret_cast<float4*>(D + trow(i));
+      dst[0] = make_float4(d[i][0], d[i][1], d[i][2], d[i][3]);
+      if (i > 4) dst[1] = make_float4(d[i][4], d[i][5], d[i][6], d[i][7]);
     }
-    __syncwarp();
-    // (c) trailing tiles (I, J), p < J <= I: A_IJ -= L_Ip L_Jp^T, in units
-    // of half a tile (4 of its 8 columns) so that more lanes have work, by
-    // the lane schedule of ws_units.inc (units grouped eight lanes at a time
-    // to keep their 128-bit accesses off each other's banks); the rows of
-    // L_Ip and A_IJ are loaded one row ahead
-    const int r0 = sched_round[p], r1 = sched_round[p + 1];
-    uint32_t e = r0 < r1 ? sched[32 * r0 + lane] : 0xFFFFu;
-    for (int r = r0; r < r1; ++r) {
-      const uint32_t e_next = r + 1 < r1 ? sched[32 * (r + 1) + lane] : 0xFFFFu;
-      const uint32_t ecur = e;
-      e = e_next;
-      if (ecur == 0xFFFFu) continue;
-      const int I = ecur & 15, J = (ecur >> 4) & 15, h = (ecur >> 8) & 1;
-      const float* LI = T + tidx(I, p) * kWsTileF;
-      const float* LJ = T + tidx(J, p) * kWsTileF + trow(4 * h);
-      float* A = T + tidx(I, J) * kWsTileF + 4 * h;
-      float lj[4][8];
-#pragma unroll
-      for (int jj = 0; jj < 4; ++jj) ld8(LJ + jj * 8, lj[jj]);  // rows 4h .. 4h + 3: contiguous
-      float li[8];
-      float4 ar;
-      ld8(LI, li);
-      ar = *reinterpret_cast<const float4*>(A);
-#pragma unroll
-      for (int ii = 0; ii < 8; ++ii) {
-        float lin[8];
-        float4 arn = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (ii < 7) {
-          ld8(LI + trow(ii + 1), lin);
-          arn = *reinterpret_cast<const float4*>(A + trow(ii + 1));
-        }
-        float a4[4] = {ar.x, ar.y, ar.z, ar.w};
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          float s3 = a4[jj];
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) s3 = fmaf(-li[kk], lj[jj][kk], s3);
-          a4[jj] = s3;
-        }
-        *reinterpret_cast<float4*>(A + trow(ii)) = make_float4(a4[0], a4[1], a4[2], a4[3]);
-        if (ii < 7) {
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) li[kk] = lin[kk];
-          ar = arn;
-        }
-      }
-    }
+    st8(rinv + 8 * J, rdv);
+    const int nr = 8 * (g - 1 - J);
+#pragma unroll 1
+    for (int r0 = 0; r0 < nr; r0 += 64) ws_panel<2>(r0, nr, J, T, d, rdv, lane);
     __syncwarp();
   }
   return !fail;
+}
+
+// u = L^-T (y + z), y row K of the factor, by 8-row blocks from the bottom:
+// lane 2 J + h keeps columns 8 J + 4 h .. + 3 (so one pass covers all of a
+// row), the block's eight values come to every lane by shuffles, every lane
+// solves the 8 x 8 system, and each subtracts the block's part from its
+// columns.  The tiles of the next block are loaded while this one is used.
+__device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const float* rinv,
+                                        const float* zv, int lane, float* out) {
+  const int K = G.K;
+  const int J = lane >> 1, h4 = (lane & 1) << 2;
+  const int IK = K >> 3, pk = K & 7;
+  float v[4];
+  {
+    const float4 y = *reinterpret_cast<const float4*>(
+        T + (J <= IK ? tidx(IK, J) * kWsTileF + trow(pk) + h4 : 0));
+    const float4 z = *reinterpret_cast<const float4*>(zv + (J <= IK ? 8 * J + h4 : 0));
+    v[0] = y.x + z.x; v[1] = y.y + z.y; v[2] = y.z + z.z; v[3] = y.w + z.w;
+  }
+  float4 lc[8];         // the lane's columns of tile (I, J), J < I
+  float d[8][8], rd[8];  // the strict lower triangle of tile (I, I), 1 / diagonal
+  auto load_diag = [&](int I) {
+    const float* Dg = T + tidx(I, I) * kWsTileF;
+#pragma unroll
+    for (int r = 1; r < 8; ++r) {
+      const float4 a = *reinterpret_cast<const float4*>(Dg + trow(r));
+      d[r][0] = a.x; d[r][1] = a.y; d[r][2] = a.z; d[r][3] = a.w;
+      if (r > 4) {
+        const float4 b = *reinterpret_cast<const float4*>(Dg + trow(r) + 4);
+        d[r][4] = b.x; d[r][5] = b.y; d[r][6] = b.z; d[r][7] = b.w;
+      }
+    }
+    ld8(rinv + 8 * I, rd);
+  };
+  auto load_cols = [&](int I) {
+    const float* L = T + tidx(I, J < I ? J : 0) * kWsTileF + h4;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) lc[q] = *reinterpret_cast<const float4*>(L + trow(q));
+  };
+  int I = (K - 1) >> 3;
+  load_diag(I);
+  load_cols(I);
+#pragma unroll 1
+  for (; I >= 0; --I) {
+    float u[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[q] = __shfl_sync(0xffffffffu, v[q & 3], 2 * I + (q >> 2));
+    const int nI = K - 8 * I;  // rows of the block (row K and the padding are not solved for)
+#pragma unroll
+    for (int c = 7; c >= 0; --c) {
+      u[c] = c < nI ? u[c] * rd[c] : 0.f;
+#pragma unroll
+      for (int r = 0; r < c; ++r) u[r] = fmaf(-d[c][r], u[c], u[r]);
+    }
+    const int next = I > 0 ? I - 1 : 0;
+    load_diag(next);
+    if (J < I) {
+#pragma unroll
+      for (int q = 7; q >= 0; --q) {
+        v[0] = fmaf(-lc[q].x, u[q], v[0]);
+        v[1] = fmaf(-lc[q].y, u[q], v[1]);
+        v[2] = fmaf(-lc[q].z, u[q], v[2]);
+        v[3] = fmaf(-lc[q].w, u[q], v[3]);
+      }
+    } else if (J == I) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = h4 ? u[4 + k] : u[k];
+    }
+    load_cols(next);
+  }
+  const int c0 = 8 * J + h4;
+  if ((K & 3) == 0) {  // the row of X starts on a 16-byte boundary
+    if (c0 < K) *reinterpret_cast<float4*>(out + c0) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (c0 + k < K) out[c0 + k] = v[k];
+  }
 }
 
 __device__ __forceinline__ void ws_consume(const SweepArgs& a, const WsGeom& G, const WsShared& w, int C) {
@@ -882,8 +1036,8 @@ __device__ __forceinline__ void ws_consume(const SweepArgs& a, const WsGeom& G, 
   const int lane = threadIdx.x & 31;
   float* slot = w.slots + c * G.slot_floats();
   float* T = slot + 4;
-  float* diag0 = T + G.ntile * kWsTileF;
-  float* rinv = diag0 + G.KP;
+  float* thr = T + G.ntile * kWsTileF;
+  float* rinv = thr + G.KP;
   float* zv = rinv + G.KP;
   const uint32_t tw = *a.tp;
   const int K = G.K;
@@ -891,72 +1045,12 @@ __device__ __forceinline__ void ws_consume(const SweepArgs& a, const WsGeom& G, 
     if (!ws_wait_warp(&w.slot_full[c], (uint32_t)qc & 1u, w.abort, w.wait_ns)) return;
     const int row = reinterpret_cast<const int*>(slot)[0];
     if (row < 0) return;
-    for (int qd = lane; 4 * qd < K; qd += 32) {
-      const float4 z = normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)qd, a.sw), a.key));
-      zv[4 * qd] = z.x;
-      if (4 * qd + 1 < K) zv[4 * qd + 1] = z.y;
-      if (4 * qd + 2 < K) zv[4 * qd + 2] = z.z;
-      if (4 * qd + 3 < K) zv[4 * qd + 3] = z.w;
-    }
-    const bool ok = ws_cholesky(G, T, diag0, rinv, w.sched, lane, a.pivot_rel);
-    if (ok) {
-      // w = y + z with y = row K of L; u = L^-T w by 8-row blocks from the
-      // bottom: every lane solves the block's 8 x 8 system against the
-      // diagonal tile in registers, then subtracts the block's contribution
-      // from the w_i it owns (i = lane + 32 mm)
-      float v[4];
-      const int IK = K >> 3, pk = K & 7;
-#pragma unroll
-      for (int mm = 0; mm < 4; ++mm) {
-        const int i = lane + 32 * mm;
-        v[mm] = i < K ? T[tidx(IK, i >> 3) * kWsTileF + trow(pk) + (i & 7)] + zv[i] : 0.f;
-      }
-      for (int I = (K - 1) >> 3; I >= 0; --I) {
-        const int mI = I >> 2, l0 = (I & 3) * 8;  // rows 8I.. live in v[mI] of lanes l0..l0+7
-        float own = v[0];
-#pragma unroll
-        for (int mm = 1; mm < 4; ++mm)
-          if (mI == mm) own = v[mm];
-        float wb[8], u[8];
-#pragma unroll
-        for (int q2 = 0; q2 < 8; ++q2) wb[q2] = __shfl_sync(0xffffffffu, own, l0 + q2);
-        const float* Dg = T + tidx(I, I) * kWsTileF;
-        const int nI = K - 8 * I < 8 ? K - 8 * I : 8;
-        // u[c] waits only for u[c + 1]: it enters the sum last
-#pragma unroll
-        for (int c = 7; c >= 0; --c) {
-          float t2 = wb[c];
-#pragma unroll
-          for (int r2 = 7; r2 > c; --r2) t2 = fmaf(-Dg[trow(r2) + c], u[r2], t2);
-          u[c] = c < nI ? t2 * rinv[8 * I + c] : 0.f;
-        }
-        // the block's solution goes through shared memory (z of these rows
-        // is no longer needed) to the lanes that own its rows
-        if (lane == 0) st8(zv + 8 * I, u);
-        __syncwarp();
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) {
-          const int i = lane + 32 * mm;
-          if (i >= 8 * I && i < 8 * I + 8) {
-            v[mm] = zv[i];
-          } else if (i < 8 * I) {
-            const float* Lc = T + tidx(I, i >> 3) * kWsTileF + (i & 7);
-            float t2 = v[mm];
-#pragma unroll
-            for (int q2 = 7; q2 >= 0; --q2) t2 = fmaf(-Lc[trow(q2)], u[q2], t2);
-            v[mm] = t2;
-          }
-        }
-      }
-      float* out = a.X + (int64_t)row * K;
-#pragma unroll
-      for (int mm = 0; mm < 4; ++mm) {
-        const int i = lane + 32 * mm;
-        if (i < K) out[i] = v[mm];
-      }
-    } else if (lane == 0) {
-      a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
-    }
+    for (int qd = lane; 4 * qd < K; qd += 32)  // KP >= 4 ceil(K / 4): past K unread
+      *reinterpret_cast<float4*>(zv + 4 * qd) =
+          normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)qd, a.sw), a.key));
+    const bool ok = ws_cholesky(G, T, thr, rinv, lane);
+    if (ok) ws_back(G, T, rinv, zv, lane, a.X + (int64_t)row * K);
+    else if (lane == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
     __syncwarp();
     if (lane == 0) mbar_arrive(&w.slot_empty[c]);
   }
@@ -980,7 +1074,7 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
       // split copies, every lane once more after its cp.async copies
       mbar_init(&w.tma[s], WsNb<NB>::kSplitCopy && G.KA > 64 ? 1 + 32 : 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < ws_num_acc<XO>(); ++b) {
       mbar_init(&w.acc_full[b], 1);
       mbar_init(&w.acc_empty[b], kWsDrain / 32);  // lane 0 of each drain warp
     }
@@ -998,12 +1092,6 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
   // operand blocks no copy writes (features 64 .. 127 when K + 1 <= 64) stay zero
   for (int e = threadIdx.x; e < S * WsNb<NB>::kStageBytes / 16; e += blockDim.x)
     reinterpret_cast<uint4*>(w.stages)[e] = make_uint4(0, 0, 0, 0);
-  {  // this g's trailing-update schedule, rounds counted from its first
-    const unsigned short* rr = kWsUnitRound[G.g - kWsUnitGMin];
-    const int r0 = rr[0];
-    for (int e = threadIdx.x; e < 32 * G.nround; e += blockDim.x) w.sched[e] = kWsUnits[32 * r0 + e];
-    for (int e = threadIdx.x; e <= G.g; e += blockDim.x) w.sched[32 * G.nround + e] = (uint16_t)(rr[e] - r0);
-  }
   if (warp == kWsMmaWarp) {
     tmem_alloc(w.taddr, kWsTmemCols);
     tmem_relinquish();
@@ -1058,10 +1146,7 @@ int ws_stage_neighbours(int64_t nnz, int64_t R) {
 
 bool ws_cross_once(int64_t nnz, int64_t R) { return R > 0 && nnz >= kWsCrossRow * R; }
 
-bool ws_supported(int K) {
-  const int g = (K + 8) / 8;  // tiles per side of the bordered matrix
-  return K >= 8 && K + 1 <= 128 && g >= kWsUnitGMin && g <= kWsUnitGMax;
-}
+bool ws_supported(int K) { return K >= 8 && K + 1 <= 128; }
 
 // Stages (a multiple of 4, one or more ring slots per gather warp) and
 // consumer warps for latent dimension K and nb neighbours per stage (cross:
