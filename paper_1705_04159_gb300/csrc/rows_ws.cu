@@ -141,10 +141,9 @@ struct WsGeom {
 };
 
 struct StageMeta {
-  int rec;    // row record index
   int cnt;    // neighbours in this stage (0 for a row without ratings)
-  int flags;  // 1: first stage of the row, 2: last stage of the row
-  int pad;
+  int flags;  // 1: first stage of the row, 2: last stage of the row, 4: no more rows
+  int pad0, pad1;
 };
 struct RowRec {
   int row;  // -1: no more rows
@@ -396,6 +395,19 @@ __host__ __device__ __forceinline__ int ws_slot(uint32_t n, int S) {
   return (int)(n & 3u) + 4 * (int)((n >> 2) % (uint32_t)(S >> 2));
 }
 
+// A position in a ring of `size` entries and the parity of its passes,
+// stepped instead of divided for: the roles take a step per stage or row.
+struct RingPos {
+  int i = 0;
+  uint32_t parity = 0;  // of the number of times the ring has been passed
+  __device__ __forceinline__ void next(int size) {
+    if (++i == size) {
+      i = 0;
+      parity ^= 1u;
+    }
+  }
+};
+
 template <int NB>
 __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, const WsShared& w,
                                           int S, int* counter, const CUtensorMap* map_hi,
@@ -409,6 +421,8 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
   // so that it can wait for those copies before the block ends
   uint32_t n = 0;             // stage sequence number (the same in every gather warp)
   int q = 0;                  // row sequence number
+  int rec = 0;                // q % kWsRecs
+  RingPos pos;                // of the warp's next stage among its S / 4 slots
   uint32_t last[4] = {~0u, ~0u, ~0u, ~0u};
   // thread 0 prefetches the next row's work entry (row, first, last rating)
   int4 wk = make_int4(-1, 0, 0, 0);
@@ -454,7 +468,7 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
     }
     for (int st = st_first; st < nst; st += 4) {
       const uint32_t nn = n + (uint32_t)st;
-      const int s = ws_slot(nn, S);
+      const int s = wg + 4 * pos.i;  // ws_slot(nn, S)
       const int e = e0 + st * NB;
       const int cnt = row < 0 ? 0 : (e1 - e < NB ? (e1 - e > 0 ? e1 - e : 0) : NB);
       int32_t j[NL];
@@ -469,18 +483,17 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
           rn[u] = __ldg(a.val + e + 4 * NB + k);
         }
       }
-      if (!ws_wait_warp(&w.empty[s], ((nn / (uint32_t)S) & 1u) ^ 1u, w.abort, w.wait_ns)) {
+      if (!ws_wait_warp(&w.empty[s], pos.parity ^ 1u, w.abort, w.wait_ns)) {
         stop = true;
         break;
       }
       if (lane == 0) {
         if (st == 0) {
-          w.recs[q % kWsRecs].row = row;
-          w.recs[q % kWsRecs].nst = row < 0 ? 0 : nst_r;
+          w.recs[rec].row = row;
+          w.recs[rec].nst = row < 0 ? 0 : nst_r;
         }
-        w.meta[s].rec = q % kWsRecs;
         w.meta[s].cnt = cnt;
-        w.meta[s].flags = (st == 0 ? 1 : 0) | (st == nst - 1 ? 2 : 0);
+        w.meta[s].flags = (st == 0 ? 1 : 0) | (st == nst - 1 ? 2 : 0) | (row < 0 ? 4 : 0);
       }
 #pragma unroll
       for (int u = 0; u < NL; ++u) {
@@ -489,7 +502,8 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
       }
       ws_issue_stage<NB>(G, a, map_hi, map_lo, w.stages + s * WsNb<NB>::kStageBytes, &w.tma[s], cnt,
                          j, lane);
-      const int li = (int)((nn >> 2) % (uint32_t)(S >> 2));
+      const int li = pos.i;
+      pos.next(S >> 2);
       last[0] = li == 0 ? nn : last[0];
       last[1] = li == 1 ? nn : last[1];
       last[2] = li == 2 ? nn : last[2];
@@ -498,6 +512,7 @@ __device__ __forceinline__ void ws_gather(const SweepArgs& a, const WsGeom& G, c
     n += (uint32_t)nst;
     if (stop || row < 0) break;
     ++q;
+    rec = rec + 1 == kWsRecs ? 0 : rec + 1;
   }
   // whatever happened downstream, the copies this warp issued land before
   // the block ends (a slot's phases complete in order: its last one is enough)
@@ -522,23 +537,21 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
   // 64-feature blocks, the stride one between atoms
   const uint64_t desc0 = smem_desc_sw128(smem_u32(w.stages), WsNb<NB>::kBlk, kWsAtom);
   uint32_t n = 0;
-  int q = 0;
+  RingPos acc_pos;   // the row's accumulator
+  bool first_row = true;
   for (;;) {
     const int s = ws_slot(n, S);
     if (!ws_wait_warp(&w.tma[s], (n / (uint32_t)S) & 1u, w.abort, w.wait_ns)) break;
     uint8_t* stage = w.stages + s * WsNb<NB>::kStageBytes;
+    const StageMeta m = w.meta[s];
 #pragma unroll
     for (int t = 0; t < NB / 32; ++t)
       ws_patch_rating<NB>(G, stage, w.rating[s * NB + lane + 32 * t], lane + 32 * t);
     fence_proxy_async_smem();
     __syncwarp();
-    const StageMeta m = w.meta[s];
-    const RowRec r = w.recs[m.rec];
-    const int b = q % ws_num_acc<XO>();
+    const int b = acc_pos.i;
     if (m.flags & 1) {
-      if (!ws_wait_warp(&w.acc_empty[b], ((uint32_t)(q / ws_num_acc<XO>()) & 1u) ^ 1u, w.abort,
-                        w.wait_ns))
-        break;
+      if (!ws_wait_warp(&w.acc_empty[b], acc_pos.parity ^ 1u, w.abort, w.wait_ns)) break;
     }
     tc_fence_after();
     if (elect_one()) {
@@ -564,13 +577,14 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
         }
       }
       tc_commit(&w.empty[s]);
-      if ((m.flags & 2) && !(hold && q == 0)) tc_commit(&w.acc_full[b]);
+      if ((m.flags & 2) && !(hold && first_row)) tc_commit(&w.acc_full[b]);
     }
     __syncwarp();
     ++n;
     if (m.flags & 2) {
-      ++q;
-      if (r.row < 0) break;
+      acc_pos.next(ws_num_acc<XO>());
+      first_row = false;
+      if (m.flags & 4) break;
     }
   }
   // every MMA issued has completed before the tensor memory is freed
@@ -645,28 +659,26 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
     }
     tmem_wait_st();
   }
-  int q = 0;
+  RingPos acc_pos, slot_pos, rec_pos;
   uint32_t nsync = 0;  // completed phases of drain_sync
   for (;;) {
-    const int b = q % ws_num_acc<XO>();
-    if (!ws_wait_warp(&w.acc_full[b], (uint32_t)(q / ws_num_acc<XO>()) & 1u, w.abort, w.wait_ns))
-      return;
+    const int b = acc_pos.i;
+    if (!ws_wait_warp(&w.acc_full[b], acc_pos.parity, w.abort, w.wait_ns)) return;
     tc_fence_after();
-    const RowRec r = w.recs[q % kWsRecs];
+    const RowRec r = w.recs[rec_pos.i];
     if (r.row < 0) {
       // one stop record per consumer, in slot order
-      for (int i = 0; i < C; ++i) {
-        const int c = (q + i) % C;
-        const int use = (q + i) / C;
-        if (!ws_wait_warp(&w.slot_empty[c], ((uint32_t)use & 1u) ^ 1u, w.abort, w.wait_ns)) return;
+      for (int i = 0; i < C; ++i, slot_pos.next(C)) {
+        const int c = slot_pos.i;
+        if (!ws_wait_warp(&w.slot_empty[c], slot_pos.parity ^ 1u, w.abort, w.wait_ns)) return;
         if (m == 0) reinterpret_cast<int*>(w.slots + c * slotf)[0] = -1;
         __syncwarp();
         if (lane == 0) mbar_arrive(&w.slot_full[c]);
       }
       return;
     }
-    const int c = q % C;
-    if (!ws_wait_warp(&w.slot_empty[c], ((uint32_t)(q / C) & 1u) ^ 1u, w.abort, w.wait_ns)) return;
+    const int c = slot_pos.i;
+    if (!ws_wait_warp(&w.slot_empty[c], slot_pos.parity ^ 1u, w.abort, w.wait_ns)) return;
     float* slot = w.slots + c * slotf;
     float* tiles = slot + 4;
     float* thr = tiles + G.ntile * kWsTileF;
@@ -756,7 +768,9 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
       mbar_arrive(&w.acc_empty[b]);
       mbar_arrive(&w.slot_full[c]);
     }
-    ++q;
+    acc_pos.next(ws_num_acc<XO>());
+    slot_pos.next(C);
+    rec_pos.next(kWsRecs);
   }
 }
 
