@@ -277,9 +277,9 @@ __device__ __forceinline__ uint32_t idesc_bf16_mn(int M, int N) {
 // ------------------------------------------------------------- gather --
 // The four gather warps take the stages of the row sequence in turn (stage n
 // by warp n % 4), so four stages are filled side by side.  In the warp that
-// fills stage n, lane l holds neighbours l, l + 32, .. (NB / 32 of them);
-// lane g < 4 ceil(cnt / 16) copies the rows of neighbours 4g .. 4g + 3 into
-// both operand tiles with one gather4 per 64-feature block and tile (with
+// fills stage n, lane l holds neighbours l, l + 32, .. (NB / 32 of them); the
+// rows of neighbours 4g .. 4g + 3, g < 4 ceil(cnt / 16), are copied into both
+// operand tiles with one gather4 per 64-feature block and tile (with
 // WsNb::kSplitCopy, the first block only: each lane copies the rest of its
 // neighbours' rows by cp.async).  Rows past cnt (up to the MMA's
 // 16-neighbour step) are read at an out-of-range row index, which the copy
@@ -317,19 +317,10 @@ __device__ __forceinline__ void ws_issue_stage(const WsGeom& G, const SweepArgs&
                                                const int32_t (&j)[NB / 32], int lane) {
   const int ngroups = 4 * ((cnt + 15) >> 4);
   const int nblk = G.KA > 64 ? 2 : 1;
-  // ids of neighbours 4 lane .. 4 lane + 3 (out of range past cnt)
-  int y[4];
+  // row ids of this lane's neighbours, out of range past cnt
+  int y[NB / 32];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int k = 4 * lane + i;
-    int v = 0;
-#pragma unroll
-    for (int u = 0; u < NB / 32; ++u) {
-      const int t = __shfl_sync(0xffffffffu, j[u], k & 31);
-      if ((k >> 5) == u) v = t;
-    }
-    y[i] = k < cnt ? v : (int)a.n_other;
-  }
+  for (int u = 0; u < NB / 32; ++u) y[u] = lane + 32 * u < cnt ? (int)j[u] : (int)a.n_other;
   // the arrive (release) publishes the lanes' metadata and rating writes with
   // the copies: the MMA warp waits for this barrier alone
   const bool split = WsNb<NB>::kSplitCopy && nblk == 2;
@@ -337,12 +328,37 @@ __device__ __forceinline__ void ws_issue_stage(const WsGeom& G, const SweepArgs&
   __syncwarp();
   if (lane == 0) mbar_arrive_expect_tx(bar, (uint32_t)(ngroups * ntma * 2 * 512));
   __syncwarp();
-  if (lane < ngroups) {
-    const uint32_t hi = smem_u32(stage) + (uint32_t)((lane >> 1) * kWsAtom + (lane & 1) * 512);
-    for (int b = 0; b < ntma; ++b) {
-      const uint32_t off = (uint32_t)(b * WsNb<NB>::kBlk);
-      tma_gather4(hi + off, map_hi, 64 * b, y[0], y[1], y[2], y[3], bar);
-      tma_gather4(hi + WsNb<NB>::kOpBytes + off, map_lo, 64 * b, y[0], y[1], y[2], y[3], bar);
+  // One elected lane issues every copy, the ids coming to it by shuffles.
+  // Issued by the lanes that hold the ids, each copy goes through a loop over
+  // the lanes' operands: about 100 cycles per gather4, 2.3-3.4k per
+  // 32-neighbour stage of K = 100 against 1.0-1.4k this way.
+  const uint32_t hi0 = smem_u32(stage);
+#pragma unroll
+  for (int u = 0; u < NB / 32; ++u) {
+    for (int g4 = 0; g4 < 8; g4 += 4) {  // 16 neighbours
+      if (8 * u + g4 >= ngroups) break;
+      int z[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) z[i] = __shfl_sync(0xffffffffu, y[u], 4 * g4 + i);
+      if (elect_one()) {
+        const uint32_t hi = hi0 + (uint32_t)((8 * u + g4) * 512);  // two groups per atom
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const int* r = z + 4 * g;
+          const uint32_t dst = hi + g * 512;
+          tma_gather4(dst, map_hi, 0, r[0], r[1], r[2], r[3], bar);
+          tma_gather4(dst + WsNb<NB>::kOpBytes, map_lo, 0, r[0], r[1], r[2], r[3], bar);
+        }
+        if (ntma == 2) {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const int* r = z + 4 * g;
+            const uint32_t dst = hi + g * 512 + WsNb<NB>::kBlk;
+            tma_gather4(dst, map_hi, 64, r[0], r[1], r[2], r[3], bar);
+            tma_gather4(dst + WsNb<NB>::kOpBytes, map_lo, 64, r[0], r[1], r[2], r[3], bar);
+          }
+        }
+      }
     }
   }
   if (split) {
