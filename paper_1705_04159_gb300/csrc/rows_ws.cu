@@ -806,13 +806,15 @@ __device__ __forceinline__ void ws_drain(const SweepArgs& a, const WsGeom& G, co
 // pair t of row g (lane 4 g + t), taking the operands' k index t for column 2t
 // and t + 4 for column 2t + 1.  So tiles are loaded by 8-byte conflict-free
 // loads and never rearranged.
-// What bounds it: instruction issue and latency of one warp (at K = 100, 14.8k
-// warp instructions and 3.7k shared-memory wavefronts a row; the right-looking
-// FP32 form before it needed 17.2k and 7.3k, and its wavefronts alone were 72%
-// of what the SM can serve).  Six rows side by side on an SM, nothing else
-// running: 5.43 -> 4.53 us per row at K = 100, 2.80 -> 2.41 at K = 64, 1.28 ->
-// 1.14 at K = 33; error of the draws against FP64 2.8e-7 -> 2.4e-7, 2.1e-7 ->
-// 1.7e-7 and 1.4e-7 -> 1.2e-7.
+// What bounds it: instruction issue and latency of one warp (at K = 100, about
+// 14k warp instructions and 3.7k shared-memory wavefronts a row; the
+// right-looking FP32 form before it needed 17.2k and 7.3k, and its wavefronts
+// alone were 72% of what the SM can serve).  Six rows side by side on an SM,
+// nothing else running: 5.43 -> 4.15 us per row at K = 100, 2.80 -> 2.10 at
+// K = 64, 1.28 -> 0.96 at K = 32; error of the draws against FP64 2.8e-7 ->
+// 2.4e-7, 2.1e-7 -> 1.7e-7 and 1.4e-7 -> 1.2e-7.  Two pairs of row tiles per
+// step of the update measured as fast as three and faster than four (4.29 us
+// at K = 100, 2.26 at K = 64), in fewer registers.
 __device__ __forceinline__ int tidx(int I, int J) { return I * (I + 1) / 2 + J; }
 
 __device__ __forceinline__ float2 ldf2(const float* p) { return *reinterpret_cast<const float2*>(p); }
@@ -940,9 +942,8 @@ __device__ __forceinline__ bool ws_cholesky(const WsGeom& G, float* T, const flo
     if (J > 0) {
       int I0 = J;
 #pragma unroll 1
-      for (; g - I0 > 4; I0 += 8) ws_update<4>(T, g, J, I0, fo);
-      if (g - I0 > 2) ws_update<2>(T, g, J, I0, fo);
-      else if (g - I0 > 0) ws_update<1>(T, g, J, I0, fo);
+      for (; g - I0 > 2; I0 += 4) ws_update<2>(T, g, J, I0, fo);
+      if (g - I0 > 0) ws_update<1>(T, g, J, I0, fo);
       __syncwarp();
     }
     float* D = T + tidx(J, J) * kWsTileF;
@@ -987,7 +988,8 @@ __device__ __forceinline__ bool ws_cholesky(const WsGeom& G, float* T, const flo
 // lane 2 J + h keeps columns 8 J + 4 h .. + 3 (so one pass covers all of a
 // row), the block's eight values come to every lane by shuffles, every lane
 // solves the 8 x 8 system, and each subtracts the block's part from its
-// columns.  The tiles of the next block are loaded while this one is used.
+// columns.  The next block's diagonal tile is loaded a step ahead; the other
+// tiles are not, which would take 32 registers more.
 __device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const float* rinv,
                                         const float* zv, int lane, float* out) {
   const int K = G.K;
@@ -1000,7 +1002,6 @@ __device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const f
     const float4 z = *reinterpret_cast<const float4*>(zv + (J <= IK ? 8 * J + h4 : 0));
     v[0] = y.x + z.x; v[1] = y.y + z.y; v[2] = y.z + z.z; v[3] = y.w + z.w;
   }
-  float4 lc[8];         // the lane's columns of tile (I, J), J < I
   float d[8][8], rd[8];  // the strict lower triangle of tile (I, I), 1 / diagonal
   auto load_diag = [&](int I) {
     const float* Dg = T + tidx(I, I) * kWsTileF;
@@ -1015,14 +1016,8 @@ __device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const f
     }
     ld8(rinv + 8 * I, rd);
   };
-  auto load_cols = [&](int I) {
-    const float* L = T + tidx(I, J < I ? J : 0) * kWsTileF + h4;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) lc[q] = *reinterpret_cast<const float4*>(L + trow(q));
-  };
   int I = (K - 1) >> 3;
   load_diag(I);
-  load_cols(I);
 #pragma unroll 1
   for (; I >= 0; --I) {
     float u[8];
@@ -1035,9 +1030,11 @@ __device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const f
 #pragma unroll
       for (int r = 0; r < c; ++r) u[r] = fmaf(-d[c][r], u[c], u[r]);
     }
-    const int next = I > 0 ? I - 1 : 0;
-    load_diag(next);
     if (J < I) {
+      const float* L = T + tidx(I, J) * kWsTileF + h4;
+      float4 lc[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) lc[q] = *reinterpret_cast<const float4*>(L + trow(q));
 #pragma unroll
       for (int q = 7; q >= 0; --q) {
         v[0] = fmaf(-lc[q].x, u[q], v[0]);
@@ -1049,7 +1046,7 @@ __device__ __forceinline__ void ws_back(const WsGeom& G, const float* T, const f
 #pragma unroll
       for (int k = 0; k < 4; ++k) v[k] = h4 ? u[4 + k] : u[k];
     }
-    load_cols(next);
+    load_diag(I > 0 ? I - 1 : 0);
   }
   const int c0 = 8 * J + h4;
   if ((K & 3) == 0) {  // the row of X starts on a 16-byte boundary
