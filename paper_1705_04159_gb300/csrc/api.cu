@@ -61,7 +61,7 @@ void free_handle(Handle* h) {
     SideDev& sd = h->side[s];
     dfree(sd.ptr); dfree(sd.idx); dfree(sd.val); dfree(sd.perm); dfree(sd.X); dfree(sd.Xhi);
     dfree(sd.Xlo); dfree(sd.work);
-    dfree(sd.lam); dfree(sd.mu); dfree(sd.lamaug); dfree(sd.lchol); dfree(sd.linvT); dfree(sd.xbar); dfree(sd.S);
+    dfree(sd.lam); dfree(sd.mu); dfree(sd.lamaug); dfree(sd.lchol); dfree(sd.linvT); dfree(sd.tiny_pre); dfree(sd.xbar); dfree(sd.S);
     dfree(sd.piece_row); dfree(sd.piece_e0); dfree(sd.piece_e1); dfree(sd.hub_piece0);
   }
   dfree(h->mu0); dfree(h->W0inv); dfree(h->red); dfree(h->wscr); dfree(h->red2); dfree(h->wscr2);

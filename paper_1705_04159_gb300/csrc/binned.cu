@@ -120,7 +120,7 @@ int launch_other_bins(Handle* h, int s, const SweepArgs& a, cudaStream_t st) {
   }
   r.row_begin = e_light;
   r.row_end = sd.R;
-  return launch_rows_rank1(r, sd.lchol, sd.linvT, (int)sd.tiny_max, st, &h->kernels);
+  return launch_rows_rank1(r, sd.lchol, sd.linvT, sd.tiny_pre, (int)sd.tiny_max, st, &h->kernels);
 }
 
 }  // namespace
@@ -139,7 +139,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
   sd.light_max = light_max;
   sd.hub_min = hub_min;
   for (int b = 0; b < kNumBins; ++b) sd.bin_count[b] = 0;
-  int64_t n_hub = 0;
+  int64_t n_hub = 0, tiny_ratings = 0;
   for (int64_t q = 0; q < R; ++q) {
     const int64_t d = sd.deg_h[q];
     int bin;
@@ -148,6 +148,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
     else if (d <= light_max) bin = kBinLight;
     else bin = kBinHeavy;
     sd.bin_count[bin] += 1;
+    if (bin == kBinTiny) tiny_ratings += d;
     if (bin == kBinHub) {
       // degree order puts every hub before every other row
       if (q != n_hub) {
@@ -156,6 +157,19 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
       }
       ++n_hub;
     }
+  }
+  const int64_t pre = rank1_pre_floats(h->K, h->side[1 - s].R, sd.bin_count[kBinTiny], tiny_ratings);
+  if (pre != sd.tiny_pre_len) {
+    BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
+    cudaFree(sd.tiny_pre);
+    sd.tiny_pre = nullptr;
+    sd.tiny_pre_len = 0;
+    // without the memory the products are formed row by row
+    if (pre > 0 && cudaMalloc(&sd.tiny_pre, sizeof(float) * pre) != cudaSuccess) {
+      cudaGetLastError();
+      sd.tiny_pre = nullptr;
+    }
+    if (sd.tiny_pre) sd.tiny_pre_len = pre;
   }
   if (!new_hubs) return BPMF_OK;
   // piece length: half the hub threshold, at most kPiece ratings

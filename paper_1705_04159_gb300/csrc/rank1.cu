@@ -24,7 +24,7 @@
 // So, with c = L_s^-1 b,
 //   y = M_{d-1}^-1 ... M_0^-1 c = L*^-1 b,
 //   u = L_s^-T M_0^-T ... M_{d-1}^-T (y + z) = L*^-T (y + z):
-// one product of L_s^-1 with d + 1 vectors, one with L_s^-T, and O(d^2)
+// products of L_s^-1 with the x_t and b, one of L_s^-T, and O(d^2)
 // warp-wide scans -- instead of d K column steps, each a dependent square root
 // and division, of successive rank-one updates of the factor.  This is the
 // cheaper kernel for rows with few ratings of paper Sec. III (Fig. 2).  The
@@ -32,17 +32,26 @@
 // the other row kernels (L*_ii^2 against Lambda*_ii) still decides which rows
 // go to the FP64 redo.
 //
+// The w_t do not depend on the row: w_t = sqrt(alpha) L_s^-1 v_j, and
+// c = L_s^-1 b0 + alpha sum_t r_t L_s^-1 v_j.  Where the bin's ratings outnumber
+// the other side's rows, lower_rows forms L_s^-1 v_j for every j once per sweep
+// (PRE), and a row is left with the scans and the product with L_s^-T.
+//
 // Layout.  linv_columns writes T = (L_s^-1)^T, KP x LD floats (KP = K rounded
 // up to 32, LD = KP + 4, zero outside the triangle), once per sweep, in FP64
 // arithmetic from the packed FP32 factor.  Each CTA keeps T in shared memory;
-// its warps take rows in turn, one warp per row, lane l owning elements
-// l + 32 m.  T[k][i] at k LD + i: the forward product reads T[k][l + 32 m]
-// (consecutive in l) one float at a time, and the transposed one reads
-// T[l + 32 m][k .. k + 3] as one 16-byte load (rows 16-byte aligned, LD = 4
-// mod 32, so eight lanes of a load phase fall on eight different groups of
-// four banks).  Per warp: d + 1 vectors (x_t, then w_t and
-// p_t; the last b, then c, then y), the d prefix sums B'_s (the backward pass
-// recomputes rho and gamma from them) and the normals z.
+// its warps take groups of kR1Rows rows in turn, one row after the other up to
+// the last product, which they share (a value of T read once serves them all).
+// Lane l owns elements l + 32 m.  T[k][i] at k LD + i: the forward product
+// reads T[k][l + 32 m] (consecutive in l) one float at a time, and the
+// transposed one reads T[l + 32 m][k .. k + 3] as one 16-byte load (rows
+// 16-byte aligned, LD = 4 mod 32, so eight lanes of a load phase fall on eight
+// different groups of four banks).  Per warp: d + 1 vectors (w_t and p_t; the
+// last c, then y), the d prefix sums B'_s (the backward pass recomputes rho and
+// gamma from them) and kR1Rows vectors of normals, then of right-hand sides.
+//
+// What bounds it: issue.  480,000 rows of 1.9 ratings on average, K = 64,
+// 5,800 rows on the other side: @PRE@.
 #include <cuda_runtime.h>
 #include <float.h>
 
@@ -56,6 +65,7 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kR1MaxWarps = 8;
+constexpr int kR1Rows = 4;  // rows of a group (they share the product with L_s^-T)
 
 __device__ __forceinline__ int tri(int i) { return (i * (i + 1)) >> 1; }
 
@@ -67,40 +77,54 @@ __device__ __forceinline__ float comp(const float4& v, int e) {
 // row k of T, i.e. column k of L_s^-1: L_s t = e_k by column-oriented forward
 // substitution in FP64 -- lane l holds t_i for i = l + 32 m; at step j the
 // owner of row j scales t_j by 1 / L_jj (computed before the loop) and
-// broadcasts it, and every lane subtracts L_ij t_j from its rows i > j, so a
-// step is one shuffle and one multiply-add, with no reduction.
-__global__ void __launch_bounds__(32) linv_columns(const float* __restrict__ lchol, int K, int KP,
+// broadcasts it, and every lane subtracts L_ij t_j from its rows, so a step is
+// one shuffle and one multiply-add, with no reduction.  The block of L from
+// row and column k on is first brought to shared memory in FP64, square with
+// zeros above the diagonal (rows at or above the step then subtract nothing)
+// and an odd row stride: no step waits for a global load, converts or branches.
+int linv_smem(int K) { return (int)sizeof(double) * K * (K | 1); }
+
+template <int NPL>
+__global__ void __launch_bounds__(32) linv_columns(const float* __restrict__ lchol, int K,
                                                    float* __restrict__ T) {
-  constexpr int kMaxNpl = kMaxK / 32;
-  const int k = blockIdx.x, lane = threadIdx.x, LD = KP + 4;
+  constexpr int KP = 32 * NPL, LD = KP + 4;
+  extern __shared__ double s_l[];
+  const int k = blockIdx.x, lane = threadIdx.x, n = K - k;
   float* out = T + (int64_t)k * LD;
-  double t[kMaxNpl], rdiag[kMaxNpl];
+  for (int i = lane; i < LD; i += 32)
+    if (i < k || i >= K) out[i] = 0.f;
+  if (n <= 0) return;
+  const int ld = n | 1;
+  for (int i = 0; i < n; ++i) {
+    const float* row = lchol + tri(k + i) + k;
 #pragma unroll
-  for (int m = 0; m < kMaxNpl; ++m) {
-    const int i = lane + 32 * m;
-    t[m] = i == k ? 1.0 : 0.0;
-    rdiag[m] = i < K ? 1.0 / (double)lchol[tri(i) + i] : 0.0;
-  }
-  for (int j = k; j < K; ++j) {
-    const int owner = j & 31, mj = j >> 5;
-    double tj = 0.0;
-#pragma unroll
-    for (int m = 0; m < kMaxNpl; ++m)
-      if (m == mj) tj = t[m] * rdiag[m];
-    tj = __shfl_sync(kFull, tj, owner);
-#pragma unroll
-    for (int m = 0; m < kMaxNpl; ++m) {
-      const int i = lane + 32 * m;
-      if (i == j) t[m] = tj;
-      else if (i > j && i < K) t[m] = fma(-(double)lchol[tri(i) + j], tj, t[m]);
+    for (int m = 0; m < NPL; ++m) {
+      const int j = lane + 32 * m;
+      if (j < n) s_l[i * ld + j] = j <= i ? (double)__ldg(row + j) : 0.0;
     }
   }
-  for (int i = lane; i < LD; i += 32) {
-    double v = 0.0;
+  __syncwarp();
+  // local row q = i - k
+  double t[NPL], rdiag[NPL];
 #pragma unroll
-    for (int m = 0; m < kMaxNpl; ++m)
-      if (i == lane + 32 * m) v = t[m];
-    out[i] = i >= k && i < K ? (float)v : 0.f;
+  for (int m = 0; m < NPL; ++m) {
+    const int q = lane + 32 * m;
+    t[m] = q == 0 ? 1.0 : 0.0;
+    rdiag[m] = q < n ? 1.0 / s_l[q * ld + q] : 0.0;
+  }
+#pragma unroll
+  for (int mb = 0; mb < NPL; ++mb) {
+    for (int jj = 0; jj < 32; ++jj) {
+      const int j = 32 * mb + jj;
+      if (j >= n) break;
+      const double tj = __shfl_sync(kFull, t[mb] * rdiag[mb], jj);
+      if (lane == jj) out[k + j] = (float)tj;
+#pragma unroll
+      for (int m = mb; m < NPL; ++m) {
+        const int q = min(lane + 32 * m, n - 1);
+        t[m] = fma(-s_l[q * ld + j], tj, t[m]);
+      }
+    }
   }
 }
 
@@ -193,26 +217,67 @@ __device__ __forceinline__ void lower_times(const float* T, float* v, int K, int
   __syncwarp();
 }
 
-// v_g <- M^-1 v_g for G vectors (each lane reads and writes its own elements)
+// The factor of p = v_0 (its rho and B', the latter to Bp) and v_g <- M^-1 v_g
+// for the G vectors v_1 .. v_G after it; the prefix sums of p^2 and of the
+// p y_g do not depend on one another, so they are scanned together.  Each lane
+// reads and writes its own elements.
 template <int NPL, int G>
-__device__ __forceinline__ void factor_solve(float* v, const float (&p)[NPL],
-                                             const float (&rho)[NPL], const float (&gam)[NPL],
-                                             int lane) {
+__device__ __forceinline__ void factor_step(float* v, float* Bp, float (&pr)[NPL], int lane) {
   constexpr int KP = 32 * NPL;
-  float y[G][NPL], s[G][NPL], ex[G][NPL];
+  float p[NPL], y[G][NPL], s[G + 1][NPL], ex[G + 1][NPL];
+#pragma unroll
+  for (int m = 0; m < NPL; ++m) {
+    p[m] = v[lane + 32 * m];
+    s[G][m] = p[m] * p[m];
+  }
 #pragma unroll
   for (int g = 0; g < G; ++g)
 #pragma unroll
     for (int m = 0; m < NPL; ++m) {
-      y[g][m] = v[g * KP + lane + 32 * m];
+      y[g][m] = v[(g + 1) * KP + lane + 32 * m];
       s[g][m] = p[m] * y[g][m];
     }
-  scan_prefix<G, NPL>(s, ex, lane);
+  scan_prefix<G + 1, NPL>(s, ex, lane);
 #pragma unroll
-  for (int g = 0; g < G; ++g)
+  for (int m = 0; m < NPL; ++m) {
+    const float Bi = 1.f + s[G][m], Be = 1.f + ex[G][m];
+    const float r1 = rsqrtf(Be), r2 = rsqrtf(Bi);
+    const float rho = Be * r1 * r2, gam = p[m] * r1 * r2;
+    Bp[lane + 32 * m] = Bi;
+    pr[m] *= rho * rho;
 #pragma unroll
-    for (int m = 0; m < NPL; ++m)
-      v[g * KP + lane + 32 * m] = fmaf(rho[m], y[g][m], -gam[m] * ex[g][m]);
+    for (int g = 0; g < G; ++g)
+      v[(g + 1) * KP + lane + 32 * m] = fmaf(rho, y[g][m], -gam * ex[g][m]);
+  }
+}
+
+// M^-1 on n vectors at v, given p and its rho and gamma (those past the first
+// few of a row with many ratings)
+template <int NPL>
+__device__ __forceinline__ void factor_rest(float* v, int n, const float* p, const float* Bp, int lane) {
+  constexpr int KP = 32 * NPL;
+  float pv[NPL], rho[NPL], gam[NPL];
+#pragma unroll
+  for (int m = 0; m < NPL; ++m) {
+    const int i = lane + 32 * m;
+    pv[m] = p[i];
+    const float Bi = Bp[i];
+    const float Be = i == 0 ? 1.f : Bp[i - 1];
+    const float r1 = rsqrtf(Be), r2 = rsqrtf(Bi);
+    rho[m] = Be * r1 * r2;
+    gam[m] = pv[m] * r1 * r2;
+  }
+  for (; n > 0; --n, v += KP) {
+    float y[NPL], s[1][NPL], ex[1][NPL];
+#pragma unroll
+    for (int m = 0; m < NPL; ++m) {
+      y[m] = v[lane + 32 * m];
+      s[0][m] = pv[m] * y[m];
+    }
+    scan_prefix<1, NPL>(s, ex, lane);
+#pragma unroll
+    for (int m = 0; m < NPL; ++m) v[lane + 32 * m] = fmaf(rho[m], y[m], -gam[m] * ex[0][m]);
+  }
 }
 
 template <int NPL>
@@ -228,28 +293,52 @@ __device__ __forceinline__ void lower_times_n(const float* T, float* v, int n, i
   }
 }
 
+// floats of shared memory per warp for rows of degree <= D
+__host__ __device__ __forceinline__ int r1_warp_floats(int D, int KP) {
+  return (2 * D + 1 + kR1Rows) * KP;
+}
+
+// W row j = L_s^-1 (row j of V) for j < n, and row n = L_s^-1 b0: KP floats per
+// row, zero past K.  A warp takes four rows at a time.
 template <int NPL>
-__device__ __forceinline__ void factor_solve_n(float* v, int n, const float (&p)[NPL],
-                                               const float (&rho)[NPL], const float (&gam)[NPL],
-                                               int lane) {
-  constexpr int KP = 32 * NPL;
-  for (int g0 = 0; g0 < n; g0 += 4) {
-    switch (min(4, n - g0)) {
-      case 1: factor_solve<NPL, 1>(v + g0 * KP, p, rho, gam, lane); break;
-      case 2: factor_solve<NPL, 2>(v + g0 * KP, p, rho, gam, lane); break;
-      case 3: factor_solve<NPL, 3>(v + g0 * KP, p, rho, gam, lane); break;
-      default: factor_solve<NPL, 4>(v + g0 * KP, p, rho, gam, lane); break;
+__global__ void __launch_bounds__(32 * kR1MaxWarps)
+    lower_rows(const float* __restrict__ V, int64_t n, int K, const float* __restrict__ b0,
+               const float* __restrict__ Tg, float* __restrict__ W) {
+  constexpr int KP = 32 * NPL, LD = KP + 4;
+  extern __shared__ __align__(16) float r1s[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int e = threadIdx.x; e < KP * LD / 4; e += blockDim.x)
+    reinterpret_cast<float4*>(r1s)[e] = __ldg(reinterpret_cast<const float4*>(Tg) + e);
+  __syncthreads();
+  float* vec = r1s + KP * LD + warp * 4 * KP;
+  const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * 4;
+  for (int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * 4; j0 <= n; j0 += stride) {
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const float* v = j0 + g < n ? V + (j0 + g) * K : b0;
+#pragma unroll
+      for (int m = 0; m < NPL; ++m) {
+        const int i = lane + 32 * m;
+        vec[g * KP + i] = j0 + g <= n && i < K ? __ldg(v + i) : 0.f;
+      }
     }
+    __syncwarp();
+    lower_times<NPL, 4>(r1s, vec, K, lane);
+#pragma unroll
+    for (int g = 0; g < 4; ++g)
+      if (j0 + g <= n) {
+#pragma unroll
+        for (int m = 0; m < NPL; ++m) W[(j0 + g) * KP + lane + 32 * m] = vec[g * KP + lane + 32 * m];
+      }
   }
 }
 
-// floats of shared memory per warp for rows of degree <= D
-__host__ __device__ __forceinline__ int r1_warp_floats(int D, int KP) { return (2 * D + 2) * KP; }
-
-template <int NPL>
+// PRE: W holds L_s^-1 of the other side's rows and of b0 (lower_rows)
+template <int NPL, bool PRE>
 __global__ void __launch_bounds__(32 * kR1MaxWarps)
     row_rank1(const SweepArgs a, const float* __restrict__ lchol, const float* __restrict__ Tg,
-              int D, int warps) {
+              const float* __restrict__ W, int D, int warps) {
   constexpr int KP = 32 * NPL, LD = KP + 4;
   extern __shared__ __align__(16) float r1s[];
   const int K = a.K;
@@ -263,10 +352,10 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
   __syncthreads();  // the only block-wide barrier; warps go their own way after it
   float* vec = T + KP * LD + warp * r1_warp_floats(D, KP);
   float* Bp = vec + (D + 1) * KP;
-  float* zb = Bp + D * KP;
+  float* zb = Bp + D * KP;  // [kR1Rows][KP]
   // per-element constants: b0 = Lambda_s mu_s (the bordered hyper matrix's
-  // last row), the diagonal of Lambda_s and that of L_s squared
-  const float* b0 = a.lamaug + (int64_t)K * (K + 1);
+  // last row) or L_s^-1 b0, the diagonal of Lambda_s and that of L_s squared
+  const float* b0 = PRE ? W + a.n_other * KP : a.lamaug + (int64_t)K * (K + 1);
   float bs[NPL], ds[NPL], ls2[NPL];
 #pragma unroll
   for (int m = 0; m < NPL; ++m) {
@@ -278,176 +367,231 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
   }
   const float sa = sqrtf(a.alpha);
   const uint32_t tw = *a.tp;
-  const int64_t stride = (int64_t)gridDim.x * warps;
-  for (int64_t slot = a.row_begin + (int64_t)blockIdx.x * warps + warp; slot < a.row_end;
-       slot += stride) {
-    __syncwarp();  // the previous row's reads of the warp's buffers are done
-    const int row = a.rows ? a.rows[slot] : (int)slot;
-    const int64_t p0 = a.ptr[row];
-    const int d = (int)(a.ptr[row + 1] - p0);
-    if (d > D) {  // not in this bin's degree range: left to the FP64 redo
-      if (lane == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
-      continue;
+  const int64_t stride = (int64_t)gridDim.x * warps * kR1Rows;
+  for (int64_t s0 = a.row_begin + ((int64_t)blockIdx.x * warps + warp) * kR1Rows; s0 < a.row_end;
+       s0 += stride) {
+    __syncwarp();  // the previous group's reads of the warp's buffers are done
+    const int nrow = (int)min((int64_t)kR1Rows, a.row_end - s0);
+    // lane r: row r of the group, its first rating and its degree
+    int grow = -1, gdeg = 0;
+    int64_t gp0 = 0;
+    if (lane < nrow) {
+      grow = a.rows ? a.rows[s0 + lane] : (int)(s0 + lane);
+      gp0 = a.ptr[grow];
+      gdeg = (int)(a.ptr[grow + 1] - gp0);
     }
-    // x_t = sqrt(alpha) v_t, b = b0 + alpha sum_t r_t v_t, Lambda*_ii
-    float b[NPL], d0[NPL];
-#pragma unroll
-    for (int m = 0; m < NPL; ++m) {
-      b[m] = bs[m];
-      d0[m] = ds[m];
-    }
-    for (int t = 0; t < d; ++t) {
-      const int32_t j = __ldg(a.idx + p0 + t);
-      const float ar = a.alpha * __ldg(a.val + p0 + t);
-      const float* vj = a.Vo + (int64_t)j * K;
-#pragma unroll
-      for (int m = 0; m < NPL; ++m) {
-        const int i = lane + 32 * m;
-        const float v = i < K ? __ldg(vj + i) : 0.f;
-        const float x = sa * v;
-        vec[t * KP + i] = x;
-        b[m] = fmaf(ar, v, b[m]);
-        d0[m] = fmaf(x, x, d0[m]);
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < NPL; ++m) vec[d * KP + lane + 32 * m] = b[m];
-    if (4 * lane < KP) {
+    // normals of the group's rows, a lane per four
+    for (int e = lane; e < kR1Rows * KP / 4; e += 32) {
+      const int r = e / (KP / 4), q = e - r * (KP / 4);
+      const int row = __shfl_sync(kFull, grow, r);
       float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (4 * lane < K) {
-        z = normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)lane, a.sw), a.key));
-        if (4 * lane + 1 >= K) z.y = 0.f;
-        if (4 * lane + 2 >= K) z.z = 0.f;
-        if (4 * lane + 3 >= K) z.w = 0.f;
+      if (4 * q < K && r < nrow) {
+        z = normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)q, a.sw), a.key));
+        if (4 * q + 1 >= K) z.y = 0.f;
+        if (4 * q + 2 >= K) z.z = 0.f;
+        if (4 * q + 3 >= K) z.w = 0.f;
       }
-      *reinterpret_cast<float4*>(zb + 4 * lane) = z;
+      *reinterpret_cast<float4*>(zb + 4 * e) = z;
     }
     __syncwarp();
-    // w_t = L_s^-1 x_t and c = L_s^-1 b
-    lower_times_n<NPL>(T, vec, d + 1, K, lane);
-    // the factors: p_s, then M_s^-1 applied to w_{s+1} .. w_{d-1} and to c
-    float pr[NPL];  // prod_s rho_s^2 = (L_s)_ii^2 / L*_ii^2
-#pragma unroll
-    for (int m = 0; m < NPL; ++m) pr[m] = 1.f;
-    for (int s = 0; s < d; ++s) {
-      float p[NPL], rho[NPL], gam[NPL], q[1][NPL], qx[1][NPL];
+    unsigned drop = 0;  // rows of the group left to the FP64 redo
+    for (int r = 0; r < nrow; ++r) {
+      const int d = __shfl_sync(kFull, gdeg, r);
+      const int64_t p0 = __shfl_sync(kFull, gp0, r);
+      if (d > D) {  // not in this bin's degree range
+        drop |= 1u << r;
+        continue;
+      }
+      // x_t = sqrt(alpha) v_t, b = b0 + alpha sum_t r_t v_t, Lambda*_ii; with
+      // PRE, of L_s^-1 v_t in place of v_t (but for Lambda*_ii)
+      float b[NPL], d0[NPL];
 #pragma unroll
       for (int m = 0; m < NPL; ++m) {
-        p[m] = vec[s * KP + lane + 32 * m];
-        q[0][m] = p[m] * p[m];
+        b[m] = bs[m];
+        d0[m] = ds[m];
       }
-      scan_prefix<1, NPL>(q, qx, lane);
+      for (int t = 0; t < d; ++t) {
+        const int32_t j = __ldg(a.idx + p0 + t);
+        const float ar = a.alpha * __ldg(a.val + p0 + t);
+        const float* vj = a.Vo + (int64_t)j * K;
+        const float* wj = PRE ? W + (int64_t)j * KP : nullptr;
 #pragma unroll
-      for (int m = 0; m < NPL; ++m) {
-        const float Bi = 1.f + q[0][m], Be = 1.f + qx[0][m];
-        const float r1 = rsqrtf(Be), r2 = rsqrtf(Bi);
-        rho[m] = Be * r1 * r2;
-        gam[m] = p[m] * r1 * r2;
-        Bp[s * KP + lane + 32 * m] = Bi;
-        pr[m] *= rho[m] * rho[m];
+        for (int m = 0; m < NPL; ++m) {
+          const int i = lane + 32 * m;
+          const float v = i < K ? __ldg(vj + i) : 0.f;
+          const float x = sa * v;
+          d0[m] = fmaf(x, x, d0[m]);
+          const float w = PRE ? __ldg(wj + i) : v;
+          vec[t * KP + i] = sa * w;
+          b[m] = fmaf(ar, w, b[m]);
+        }
       }
-      factor_solve_n<NPL>(vec + (s + 1) * KP, d - s, p, rho, gam, lane);
-    }
-    __syncwarp();  // B' of other lanes is read below
-    // w = y + z, then M_{d-1}^-T .. M_0^-T
-    float w[NPL];
 #pragma unroll
-    for (int m = 0; m < NPL; ++m) w[m] = vec[d * KP + lane + 32 * m] + zb[lane + 32 * m];
-    for (int s = d - 1; s >= 0; --s) {
-      float t[NPL], ex[NPL], p[NPL], rho[NPL];
+      for (int m = 0; m < NPL; ++m) vec[d * KP + lane + 32 * m] = b[m];
+      if (!PRE) {
+        __syncwarp();
+        // w_t = L_s^-1 x_t and c = L_s^-1 b
+        lower_times_n<NPL>(T, vec, d + 1, K, lane);
+      }
+      // the factors: p_s, then M_s^-1 applied to w_{s+1} .. w_{d-1} and to c
+      float pr[NPL];  // prod_s rho_s^2 = (L_s)_ii^2 / L*_ii^2
+#pragma unroll
+      for (int m = 0; m < NPL; ++m) pr[m] = 1.f;
+      for (int s = 0; s < d; ++s) {
+        float* v = vec + s * KP;
+        float* B = Bp + s * KP;
+        const int n = d - s;
+        switch (n) {
+          case 1: factor_step<NPL, 1>(v, B, pr, lane); break;
+          case 2: factor_step<NPL, 2>(v, B, pr, lane); break;
+          default: factor_step<NPL, 3>(v, B, pr, lane); break;
+        }
+        if (n > 3) {
+          __syncwarp();  // B' of the lanes before
+          factor_rest<NPL>(v + 4 * KP, n - 3, v, B, lane);
+        }
+      }
+      __syncwarp();  // B' of other lanes is read below
+      // w = y + z, then M_{d-1}^-T .. M_0^-T
+      float* zr = zb + r * KP;
+      float w[NPL];
+#pragma unroll
+      for (int m = 0; m < NPL; ++m) w[m] = vec[d * KP + lane + 32 * m] + zr[lane + 32 * m];
+      for (int s = d - 1; s >= 0; --s) {
+        float t[NPL], ex[NPL], p[NPL], rho[NPL];
+#pragma unroll
+        for (int m = 0; m < NPL; ++m) {
+          const int i = lane + 32 * m;
+          p[m] = vec[s * KP + i];
+          const float Bi = Bp[s * KP + i];
+          const float Be = i == 0 ? 1.f : Bp[s * KP + i - 1];
+          const float r1 = rsqrtf(Be), r2 = rsqrtf(Bi);
+          rho[m] = Be * r1 * r2;
+          t[m] = p[m] * r1 * r2 * w[m];  // gamma_i w_i
+        }
+        scan_suffix<NPL>(t, ex, lane);
+#pragma unroll
+        for (int m = 0; m < NPL; ++m) w[m] = fmaf(rho[m], w[m], -p[m] * ex[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < NPL; ++m) zr[lane + 32 * m] = w[m];
+      // pivot rule: L*_ii^2 = (L_s)_ii^2 / pr_i against pivot_rel Lambda*_ii
+      bool bad = false;
 #pragma unroll
       for (int m = 0; m < NPL; ++m) {
         const int i = lane + 32 * m;
-        p[m] = vec[s * KP + i];
-        const float Bi = Bp[s * KP + i];
-        const float Be = i == 0 ? 1.f : Bp[s * KP + i - 1];
-        const float r1 = rsqrtf(Be), r2 = rsqrtf(Bi);
-        rho[m] = Be * r1 * r2;
-        t[m] = p[m] * r1 * r2 * w[m];  // gamma_i w_i
+        if (i < K && !(ls2[m] > pr[m] * fmaxf(a.pivot_rel * d0[m], FLT_MIN))) bad = true;
       }
-      scan_suffix<NPL>(t, ex, lane);
-#pragma unroll
-      for (int m = 0; m < NPL; ++m) w[m] = fmaf(rho[m], w[m], -p[m] * ex[m]);
+      if (__any_sync(kFull, bad)) drop |= 1u << r;
+      __syncwarp();  // the row's buffers are rewritten by the next row
     }
-    // u = L_s^-T w: lane l sums T[l + 32 m][k] w_k over k >= 32 m
-    __syncwarp();  // every lane has read its z
+    // u = L_s^-T w: lane l sums T[l + 32 m][k] w_k over k >= 32 m, for all rows
+    float u[kR1Rows][NPL];
 #pragma unroll
-    for (int m = 0; m < NPL; ++m) zb[lane + 32 * m] = w[m];
-    __syncwarp();
-    float u[NPL];
+    for (int r = 0; r < kR1Rows; ++r)
 #pragma unroll
-    for (int m = 0; m < NPL; ++m) u[m] = 0.f;
+      for (int m = 0; m < NPL; ++m) u[r][m] = 0.f;
 #pragma unroll
     for (int kc = 0; kc < NPL; ++kc) {
 #pragma unroll 2
       for (int k4 = 0; k4 < 32; k4 += 4) {
         const int k = 32 * kc + k4;
         if (k >= K) break;
-        const float4 wv = *reinterpret_cast<const float4*>(zb + k);
+        float4 wv[kR1Rows];
+#pragma unroll
+        for (int r = 0; r < kR1Rows; ++r) wv[r] = *reinterpret_cast<const float4*>(zb + r * KP + k);
 #pragma unroll
         for (int m = 0; m <= kc; ++m) {
           const float4 t4 = *reinterpret_cast<const float4*>(T + (lane + 32 * m) * LD + k);
-          u[m] = fmaf(t4.x, wv.x, u[m]);
-          u[m] = fmaf(t4.y, wv.y, u[m]);
-          u[m] = fmaf(t4.z, wv.z, u[m]);
-          u[m] = fmaf(t4.w, wv.w, u[m]);
+#pragma unroll
+          for (int r = 0; r < kR1Rows; ++r) {
+            u[r][m] = fmaf(t4.x, wv[r].x, u[r][m]);
+            u[r][m] = fmaf(t4.y, wv[r].y, u[r][m]);
+            u[r][m] = fmaf(t4.z, wv[r].z, u[r][m]);
+            u[r][m] = fmaf(t4.w, wv[r].w, u[r][m]);
+          }
         }
       }
     }
-    // pivot rule: L*_ii^2 = (L_s)_ii^2 / pr_i against pivot_rel Lambda*_ii
-    bool bad = false;
 #pragma unroll
-    for (int m = 0; m < NPL; ++m) {
-      const int i = lane + 32 * m;
-      if (i < K && !(ls2[m] > pr[m] * fmaxf(a.pivot_rel * d0[m], FLT_MIN))) bad = true;
-    }
-    if (__any_sync(kFull, bad)) {
-      if (lane == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
-      continue;
-    }
-    float* out = a.X + (int64_t)row * K;
+    for (int r = 0; r < kR1Rows; ++r) {
+      const int row = __shfl_sync(kFull, grow, r);
+      if (r < nrow && !(drop >> r & 1u)) {
+        float* out = a.X + (int64_t)row * K;
 #pragma unroll
-    for (int m = 0; m < NPL; ++m) {
-      const int i = lane + 32 * m;
-      if (i < K) out[i] = u[m];
+        for (int m = 0; m < NPL; ++m) {
+          const int i = lane + 32 * m;
+          if (i < K) out[i] = u[r][m];
+        }
+      }
     }
+    if (lane < nrow && (drop >> lane & 1u)) a.flag_rows[atomicAdd(a.flag_count, 1)] = grow;
   }
 }
 
+// CTAs of `kern` that fill the device, at most `need`
+template <typename F>
+int r1_grid(F kern, int threads, size_t smem, int64_t need, unsigned* grid) {
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  int dev = 0, sms = 1, occ = 1;
+  BPMF_CUDA_CHECK(cudaGetDevice(&dev));
+  BPMF_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  BPMF_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem));
+  *grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sms * std::max(occ, 1)));
+  return BPMF_OK;
+}
+
 template <int NPL>
-int launch_r1(const SweepArgs& a, const float* lchol, float* T, int D, cudaStream_t st) {
+int launch_r1(const SweepArgs& a, const float* lchol, float* T, float* W, int D, cudaStream_t st) {
   constexpr int KP = 32 * NPL, LD = KP + 4;
-  linv_columns<<<KP, 32, 0, st>>>(lchol, a.K, KP, T);
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(linv_columns<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       linv_smem(a.K)));
+  linv_columns<NPL><<<KP, 32, linv_smem(a.K), st>>>(lchol, a.K, T);
   BPMF_CUDA_CHECK(cudaGetLastError());
   const size_t tbytes = sizeof(float) * KP * LD;
+  unsigned grid = 1;
+  if (W != nullptr) {
+    const size_t smem = tbytes + sizeof(float) * kR1MaxWarps * 4 * KP;
+    BPMF_TRY(r1_grid(lower_rows<NPL>, 32 * kR1MaxWarps, smem,
+                     (a.n_other + 4 * kR1MaxWarps) / (4 * kR1MaxWarps), &grid));
+    lower_rows<NPL><<<grid, 32 * kR1MaxWarps, smem, st>>>(a.Vo, a.n_other, a.K,
+                                                          a.lamaug + (int64_t)a.K * (a.K + 1), T, W);
+    BPMF_CUDA_CHECK(cudaGetLastError());
+  }
   const size_t per = sizeof(float) * (size_t)r1_warp_floats(D, KP);
   int w = kR1MaxWarps;
   while (w > 1 && tbytes + w * per > 200 * 1024) --w;
   const size_t smem = tbytes + w * per;
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_rank1<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-  int dev = 0, sms = 1, occ = 1;
-  BPMF_CUDA_CHECK(cudaGetDevice(&dev));
-  BPMF_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  BPMF_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, row_rank1<NPL>, 32 * w, smem));
-  const int64_t n = a.row_end - a.row_begin;
-  const int64_t grid = std::min<int64_t>((n + w - 1) / w, (int64_t)sms * std::max(occ, 1));
-  row_rank1<NPL><<<(unsigned)grid, 32 * w, smem, st>>>(a, lchol, T, D, w);
+  const int64_t n = a.row_end - a.row_begin, per_cta = (int64_t)w * kR1Rows;
+  auto kern = W != nullptr ? row_rank1<NPL, true> : row_rank1<NPL, false>;
+  BPMF_TRY(r1_grid(kern, 32 * w, smem, (n + per_cta - 1) / per_cta, &grid));
+  kern<<<grid, 32 * w, smem, st>>>(a, lchol, T, W, D, w);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
 }
 
 }  // namespace
 
-int launch_rows_rank1(const SweepArgs& a, const float* lchol, float* linvT, int max_degree,
-                      cudaStream_t st, int64_t* launches) {
+int64_t rank1_pre_floats(int K, int64_t n_other, int64_t rows, int64_t ratings) {
+  // one product of L_s^-1 per row of the other side against one per row and
+  // rating of the bin, the former in batches of four.  100,000 rows, K = 64, the
+  // products formed once against row by row: two ratings a row, 6, 3, 2 and 1
+  // times as many rows and ratings as rows on the other side: 343 / 417,
+  // 367 / 423, 382 / 426, 439 / 440 us; six ratings a row, 3.5 and 2 times:
+  // 936 / 956, 1014 / 975 us (K = 100: ahead from 1 times on; K = 16: even at 3).
+  if (ratings == 0 || rows + ratings < 3 * n_other) return 0;
+  return (n_other + 1) * ((K + 31) & ~31);
+}
+
+int launch_rows_rank1(const SweepArgs& a, const float* lchol, float* linvT, float* pre,
+                      int max_degree, cudaStream_t st, int64_t* launches) {
   if (a.row_end <= a.row_begin) return BPMF_OK;
   if (max_degree < 0 || max_degree > kTinyDegreeMax) return BPMF_EINVAL;
-  *launches += 2;
-  if (a.K <= 32) return launch_r1<1>(a, lchol, linvT, max_degree, st);
-  if (a.K <= 64) return launch_r1<2>(a, lchol, linvT, max_degree, st);
-  if (a.K <= 96) return launch_r1<3>(a, lchol, linvT, max_degree, st);
-  return launch_r1<4>(a, lchol, linvT, max_degree, st);
+  *launches += pre != nullptr ? 3 : 2;
+  if (a.K <= 32) return launch_r1<1>(a, lchol, linvT, pre, max_degree, st);
+  if (a.K <= 64) return launch_r1<2>(a, lchol, linvT, pre, max_degree, st);
+  if (a.K <= 96) return launch_r1<3>(a, lchol, linvT, pre, max_degree, st);
+  return launch_r1<4>(a, lchol, linvT, pre, max_degree, st);
 }
 
 }  // namespace gb

@@ -72,10 +72,14 @@ bool ws_cross_once(int64_t nnz, int64_t R);
 // rows row_begin..row_end, one warp per row, FP32 (rows_warp.cu); 1 <= K <= 32
 bool warp_supported(int K);
 int launch_rows_warp(const SweepArgs& a, cudaStream_t st, int64_t* launches);
-// rows row_begin..row_end by rank-one updates of chol(Lambda_s) (rank1.cu)
-// rows of degree <= max_degree (<= kTinyDegreeMax) from chol(Lambda_s); linvT is
-// scratch of KP x (KP + 4) floats that the call fills with (L_s^-1)^T first
-int launch_rows_rank1(const SweepArgs& a, const float* lchol, float* linvT, int max_degree,
-                      cudaStream_t st, int64_t* launches);
+// rows row_begin..row_end of degree <= max_degree (<= kTinyDegreeMax) from
+// chol(Lambda_s) (rank1.cu); linvT is scratch of KP x (KP + 4) floats that the
+// call fills with (L_s^-1)^T first, pre scratch of rank1_pre_floats floats for
+// L_s^-1 of the other side's rows (nullptr: formed row by row)
+int launch_rows_rank1(const SweepArgs& a, const float* lchol, float* linvT, float* pre,
+                      int max_degree, cudaStream_t st, int64_t* launches);
+// floats of that scratch for a bin of `rows` rows with `ratings` ratings in all;
+// 0 where L_s^-1 is better applied row by row
+int64_t rank1_pre_floats(int K, int64_t n_other, int64_t rows, int64_t ratings);
 
 }  // namespace gb

@@ -212,7 +212,7 @@ __device__ __forceinline__ int tc_gram(const SweepArgs& a, const TcSmem& s, uint
       for (int q = 0; q < 8; ++q) xc[i][q] = xn[i][q];
     fence_proxy_async_smem();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32 && elect_one()) {
       tc_fence_after();
       const uint32_t hi = base + b * kTcStageBytes, lo = hi + kTcTile;
       const int ksteps = (cnt + 15) >> 4;

@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "bpmf_impl.cuh"
+#include "rows.cuh"
 
 namespace gb {
 namespace {
@@ -79,6 +80,8 @@ int64_t job_bytes(const Job& j, int num_sms) {
   b += j.n_test * (4 + 4 + 4 + 8);                  // test set and running sums
   b += (j.nnz / 2048 + 16) * (K + 8) * (K + 8) * 4; // split-row partial Grams
   b += j.nnz * 32 + (j.M + j.N) * 16;               // sort and copy buffers of bpmf_init
+  for (const int64_t n : {j.M, j.N})                // L^-1 of the other side's rows (tiny rows)
+    b += rank1_pre_floats((int)K, n, j.M + j.N - n, j.nnz) * 4;
   return b + (8LL << 20);
 }
 
