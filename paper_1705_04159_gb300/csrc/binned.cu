@@ -13,7 +13,7 @@
 //   heavy (light_max < degree < hub_min): one CTA per row, tensor-core Gram
 //         on the MIXED path, FP32 Gram otherwise;
 //   light (tiny_max < degree <= light_max): FP32 Gram; one warp per row for
-//         K <= 32 (rows_warp.cu), else one CTA per row;
+//         K <= 55 (rows_small.cu), else one CTA per row;
 //   tiny  (degree <= tiny_max, degree 0 included): one warp per row, rank-one
 //         updates of chol(Lambda_s) (rank1.cu).
 // The thresholds are fixed by the configuration, or by defaults, or -- with
@@ -64,7 +64,7 @@ int launch_sweep_binned(Handle* h, int s, const SweepArgs& a0) {
       SweepArgs f = a;
       f.row_begin = 0;
       f.row_end = sd.n_hub;
-      rc = launch_hub_finish_fp32(f, hs, &h->kernels);
+      rc = launch_hub_draw(f, hs, &h->kernels);
     }
   }
   if (fork) {
@@ -104,15 +104,7 @@ int launch_other_bins(Handle* h, int s, const SweepArgs& a, cudaStream_t st) {
       BPMF_TRY(launch_rows_fp32(r, st, &h->kernels));
     r.row_begin = e_heavy;
     r.row_end = e_light;
-    if (warp_supported(h->K)) BPMF_TRY(launch_rows_warp(r, st, &h->kernels));
-    else BPMF_TRY(launch_rows_fp32(r, st, &h->kernels));
-  } else if (warp_supported(h->K)) {
-    r.row_begin = e_hub;
-    r.row_end = e_heavy;
     BPMF_TRY(launch_rows_fp32(r, st, &h->kernels));
-    r.row_begin = e_heavy;
-    r.row_end = e_light;
-    BPMF_TRY(launch_rows_warp(r, st, &h->kernels));
   } else {
     r.row_begin = e_hub;
     r.row_end = e_light;
@@ -441,8 +433,7 @@ int autotune_bins(Handle* h, int s, float* scratch) {
     BPMF_TRY(apply_bins(h, s, sd.tiny_max, sd.light_max, best_v));
   }
   const bool light_differs =
-      (h->cfg.path == BPMF_PATH_MIXED && (tc_supported(h->K) || (ws_supported(h->K) && sd.Xhi))) ||
-      (h->cfg.path == BPMF_PATH_BINNED && warp_supported(h->K));
+      h->cfg.path == BPMF_PATH_MIXED && (tc_supported(h->K) || (ws_supported(h->K) && sd.Xhi));
   if (h->cfg.light_max < 0 && light_differs) {
     int64_t best_v = sd.light_max;
     float best = 3.0e38f;

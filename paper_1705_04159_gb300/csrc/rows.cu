@@ -17,8 +17,9 @@
 // symmetric Gram of the (K+1)-vectors x_j = [v_j, r_ij] gives both
 // sum v_j v_j^T and sum r_ij v_j (its last row).  Rows are staged 32 at a
 // time in shared memory with cp.async, double-buffered, and accumulated in
-// FP32 register tiles (tile_chol.cuh); the same tiles then hold the bordered
-// matrix through the Cholesky.
+// FP32 register tiles, a thread per tile (tile_chol.cuh numbers them); the
+// bordered matrix is then factored from shared memory by one warp
+// (warp_chol.cuh).  Latent dimensions up to 55 take rows_small.cu instead.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +27,7 @@
 #include "bpmf_impl.cuh"
 #include "rows.cuh"
 #include "tile_chol.cuh"
+#include "warp_chol.cuh"
 
 namespace gb {
 namespace {
@@ -44,33 +46,48 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-// Stages neighbour rows [e0, e0 + cnt) as (K+1)-vectors [v_j, r] at stride KPs.
+// Stages neighbour rows [e0, e0 + cnt) as (K+1)-vectors [v_j, r] at stride KPs;
+// thread t copies pieces t, t + nt, .. of the rows, stepped without divisions.
 __device__ __forceinline__ void stage_rows(const SweepArgs& a, int KPs, float* dst, int64_t e0,
                                            int cnt) {
-  const int K = a.K, nt = blockDim.x;
-  if ((K & 3) == 0) {
-    const int Q = K >> 2;
-    for (int e = threadIdx.x; e < cnt * Q; e += nt) {
-      const int rr = e / Q, q = e - rr * Q;
-      const int64_t j = a.idx[e0 + rr];
-      cp_async16(dst + rr * KPs + 4 * q, a.Vo + j * K + 4 * q);
-    }
-  } else {
-    for (int e = threadIdx.x; e < cnt * K; e += nt) {
-      const int rr = e / K, k = e - rr * K;
-      const int64_t j = a.idx[e0 + rr];
-      cp_async4(dst + rr * KPs + k, a.Vo + j * K + k);
+  const int K = a.K, nt = blockDim.x, t = threadIdx.x;
+  const bool vec = (K & 3) == 0;
+  const int P = vec ? K >> 2 : K;
+  const int dr = nt / P, dq = nt - dr * P;
+  int rr = t / P, q = t - rr * P;
+  while (rr < cnt) {
+    const int64_t j = a.idx[e0 + rr];
+    if (vec) cp_async16(dst + rr * KPs + 4 * q, a.Vo + j * K + 4 * q);
+    else cp_async4(dst + rr * KPs + q, a.Vo + j * K + q);
+    rr += dr;
+    q += dq;
+    if (q >= P) {
+      q -= P;
+      ++rr;
     }
   }
-  for (int rr = threadIdx.x; rr < cnt; rr += nt) cp_async4(dst + rr * KPs + K, a.val + e0 + rr);
+  for (int r2 = t; r2 < cnt; r2 += nt) cp_async4(dst + r2 * KPs + K, a.val + e0 + r2);
   cp_async_commit();
 }
 
+// Two FP32 fused multiply-adds in one instruction (d0 += a b0, d1 += a b1),
+// each rounded as fmaf rounds it.
+__device__ __forceinline__ void ffma2(float& d0, float& d1, float a, float b0, float b1) {
+  asm("{\n\t.reg .b64 ra, rb, rc;\n\t"
+      "mov.b64 ra, {%2, %2};\n\t"
+      "mov.b64 rb, {%3, %4};\n\t"
+      "mov.b64 rc, {%0, %1};\n\t"
+      "fma.rn.f32x2 rc, ra, rb, rc;\n\t"
+      "mov.b64 {%0, %1}, rc;\n\t}"
+      : "+f"(d0), "+f"(d1)
+      : "f"(a), "f"(b0), "f"(b1));
+}
+
 // acc += sum over ratings [e0, e1) of x_j x_j^T (lower tiles, FP32).
-template <int TM>
 __device__ __forceinline__ void gram_gather(const SweepArgs& a, const TileGeom& G, float* Vs,
                                             int64_t e0, int64_t e1, bool active, int ty, int tx,
-                                            float (&acc)[TM][TM]) {
+                                            float (&acc)[8][8]) {
+  constexpr int TM = 8;
   const int KPs = G.KPs;
   const int buf_floats = kChunk * KPs;
   // padding columns K+1 .. KPs-1 stay zero (cp.async writes columns 0..K only)
@@ -96,94 +113,81 @@ __device__ __forceinline__ void gram_gather(const SweepArgs& a, const TileGeom& 
     if (active) {
       for (int rr = 0; rr < cnt; ++rr) {
         float va[TM], vb[TM];
-        lds_vec<TM>(B + rr * KPs + ty * TM, va);
-        lds_vec<TM>(B + rr * KPs + tx * TM, vb);
+        ld8(B + rr * KPs + ty * TM, va);
+        ld8(B + rr * KPs + tx * TM, vb);
 #pragma unroll
         for (int p = 0; p < TM; ++p)
 #pragma unroll
-          for (int q = 0; q < TM; ++q) acc[p][q] = fmaf(va[p], vb[q], acc[p][q]);
+          for (int q = 0; q < TM; q += 2) ffma2(acc[p][q], acc[p][q + 1], va[p], vb[q], vb[q + 1]);
       }
     }
     __syncthreads();
   }
 }
 
-// staging buffers and L share the front of shared memory; the rest follows
-__device__ __forceinline__ CholSmem carve(float* smem, const TileGeom& G) {
-  return carve_chol(smem, smem + G.union_floats(2 * kChunk * G.KPs), G);
-}
-
+// the tiles reuse the staging buffers; thresholds, 1 / diagonal and z follow
 int smem_bytes_fp32(const TileGeom& G) {
-  return (int)sizeof(float) * (G.union_floats(2 * kChunk * G.KPs) + G.tail_floats());
+  return (int)sizeof(float) * (std::max(2 * kChunk * G.KPs, G.ntiles * kTileF) + 3 * G.KP);
 }
 
 }  // namespace
 
-// Whole rows (mode 0) or hub rows from their partial Grams (mode 1).
-template <int TM>
-__global__ void __launch_bounds__(160) row_fp32(const SweepArgs a, int mode) {
+// A row of latent dimension past rows_small.cu's by one CTA: the Gram in
+// register tiles, then the tiles go to shared memory and one warp factors them
+// and draws.
+__global__ void __launch_bounds__(160) row_fp32(const SweepArgs a) {
   extern __shared__ __align__(16) float smem[];
-  __shared__ int fail_sh;
-  const TileGeom G(a.K, TM);
+  const TileGeom G(a.K, 8);
   const int64_t slot = a.row_begin + blockIdx.x;
   if (slot >= a.row_end) return;
   const int row = a.rows ? a.rows[slot] : (int)slot;
-  const CholSmem s = carve(smem, G);
   const int tid = threadIdx.x;
   const bool active = tid < G.ntiles;
   int ty = 0, tx = 0;
   if (active) tri_tile(tid, G.g, ty, tx);
-  if (tid == 0) fail_sh = 0;
-  row_normals(s.zv, a.K, row, *a.tp, a.sw, a.key);
-
-  float acc[TM][TM];
+  float acc[8][8];
 #pragma unroll
-  for (int p = 0; p < TM; ++p)
+  for (int p = 0; p < 8; ++p)
 #pragma unroll
-    for (int q = 0; q < TM; ++q) acc[p][q] = 0.f;
-
-  if (mode == 0) {
-    gram_gather<TM>(a, G, smem, a.ptr[row], a.ptr[row + 1], active, ty, tx, acc);
-  } else if (active) {
-    const int32_t pb = a.hub_piece0[slot], pe = a.hub_piece0[slot + 1];
-    for (int32_t pc = pb; pc < pe; ++pc) {
-      const float* src = a.part + ((int64_t)pc * G.ntiles + tid) * (TM * TM);
+    for (int q = 0; q < 8; ++q) acc[p][q] = 0.f;
+  gram_gather(a, G, smem, a.ptr[row], a.ptr[row + 1], active, ty, tx, acc);
+  __syncthreads();  // a row without ratings has met no barrier since it zeroed the padding
+  float* T = smem;
+  float* thr = smem + max(2 * kChunk * G.KPs, G.ntiles * kTileF);
+  if (active) {
 #pragma unroll
-      for (int p = 0; p < TM; ++p)
+    for (int p = 0; p < 8; ++p) {
+      float x[8];
 #pragma unroll
-        for (int q = 0; q < TM; ++q) acc[p][q] += __ldcs(src + p * TM + q);
+      for (int q = 0; q < 8; ++q) x[q] = row_elem(a, 8 * ty + p, 8 * tx + q, acc[p][q]);
+      st8(T + tidx(ty, tx) * kTileF + trow(p), x);
+      if (ty == tx)
+        thr[8 * ty + p] = 8 * ty + p < a.K ? pivot_threshold(a.pivot_rel, x[p]) : -INFINITY;
     }
   }
-  form_bordered<TM>(acc, active, ty, tx, G, a.lamaug, a.alpha, s.diag0);
   __syncthreads();
-  if (!chol_solve_write<TM>(acc, active, ty, tx, G, s, a.pivot_rel, &fail_sh,
-                           a.X + (int64_t)row * a.K)) {
-    if (tid == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
-  }
+  if (tid < 32) row_draw(a, G.g, T, thr, thr + G.KP, thr + 2 * G.KP, row, tid);
 }
 
 // Partial Gram of one piece of a split row, stored as raw tiles.
-template <int TM>
 __global__ void __launch_bounds__(160) piece_fp32(const SweepArgs a) {
   extern __shared__ __align__(16) float smem[];
-  const TileGeom G(a.K, TM);
+  const TileGeom G(a.K, 8);
   const int64_t pc = blockIdx.x;
   const int tid = threadIdx.x;
   const bool active = tid < G.ntiles;
   int ty = 0, tx = 0;
   if (active) tri_tile(tid, G.g, ty, tx);
-  float acc[TM][TM];
+  float acc[8][8];
 #pragma unroll
-  for (int p = 0; p < TM; ++p)
+  for (int p = 0; p < 8; ++p)
 #pragma unroll
-    for (int q = 0; q < TM; ++q) acc[p][q] = 0.f;
-  gram_gather<TM>(a, G, smem, a.piece_e0[pc], a.piece_e1[pc], active, ty, tx, acc);
+    for (int q = 0; q < 8; ++q) acc[p][q] = 0.f;
+  gram_gather(a, G, smem, a.piece_e0[pc], a.piece_e1[pc], active, ty, tx, acc);
   if (active) {
-    float* dst = a.part + (pc * G.ntiles + tid) * (TM * TM);
+    float* dst = a.part + (pc * G.ntiles + tid) * 64;
 #pragma unroll
-    for (int p = 0; p < TM; ++p)
-#pragma unroll
-      for (int q = 0; q < TM; ++q) dst[p * TM + q] = acc[p][q];
+    for (int p = 0; p < 8; ++p) st8(dst + 8 * p, acc[p]);
   }
 }
 
@@ -279,66 +283,36 @@ int set_smem_attr(const void* fn, int bytes) {
   return BPMF_OK;
 }
 
-template <int TM>
-int rows_fp32_tm(const SweepArgs& a, int mode, cudaStream_t st, int64_t* launches) {
+}  // namespace
+
+int launch_rows_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
+  if (small_supported(a.K)) return launch_rows_small(a, st, launches);
   const int64_t nrows = a.row_end - a.row_begin;
   if (nrows <= 0) return BPMF_OK;
-  const TileGeom G(a.K, TM);
+  const TileGeom G(a.K, 8);
   const int smem = smem_bytes_fp32(G);
-  BPMF_TRY(set_smem_attr((const void*)row_fp32<TM>, smem));
+  BPMF_TRY(set_smem_attr((const void*)row_fp32, smem));
   for (int64_t off = 0; off < nrows; off += 1LL << 30) {
     SweepArgs b = a;
     b.row_begin = a.row_begin + off;
     b.row_end = b.row_begin + std::min<int64_t>(nrows - off, 1LL << 30);
-    row_fp32<TM><<<(unsigned)(b.row_end - b.row_begin), G.nthreads, smem, st>>>(b, mode);
+    row_fp32<<<(unsigned)(b.row_end - b.row_begin), G.nthreads, smem, st>>>(b);
     BPMF_CUDA_CHECK(cudaGetLastError());
     if (launches) *launches += 1;
   }
   return BPMF_OK;
 }
 
-template <int TM>
-int pieces_fp32_tm(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
+int launch_pieces_fp32(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
+  if (small_supported(a.K)) return launch_pieces_small(a, npieces, st, launches);
   if (npieces <= 0) return BPMF_OK;
-  const TileGeom G(a.K, TM);
+  const TileGeom G(a.K, 8);
   const int smem = (int)sizeof(float) * 2 * kChunk * G.KPs;
-  BPMF_TRY(set_smem_attr((const void*)piece_fp32<TM>, smem));
-  piece_fp32<TM><<<(unsigned)npieces, G.nthreads, smem, st>>>(a);
+  BPMF_TRY(set_smem_attr((const void*)piece_fp32, smem));
+  piece_fp32<<<(unsigned)npieces, G.nthreads, smem, st>>>(a);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;
   return BPMF_OK;
-}
-
-}  // namespace
-
-int64_t partial_floats_per_piece(int K) {
-  const int TM = tile_edge_for(K);
-  const TileGeom G(K, TM);
-  return (int64_t)G.ntiles * TM * TM;
-}
-
-int launch_rows_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
-  switch (tile_edge_for(a.K)) {
-    case 2: return rows_fp32_tm<2>(a, 0, st, launches);
-    case 4: return rows_fp32_tm<4>(a, 0, st, launches);
-    default: return rows_fp32_tm<8>(a, 0, st, launches);
-  }
-}
-
-int launch_hub_finish_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
-  switch (tile_edge_for(a.K)) {
-    case 2: return rows_fp32_tm<2>(a, 1, st, launches);
-    case 4: return rows_fp32_tm<4>(a, 1, st, launches);
-    default: return rows_fp32_tm<8>(a, 1, st, launches);
-  }
-}
-
-int launch_pieces_fp32(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
-  switch (tile_edge_for(a.K)) {
-    case 2: return pieces_fp32_tm<2>(a, npieces, st, launches);
-    case 4: return pieces_fp32_tm<4>(a, npieces, st, launches);
-    default: return pieces_fp32_tm<8>(a, npieces, st, launches);
-  }
 }
 
 SweepArgs make_sweep_args(Handle* h, int s) {

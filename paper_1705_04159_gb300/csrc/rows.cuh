@@ -35,7 +35,7 @@ struct SweepArgs {
   const int64_t* piece_e0;
   const int64_t* piece_e1;
   const int32_t* hub_piece0;
-  float* part;          // partial Gram tiles [piece][tile][TM * TM]
+  float* part;          // partial Gram tiles [piece][tile][8 * 8]
   // bf16 hi/lo shadow of the other side's factors, rows padded to KS (mixed path)
   const __nv_bfloat16* Vhi;
   const __nv_bfloat16* Vlo;
@@ -50,8 +50,8 @@ SweepArgs make_sweep_args(Handle* h, int s);
 int launch_rows_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches);
 // partial Grams of pieces [0, npieces)
 int launch_pieces_fp32(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches);
-// hub rows row_begin..row_end (degree order) from their partial Grams
-int launch_hub_finish_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches);
+// hub rows row_begin..row_end (degree order) from their partial Grams (rows_small.cu)
+int launch_hub_draw(const SweepArgs& a, cudaStream_t st, int64_t* launches);
 int64_t partial_floats_per_piece(int K);
 // tensor-core Gram (rows_tc.cu); supported for 48 <= K <= 119
 bool tc_supported(int K);
@@ -69,9 +69,11 @@ int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross
 int ws_stage_neighbours(int64_t nnz, int64_t R);
 // whether that side's 64-neighbour stages form the cross term from one product
 bool ws_cross_once(int64_t nnz, int64_t R);
-// rows row_begin..row_end, one warp per row, FP32 (rows_warp.cu); 1 <= K <= 32
-bool warp_supported(int K);
-int launch_rows_warp(const SweepArgs& a, cudaStream_t st, int64_t* launches);
+// whole rows by one warp each and pieces of split rows, FP32; 1 <= K <= 55
+// (rows_small.cu; launch_rows_fp32 and launch_pieces_fp32 take them where they can)
+bool small_supported(int K);
+int launch_rows_small(const SweepArgs& a, cudaStream_t st, int64_t* launches);
+int launch_pieces_small(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches);
 // rows row_begin..row_end of degree <= max_degree (<= kTinyDegreeMax) from
 // chol(Lambda_s) (rank1.cu); linvT is scratch of KP x (KP + 4) floats that the
 // call fills with (L_s^-1)^T first, pre scratch of rank1_pre_floats floats for
