@@ -9,7 +9,7 @@
 // and one warp holds the whole Gram of the rating-augmented neighbours
 // x_j = [v_j, r_ij] in registers, so no block-wide barrier is needed (the
 // light-row kernel of the degree bins, paper Sec. III):
-//   Gram: neighbours are staged 16 at a time in the warp's shared memory with
+//   Gram: neighbours are staged 16 or 32 at a time in the warp's shared memory with
 //     cp.async (double-buffered) and multiplied eight at a time on the tensor
 //     cores, mma.m16n8k8 over pairs of row tiles; FP32 operands are split into
 //     two TF32 parts, x = h + l, and l h + h l + h h of one step of eight is
@@ -23,11 +23,18 @@
 // The base matrix (Lambda_s bordered by Lambda_s mu_s) is shared by the CTA's
 // warps.  Pieces of split rows (hubs) take the same Gram and store it; one CTA
 // per hub adds its pieces in order and draws.
-// What bounds it: instruction issue.  A sweep of
-// 30,000 rows with 3M ratings, K = 50, took 1,450 us with one CTA per row and
-// FP32 multiply-adds, and takes 729; an iteration of 138,493 x 26,744 with 20M
-// ratings, K = 32, 3,560 us with one warp per row and FP32 multiply-adds (hub
-// pieces: a CTA each), and takes 2,816.
+// Where K is a multiple of eight the rating would make a tile row of its own;
+// the Gram then covers the features alone, and sum_j r_ij v_j is formed by
+// FP32 multiply-adds from the fragments at hand (K = 32: 18 tensor products a
+// step instead of 33).
+// What bounds it: issue and latency, more in the factorisation than in the Gram
+// at 100 ratings a row (K = 50: 10.8k warp instructions a row, issue slots 49%
+// busy, tensor pipe 28%; K = 32: 5.6k, 63%, 22%).  A sweep of 30,000 rows with
+// 3M ratings, K = 50, took 1,450 us with one CTA per row and FP32
+// multiply-adds, and takes 732; K = 32, 546 -> 331 us.  An iteration of
+// 138,493 x 26,744 with 20M ratings, K = 32, took 3,560 us with one warp per
+// row and FP32 multiply-adds (hub pieces: a CTA each), 2,816 with the rating as
+// a tile row, and takes 2,208; stages of 16 neighbours instead of 32: 2,321.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -41,33 +48,38 @@
 namespace gb {
 namespace {
 
-constexpr int kSmChunk = 16;  // neighbours staged per step
 constexpr int kSmWarps = 4;   // warps (rows) per CTA
 // CTAs per SM the registers are cut for: 128 a thread, 168 where the Gram takes up to 76
 constexpr int sm_ctas(int g) { return g <= 5 ? 4 : 3; }
 constexpr int kSmMaxG = 7;    // K <= 55
 
-template <int g>
+// g tile rows, the last of them row K alone if B (K = 8 (g - 1)): the Gram's
+// tiles then cover the K features, and sum_j r_ij v_j is kept aside.
+template <int g, bool B>
 struct SmGeom {
   static constexpr int KP = 8 * g;
-  static constexpr int LDT = g & 1 ? KP : KP + 8;  // staged row stride: an odd multiple of 8
-  static constexpr int NP = (g + 1) / 2;           // pairs of row tiles
-  static constexpr int NT = g * (g + 1) / 2;       // tiles
-  // accumulators: pair k covers tile columns 0 .. min(2 k + 1, g - 1), from k (k + 1)
-  static constexpr int NA = g & 1 ? (NP - 1) * NP + 2 * NP - 1 : NP * (NP + 1);
-  __host__ __device__ static constexpr int cols(int k) { return 2 * k + 2 < g ? 2 * k + 2 : g; }
-  static constexpr int kStage = 2 * kSmChunk * LDT;
+  static constexpr int G = B ? g - 1 : g;             // tile rows of the Gram
+  static constexpr int LDT = G & 1 ? 8 * G : 8 * G + 8;  // staged row stride: an odd multiple of 8
+  static constexpr int NP = (G + 1) / 2;              // pairs of row tiles
+  static constexpr int NT = g * (g + 1) / 2;          // tiles
+  // accumulators: pair k covers tile columns 0 .. min(2 k + 1, G - 1), from k (k + 1)
+  static constexpr int NA = G & 1 ? (NP - 1) * NP + 2 * NP - 1 : NP * (NP + 1);
+  __host__ __device__ static constexpr int cols(int k) { return 2 * k + 2 < G ? 2 * k + 2 : G; }
+  // neighbours staged at a time; 32 of seven tile rows would leave the L1 32 KB
+  // (K = 50: 744 us instead of 732, K = 32: 331 instead of 340)
+  static constexpr int kChunk = G < 7 ? 32 : 16;
+  static constexpr int kRows = 2 * kChunk * LDT;    // staged rows, then ratings if B
+  static constexpr int kStage = kRows + (B ? 2 * kChunk : 0);
   // per warp: staging buffers, reused by the tiles; thresholds, 1 / diagonal, z
   static constexpr int kFloats = (kStage > NT * kTileF ? kStage : NT * kTileF) + 3 * KP;
 };
 
-// 16-, 8- and 4-byte copies, zero-filling when not live
-__device__ __forceinline__ void cp_async_z(float* dst, const float* src, int bytes, bool live) {
+template <int V>
+__device__ __forceinline__ void cp_async(float* dst, const float* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  const int n = live ? bytes : 0;
-  if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-  else if (bytes == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+  if constexpr (V == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+  else if constexpr (V == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -76,26 +88,33 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // Stages neighbours whose ids and ratings lanes 0 .. cnt - 1 hold, V floats per
-// copy; the rows up to the next multiple of eight are zeroed.
-template <int g, int V>
-__device__ __forceinline__ void sm_stage(const float* __restrict__ Vo, int K, float* T, int j, float r,
-                                         int cnt, int lane) {
-  constexpr int LDT = SmGeom<g>::LDT;
-  const int P = K / V, n = ((cnt + 7) & ~7) * P;
-  // lane l copies pieces l, l + 32, ..: row rr, piece q, stepped without divisions
-  int rr = lane / P, q = lane - rr * P;
-  const int dr = 32 / P, dq = 32 - dr * P;
-  for (int e0 = 0; e0 < n; e0 += 32) {
-    const int jr = __shfl_sync(0xffffffffu, j, rr & 31);
-    if (e0 + lane < n) cp_async_z(T + rr * LDT + V * q, Vo + (int64_t)jr * K + V * q, 4 * V, rr < cnt);
-    rr += dr;
-    q += dq;
-    if (q >= P) {
-      q -= P;
-      ++rr;
+// copy, 8, 16 or 32 lanes (V = 4, 2, 1) a row and at most two copies each; the
+// ratings go Rs floats apart to R; the rows up to the next multiple of eight
+// are zeroed.
+template <int LDT, int V>
+__device__ __forceinline__ void sm_stage(const float* __restrict__ Vo, int K, float* T, float* R, int Rs,
+                                         int j, float r, int cnt, int lane) {
+  constexpr int kLanes = 32 / V, kStep = V;  // lanes a row, rows a step
+  const int q = V * (lane % kLanes);
+  int rr = lane / kLanes;
+  float* dst = T + rr * LDT + q;
+#pragma unroll 4
+  for (int k = 0; k < cnt; k += kStep) {
+    const int jr = __shfl_sync(0xffffffffu, j, rr);
+    const float* src = Vo + (int64_t)jr * K + q;
+    if (rr < cnt) {
+      if (q < K) cp_async<V>(dst, src);
+      if (q + 32 < K) cp_async<V>(dst + 32, src + 32);
     }
+    rr += kStep;
+    dst += kStep * LDT;
   }
-  if (lane < ((cnt + 7) & ~7)) T[lane * LDT + K] = lane < cnt ? r : 0.f;
+  const int pad = -cnt & 7;
+  if (pad) {
+    for (int k = 0; k < pad; ++k)
+      for (int c = lane; c < K; c += 32) T[(cnt + k) * LDT + c] = 0.f;
+  }
+  if (lane < cnt + pad) R[lane * Rs] = lane < cnt ? r : 0.f;
   cp_async_commit();
 }
 
@@ -108,21 +127,30 @@ __device__ __forceinline__ void mma_tf32_zero(float (&d)[4], uint32_t a0, uint32
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// o += sum over eight staged neighbours of x x^T (lower tiles, in pairs)
-template <int g>
-__device__ __forceinline__ void sm_step(const float* X, float (&o)[SmGeom<g>::NA][4]) {
-  using S = SmGeom<g>;
-  uint32_t h0[g], h1[g], l0[g], l1[g];
+// o += sum over eight staged neighbours of x x^T (lower tiles, in pairs); if
+// B, s += their r x (R: their ratings; a lane's own two neighbours only)
+template <int g, bool B>
+__device__ __forceinline__ void sm_step(const float* X, const float* R, float (&o)[SmGeom<g, B>::NA][4],
+                                        float (&s)[SmGeom<g, B>::G]) {
+  using S = SmGeom<g, B>;
+  uint32_t h0[S::G], h1[S::G], l0[S::G], l1[S::G];
+  float r0 = 0.f, r1 = 0.f;
+  if (B) {
+    r0 = R[0];
+    r1 = R[4];
+  }
 #pragma unroll
-  for (int I = 0; I < g; ++I) {
-    split_tf32(X[8 * I], h0[I], l0[I]);
-    split_tf32(X[4 * S::LDT + 8 * I], h1[I], l1[I]);
+  for (int I = 0; I < S::G; ++I) {
+    const float x0 = X[8 * I], x1 = X[4 * S::LDT + 8 * I];
+    split_tf32(x0, h0[I], l0[I]);
+    split_tf32(x1, h1[I], l1[I]);
+    if (B) s[I] = fmaf(r1, x1, fmaf(r0, x0, s[I]));
   }
 #pragma unroll
   for (int k = 0; k < S::NP; ++k) {
-    const int u = 2 * k, v = 2 * k + 1 < g ? 2 * k + 1 : 2 * k;
+    const int u = 2 * k, v = 2 * k + 1 < S::G ? 2 * k + 1 : 2 * k;
 #pragma unroll
-    for (int J0 = 0; J0 < g; J0 += 4) {
+    for (int J0 = 0; J0 < S::G; J0 += 4) {
       float d[4][4];
 #pragma unroll
       for (int c = 0; c < 4; ++c)
@@ -144,70 +172,90 @@ __device__ __forceinline__ void sm_step(const float* X, float (&o)[SmGeom<g>::NA
   }
 }
 
-// o = sum over ratings [e0, e1) of x x^T
-template <int g, int V>
+// o (and s) = sums over ratings [e0, e1)
+template <int g, bool B, int V>
 __device__ __forceinline__ void sm_gram_v(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int lane,
-                                          float (&o)[SmGeom<g>::NA][4]) {
-  using S = SmGeom<g>;
-  constexpr int kBuf = kSmChunk * S::LDT;
+                                          float (&o)[SmGeom<g, B>::NA][4], float (&s)[SmGeom<g, B>::G]) {
+  using S = SmGeom<g, B>;
+  constexpr int kBuf = S::kChunk * S::LDT;
   const int K = a.K;
   const int64_t n = e1 - e0;
   const float* X = T + (lane & 3) * S::LDT + (lane >> 2);
+  const float* R = T + S::kRows + (lane & 3);
   // ids and ratings of the chunk after the one being staged, a lane each
   int j = 0;
   float r = 0.f;
   auto load = [&](int64_t c0) {
     j = 0;
     r = 0.f;
-    if (lane < kSmChunk && c0 + lane < n) {
+    if (lane < S::kChunk && c0 + lane < n) {
       j = __ldg(a.idx + e0 + c0 + lane);
       r = __ldg(a.val + e0 + c0 + lane);
     }
   };
-  auto count = [&](int64_t c0) { return (int)min((int64_t)kSmChunk, n - c0); };
+  auto count = [&](int64_t c0) { return (int)min((int64_t)S::kChunk, n - c0); };
+  auto stage = [&](int64_t c0, int buf) {
+    float* row = T + buf * kBuf;
+    sm_stage<S::LDT, V>(a.Vo, K, row, B ? T + S::kRows + buf * S::kChunk : row + K, B ? 1 : S::LDT, j, r,
+                        count(c0), lane);
+  };
   if (n <= 0) return;
   load(0);
-  sm_stage<g, V>(a.Vo, K, T, j, r, count(0), lane);
-  load(kSmChunk);
+  stage(0, 0);
+  load(S::kChunk);
   int buf = 0;
-  for (int64_t c0 = 0; c0 < n; c0 += kSmChunk, buf ^= 1) {
-    if (c0 + kSmChunk < n) {
-      sm_stage<g, V>(a.Vo, K, T + (buf ^ 1) * kBuf, j, r, count(c0 + kSmChunk), lane);
-      load(c0 + 2 * kSmChunk);
+  for (int64_t c0 = 0; c0 < n; c0 += S::kChunk, buf ^= 1) {
+    if (c0 + S::kChunk < n) {
+      stage(c0 + S::kChunk, buf ^ 1);
+      load(c0 + 2 * S::kChunk);
       cp_async_wait<1>();
     } else {
       cp_async_wait<0>();
     }
     __syncwarp();
-    sm_step<g>(X + buf * kBuf, o);
-    if (count(c0) > 8) sm_step<g>(X + buf * kBuf + 8 * S::LDT, o);
+    const float *Xb = X + buf * kBuf, *Rb = R + buf * S::kChunk;
+    const int cnt = count(c0);
+#pragma unroll 1
+    for (int k = 0; k < cnt; k += 8) sm_step<g, B>(Xb + k * S::LDT, Rb + k, o, s);
     __syncwarp();  // the buffer is refilled next
   }
 }
 
-template <int g>
+template <int g, bool B>
 __device__ __forceinline__ void sm_gram(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int lane,
-                                        float (&o)[SmGeom<g>::NA][4]) {
-  using S = SmGeom<g>;
+                                        float (&o)[SmGeom<g, B>::NA][4], float (&s)[SmGeom<g, B>::G]) {
+  using S = SmGeom<g, B>;
 #pragma unroll
   for (int i = 0; i < S::NA; ++i)
 #pragma unroll
     for (int q = 0; q < 4; ++q) o[i][q] = 0.f;
-  // the columns past the rating stay zero in both buffers
-  for (int e = lane; e < 2 * kSmChunk; e += 32) {
 #pragma unroll
-    for (int c = S::KP - 8; c < S::KP; ++c)
-      if (c > a.K) T[e * S::LDT + c] = 0.f;
+  for (int i = 0; i < S::G; ++i) s[i] = 0.f;
+  if constexpr (B) {
+    sm_gram_v<g, B, 4>(a, T, e0, e1, lane, o, s);
+    // over the four lanes that share a feature
+#pragma unroll
+    for (int i = 0; i < S::G; ++i) {
+      s[i] += __shfl_xor_sync(0xffffffffu, s[i], 1);
+      s[i] += __shfl_xor_sync(0xffffffffu, s[i], 2);
+    }
+  } else {
+    // the columns past the rating stay zero in both buffers
+    for (int e = lane; e < 2 * S::kChunk; e += 32) {
+#pragma unroll
+      for (int c = S::KP - 8; c < S::KP; ++c)
+        if (c > a.K) T[e * S::LDT + c] = 0.f;
+    }
+    __syncwarp();
+    if ((a.K & 3) == 0) sm_gram_v<g, B, 4>(a, T, e0, e1, lane, o, s);
+    else if ((a.K & 1) == 0) sm_gram_v<g, B, 2>(a, T, e0, e1, lane, o, s);
+    else sm_gram_v<g, B, 1>(a, T, e0, e1, lane, o, s);
   }
-  __syncwarp();
-  if ((a.K & 3) == 0) sm_gram_v<g, 4>(a, T, e0, e1, lane, o);
-  else if ((a.K & 1) == 0) sm_gram_v<g, 2>(a, T, e0, e1, lane, o);
-  else sm_gram_v<g, 1>(a, T, e0, e1, lane, o);
 }
 
-template <int g>
+template <int g, bool B>
 __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) row_small(const SweepArgs a) {
-  using S = SmGeom<g>;
+  using S = SmGeom<g, B>;
   extern __shared__ __align__(16) float ssm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* base = ssm;
@@ -224,18 +272,18 @@ __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) row_small(const Swe
   float* rinv = thr + S::KP;
   float* zv = rinv + S::KP;
   {
-    float o[S::NA][4];
-    sm_gram<g>(a, T, a.ptr[row], a.ptr[row + 1], lane, o);
+    float o[S::NA][4], s[S::G];
+    sm_gram<g, B>(a, T, a.ptr[row], a.ptr[row + 1], lane, o, s);
     // A = base + alpha G as tiles, over the staging buffers
     const int gr = lane >> 2, t2 = 2 * (lane & 3), fo = trow(gr) + t2;
 #pragma unroll
     for (int k = 0; k < S::NP; ++k)
 #pragma unroll
-      for (int J = 0; J < g; ++J)
+      for (int J = 0; J < S::G; ++J)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int I = 2 * k + h;
-          if (J <= I && I < g) {
+          if (J <= I && I < S::G) {
             const int off = tidx(I, J) * kTileF + fo;
             const float2 b = ldf2(base + off);
             const float x = fmaf(a.alpha, o[k * (k + 1) + J][2 * h], b.x);
@@ -245,6 +293,20 @@ __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) row_small(const Swe
               thr[8 * I + gr] = 8 * I + gr < a.K ? pivot_threshold(a.pivot_rel, gr & 1 ? y : x) : -INFINITY;
           }
         }
+    if (B) {  // row K, and the padding after it
+#pragma unroll
+      for (int J = 0; J < g; ++J) {
+        const int off = tidx(g - 1, J) * kTileF + fo;
+        float2 b = ldf2(base + off);
+        if (J < S::G) {
+          const float sx = __shfl_sync(0xffffffffu, s[J < S::G ? J : 0], 4 * t2);
+          const float sy = __shfl_sync(0xffffffffu, s[J < S::G ? J : 0], 4 * t2 + 4);
+          if (gr == 0) b = make_float2(fmaf(a.alpha, sx, b.x), fmaf(a.alpha, sy, b.y));
+        }
+        *reinterpret_cast<float2*>(T + off) = b;
+      }
+      if (lane < 8) thr[8 * (g - 1) + lane] = -INFINITY;
+    }
   }
   __syncwarp();
   row_draw(a, g, T, thr, rinv, zv, row, lane);
@@ -252,27 +314,31 @@ __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) row_small(const Swe
 
 // Partial Gram of one piece of a split row by one warp, stored as raw tiles in
 // the numbering of tile_chol.cuh.
-template <int g>
+template <int g, bool B>
 __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) piece_small(const SweepArgs a, int64_t npieces) {
-  using S = SmGeom<g>;
+  using S = SmGeom<g, B>;
   extern __shared__ __align__(16) float ssm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t pc = (int64_t)blockIdx.x * kSmWarps + warp;
   if (pc >= npieces) return;
-  float o[S::NA][4];
-  sm_gram<g>(a, ssm + warp * S::kStage, a.piece_e0[pc], a.piece_e1[pc], lane, o);
+  float o[S::NA][4], s[S::G];
+  sm_gram<g, B>(a, ssm + warp * S::kStage, a.piece_e0[pc], a.piece_e1[pc], lane, o, s);
   float* dst = a.part + pc * S::NT * 64 + 2 * lane;
 #pragma unroll
   for (int k = 0; k < S::NP; ++k)
 #pragma unroll
-    for (int J = 0; J < g; ++J)
+    for (int J = 0; J < S::G; ++J)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int I = 2 * k + h;
-        if (J <= I && I < g)
+        if (J <= I && I < S::G)
           *reinterpret_cast<float2*>(dst + tile_id(I, J, g) * 64) =
               make_float2(o[k * (k + 1) + J][2 * h], o[k * (k + 1) + J][2 * h + 1]);
       }
+  if (B && (lane & 3) == 0) {  // row K of the last tile row, all that the draw reads of it
+#pragma unroll
+    for (int J = 0; J < S::G; ++J) a.part[(pc * S::NT + tile_id(g - 1, J, g)) * 64 + (lane >> 2)] = s[J];
+  }
 }
 
 // Hub rows from their partial Grams, any K: a CTA adds the pieces of its hub
@@ -322,30 +388,30 @@ __global__ void __launch_bounds__(kHubThreads) hub_draw(const SweepArgs a) {
   if (threadIdx.x < 32) row_draw(a, g, T, thr, rinv, zv, a.rows ? a.rows[slot] : (int)slot, threadIdx.x);
 }
 
-template <int g>
+template <int g, bool B>
 int launch_small(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
-  using S = SmGeom<g>;
+  using S = SmGeom<g, B>;
   const int smem = (S::NT * kTileF + kSmWarps * S::kFloats) * (int)sizeof(float);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_small<g>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_small<g, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   const int64_t n = a.row_end - a.row_begin;
   for (int64_t off = 0; off < n; off += (int64_t)kSmWarps << 27) {
     SweepArgs b = a;
     b.row_begin = a.row_begin + off;
     b.row_end = b.row_begin + std::min<int64_t>(n - off, (int64_t)kSmWarps << 27);
     const int64_t blocks = (b.row_end - b.row_begin + kSmWarps - 1) / kSmWarps;
-    row_small<g><<<(unsigned)blocks, 32 * kSmWarps, smem, st>>>(b);
+    row_small<g, B><<<(unsigned)blocks, 32 * kSmWarps, smem, st>>>(b);
     BPMF_CUDA_CHECK(cudaGetLastError());
     if (launches) *launches += 1;
   }
   return BPMF_OK;
 }
 
-template <int g>
+template <int g, bool B>
 int launch_small_pieces(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
-  using S = SmGeom<g>;
+  using S = SmGeom<g, B>;
   const int smem = kSmWarps * S::kStage * (int)sizeof(float);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(piece_small<g>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  piece_small<g><<<(unsigned)((npieces + kSmWarps - 1) / kSmWarps), 32 * kSmWarps, smem, st>>>(a, npieces);
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(piece_small<g, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  piece_small<g, B><<<(unsigned)((npieces + kSmWarps - 1) / kSmWarps), 32 * kSmWarps, smem, st>>>(a, npieces);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;
   return BPMF_OK;
@@ -357,31 +423,35 @@ bool small_supported(int K) { return K >= 1 && (K + 8) / 8 <= kSmMaxG; }
 
 int launch_rows_small(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
   if (a.row_end <= a.row_begin) return BPMF_OK;
-  switch ((a.K + 8) / 8) {
-    case 1: return launch_small<1>(a, st, launches);
-    case 2: return launch_small<2>(a, st, launches);
-    case 3: return launch_small<3>(a, st, launches);
-    case 4: return launch_small<4>(a, st, launches);
-    case 5: return launch_small<5>(a, st, launches);
-    case 6: return launch_small<6>(a, st, launches);
-    case 7: return launch_small<7>(a, st, launches);
-    default: return BPMF_EINVAL;
+#define GB_SMALL(fn, ...)                                                                      \
+  if (a.K % 8 == 0) {                                                                          \
+    switch (a.K / 8) {                                                                         \
+      case 1: return fn<2, true>(__VA_ARGS__);                                                 \
+      case 2: return fn<3, true>(__VA_ARGS__);                                                 \
+      case 3: return fn<4, true>(__VA_ARGS__);                                                 \
+      case 4: return fn<5, true>(__VA_ARGS__);                                                 \
+      case 5: return fn<6, true>(__VA_ARGS__);                                                 \
+      case 6: return fn<7, true>(__VA_ARGS__);                                                 \
+    }                                                                                          \
+  }                                                                                            \
+  switch ((a.K + 8) / 8) {                                                                     \
+    case 1: return fn<1, false>(__VA_ARGS__);                                                  \
+    case 2: return fn<2, false>(__VA_ARGS__);                                                  \
+    case 3: return fn<3, false>(__VA_ARGS__);                                                  \
+    case 4: return fn<4, false>(__VA_ARGS__);                                                  \
+    case 5: return fn<5, false>(__VA_ARGS__);                                                  \
+    case 6: return fn<6, false>(__VA_ARGS__);                                                  \
+    case 7: return fn<7, false>(__VA_ARGS__);                                                  \
+    default: return BPMF_EINVAL;                                                               \
   }
+  GB_SMALL(launch_small, a, st, launches)
 }
 
 int launch_pieces_small(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
   if (npieces <= 0) return BPMF_OK;
-  switch ((a.K + 8) / 8) {
-    case 1: return launch_small_pieces<1>(a, npieces, st, launches);
-    case 2: return launch_small_pieces<2>(a, npieces, st, launches);
-    case 3: return launch_small_pieces<3>(a, npieces, st, launches);
-    case 4: return launch_small_pieces<4>(a, npieces, st, launches);
-    case 5: return launch_small_pieces<5>(a, npieces, st, launches);
-    case 6: return launch_small_pieces<6>(a, npieces, st, launches);
-    case 7: return launch_small_pieces<7>(a, npieces, st, launches);
-    default: return BPMF_EINVAL;
-  }
+  GB_SMALL(launch_small_pieces, a, npieces, st, launches)
 }
+#undef GB_SMALL
 
 int64_t partial_floats_per_piece(int K) {
   const int g = (K + 8) / 8;

@@ -309,11 +309,11 @@ __device__ __forceinline__ float row_base(const SweepArgs& a, int i, int j) {
   return j > i ? 0.f : i == K && j == K ? 1e30f : __ldg(a.lamaug + i * KA + j);
 }
 
-// Element (i, j) of base + alpha G from the Gram's; what the Gram holds outside
-// the bordered lower triangle is not looked at.
+// Element (i, j) of base + alpha G from the Gram's; what the Gram holds in the
+// corner (K, K) and outside the bordered lower triangle is not looked at.
 __device__ __forceinline__ float row_elem(const SweepArgs& a, int i, int j, float s) {
   const float b = row_base(a, i, j);
-  return i > a.K || j > i ? b : fmaf(a.alpha, s, b);
+  return i > a.K || j > i || j >= a.K ? b : fmaf(a.alpha, s, b);
 }
 
 // One warp factors the tiles and draws the row, or leaves it to the FP64 redo;
