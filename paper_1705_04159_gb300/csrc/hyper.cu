@@ -14,18 +14,13 @@
 // Device work: (1) column sums of the factor rows with FP32 partials per block
 // combined in FP64; (2) the centred scatter, a K x K Gram over all rows with
 // FP32 register tiles per block, combined in FP64 in a fixed block order;
-// (3) the FP64 draw (O(K^3), independent of the row count): the posterior,
-// its Cholesky factorisation and the Bartlett draws in one CTA, the
-// triangular inverse a warp per column, the two K^3 / 6 products a CTA per
-// row, mu in one CTA.  On a GB300 a dependent FP64 multiply-add takes 64
-// cycles and an SM issues one FP64 warp instruction per 19 cycles whatever the
-// number of active lanes, so the one-CTA steps keep their operands in shared
-// memory (filled by asynchronous copies) and their chains short.
+// (3) the FP64 draw, O(K^3) and independent of the row count (wishart.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
 
 #include "bpmf_impl.cuh"
+#include "hyper.cuh"
 
 namespace gb {
 namespace {
@@ -161,9 +156,6 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
 }
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -322,8 +314,9 @@ __global__ void __launch_bounds__(32 * kFinalWarps) scatter_final(
   }
 }
 
-// ---- (3) FP64 dense algebra by one CTA on row-major K x K matrices in
-// global scratch.  Every helper starts and ends with the block synchronised.
+// ---- FP64 dense algebra by one CTA on row-major K x K matrices in global
+// scratch, for the prior and for hyperparameters that are set.  Every helper
+// starts and ends with the block synchronised.
 
 // In-place lower Cholesky (upper part zeroed), right-looking by columns.
 // Returns false (to all threads) if a pivot is not positive.  FP64 roots and
@@ -333,18 +326,16 @@ __global__ void __launch_bounds__(32 * kFinalWarps) scatter_final(
 // k, warp 0 first updates A[k+1][k+1] (the only entry of row k + 1 that
 // column k changes) and its lane 0 forms the next pivot while the other warps
 // update the remaining rows.  Two barriers per column.
-__device__ bool cta_cholesky(double* A, int K, int* bad, double* rdiag = nullptr, int ld = 0) {
-  if (ld == 0) ld = K;
+__device__ bool cta_cholesky(double* A, int K, int* bad) {
   __shared__ double s_rd[2];
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
   auto pivot = [&](int k) {  // one thread
-    const double piv = A[k * ld + k];
+    const double piv = A[k * K + k];
     const bool ok = piv > 0.0;
     const double r = ok ? rsqrt(piv) : 1.0;
     if (!ok) *bad = 1;
-    A[k * ld + k] = ok ? piv * r : 1.0;
+    A[k * K + k] = ok ? piv * r : 1.0;
     s_rd[k & 1] = r;
-    if (rdiag != nullptr) rdiag[k] = r;
   };
   if (tid == 0) {
     *bad = 0;
@@ -355,27 +346,27 @@ __device__ bool cta_cholesky(double* A, int K, int* bad, double* rdiag = nullptr
   const int slot = (w + nw - 1) % nw;
   for (int k = 0; k < K; ++k) {
     const double rd = s_rd[k & 1];
-    for (int i = k + 1 + tid; i < K; i += nt) A[i * ld + k] *= rd;
+    for (int i = k + 1 + tid; i < K; i += nt) A[i * K + k] *= rd;
     __syncthreads();
     if (w == 0 && k + 1 < K) {
       if (lane == 0) {
-        const double l = A[(k + 1) * ld + k];
-        A[(k + 1) * ld + k + 1] = fma(-l, l, A[(k + 1) * ld + k + 1]);
+        const double l = A[(k + 1) * K + k];
+        A[(k + 1) * K + k + 1] = fma(-l, l, A[(k + 1) * K + k + 1]);
         pivot(k + 1);
       }
       __syncwarp();
     }
     // the rest of the trailing update of the lower triangle, a warp per row
     for (int i = k + 2 + slot; i < K; i += nw) {
-      const double aik = A[i * ld + k];
+      const double aik = A[i * K + k];
       for (int j = k + 1 + lane; j <= i; j += 32)
-        A[i * ld + j] = fma(-aik, A[j * ld + k], A[i * ld + j]);
+        A[i * K + j] = fma(-aik, A[j * K + k], A[i * K + j]);
     }
     __syncthreads();
   }
   for (int e = tid; e < K * K; e += nt) {
     const int i = e / K, j = e % K;
-    if (j > i) A[i * ld + j] = 0.0;
+    if (j > i) A[i * K + j] = 0.0;
   }
   __syncthreads();
   const bool ok = *bad == 0;
@@ -418,64 +409,6 @@ __device__ void cta_tri_inverse(const double* L, double* Linv, int K) {
   __syncthreads();
 }
 
-// T = L^-1 for lower-triangular L (row-major, K x K, in global memory; rdiag
-// = 1 / L_ii), one warp per column (blockIdx.x = j): L t_j = e_j by
-// column-oriented forward substitution -- lane l holds the entries
-// l + 32 m; at step i the owner of row i scales it by rdiag[i] and
-// broadcasts it, and every lane subtracts L[r][i] t_i from its rows r > i.
-// The block L[j..K-1][j..K-1] and rdiag are first copied to shared memory
-// (row stride odd in doubles, so that the lanes' reads of a column fall on
-// different banks), so the chain of steps waits on no global load; a lane
-// group m is skipped once all its rows are at or above the step.  The
-// columns are independent, so K CTAs run them side by side.
-int tri_inverse_smem(int K) { return (int)sizeof(double) * (K * (K + 2) + K); }
-
-__global__ void __launch_bounds__(32) tri_inverse_cols(const double* __restrict__ L,
-                                                       const double* __restrict__ rdiag, double* T,
-                                                       int K, const double* ok) {
-  constexpr int kNpl = kMaxK / 32;
-  extern __shared__ double s_l[];
-  if (ok != nullptr && *ok == 0.0) return;
-  const int j = blockIdx.x, lane = threadIdx.x;
-  const int n = K - j, ld = (n & 1) ? n + 2 : n + 1;
-  double* s_rd = s_l + n * ld;
-  // asynchronous 8-byte copies: all of a lane's loads are in flight at once
-  for (int e = lane; e < n * n; e += 32) {
-    const int r = e / n, c = e - r * n;
-    if (c <= r) cp_async8(s_l + r * ld + c, L + (int64_t)(j + r) * K + j + c);
-    else s_l[r * ld + c] = 0.0;
-  }
-  for (int i = lane; i < n; i += 32) cp_async8(s_rd + i, rdiag + j + i);
-  cp_async_commit();
-  cp_async_wait<0>();
-  __syncwarp();
-  // local row index q = r - j
-  double t[kNpl];
-#pragma unroll
-  for (int m = 0; m < kNpl; ++m) t[m] = lane + 32 * m == 0 ? 1.0 : 0.0;
-  for (int i = 0; i < n; ++i) {
-    const int mi = i >> 5;
-    double ti = 0.0;
-#pragma unroll
-    for (int m = 0; m < kNpl; ++m)
-      if (m == mi) ti = t[m] * s_rd[i];
-    ti = __shfl_sync(0xffffffffu, ti, i & 31);
-#pragma unroll
-    for (int m = 0; m < kNpl; ++m) {
-      if (32 * m + 31 < i) continue;  // every row of group m is at or above i (warp-uniform)
-      const int q = lane + 32 * m;
-      if (q == i) t[m] = ti;
-      else if (q > i && q < n) t[m] = fma(-s_l[q * ld + i], ti, t[m]);
-    }
-  }
-#pragma unroll
-  for (int m = 0; m < kNpl; ++m) {
-    const int q = lane + 32 * m;
-    if (q < n) T[(j + q) * K + j] = t[m];
-  }
-  for (int r = lane; r < j; r += 32) T[r * K + j] = 0.0;
-}
-
 // C = A^T A (symmetric)
 __device__ void cta_ata(const double* A, double* C, int K) {
   for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
@@ -483,52 +416,6 @@ __device__ void cta_ata(const double* A, double* C, int K) {
     double s = 0.0;
     for (int k = 0; k < K; ++k) s += A[k * K + i] * A[k * K + j];
     C[e] = s;
-  }
-  __syncthreads();
-}
-
-// Bartlett's lower-triangular A for Wishart(., nu): A_kl ~ N(0, 1) for
-// k > l (normal number k (k - 1) / 2 + l of counter base (0, t, ., WISHART),
-// Box-Muller in FP32 like the row normals: these decide nothing discrete)
-// and A_kk = sqrt(chi^2(nu - k)), chi^2(m) = 2 Gamma(m / 2) by Marsaglia-Tsang
-// in FP64 with the attempt number as the counter's third word (counter (k, t,
-// a, GAMMA)); the acceptance test decides which attempt is kept, so it runs
-// in FP64 like the reference.  The attempt cap flags kStatusRng.
-__device__ void cta_bartlett_A(double* A, int K, double nu, uint2 key, uint32_t t, int side,
-                               int cap, int* status) {
-  const uint32_t sw_w = stream_word(kStreamWishart, side);
-  const uint32_t sw_g = stream_word(kStreamGamma, side);
-  for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-    const int k = e / K, l = e % K;
-    double v = 0.0;
-    if (l < k) v = (double)normal_at_f32(key, 0u, t, sw_w, (uint32_t)(k * (k - 1) / 2 + l));
-    A[e] = v;
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const double shape = 0.5 * (nu - (double)k);
-    const double s = shape < 1.0 ? shape + 1.0 : shape;
-    const double d = s - 1.0 / 3.0;
-    const double c = 1.0 / sqrt(9.0 * d);
-    double g = -1.0;
-    for (int a = 0; a < cap && g < 0.0; ++a) {
-      const uint4 w = philox(make_uint4((uint32_t)k, t, (uint32_t)a, sw_g), key);
-      double zn, zs;
-      normal2_f64(w.x, w.y, zn, zs);
-      double v = 1.0 + c * zn;
-      if (v <= 0.0) continue;
-      v = v * v * v;
-      const double u = unit_f64(w.z);
-      if (log(u) < 0.5 * zn * zn + d - d * v + d * log(v)) {
-        g = d * v;
-        if (shape < 1.0) g *= pow(unit_f64(w.w), 1.0 / shape);
-      }
-    }
-    if (g < 0.0) {
-      atomicOr(status, kStatusRng);
-      g = s;
-    }
-    A[k * K + k] = sqrt(2.0 * g);
   }
   __syncthreads();
 }
@@ -573,188 +460,6 @@ __device__ void write_bordered(const double* lam, const double* mu, int K, float
   }
   if (threadIdx.x == 0) out[K * KA + K] = 0.f;
   __syncthreads();
-}
-
-struct HyperArgs {
-  const double* xbar;
-  const double* S;
-  int64_t n;
-  const double* mu0;
-  double beta0, nu0;
-  const double* W0inv;
-  uint64_t seed;
-  const uint32_t* tp;  // iteration word on the device
-  int side;
-  int K;
-  double* scr;  // 6 K*K + 2 K doubles
-  double* lam;
-  double* mu;
-  float* lamaug;
-  float* lchol;  // chol(Lambda) = B in FP32, packed by rows, for the rank-one row kernel
-  int* status;
-  int gamma_cap;  // Gamma rejection attempts per draw before kStatusRng
-};
-
-// The posterior draw.  Two exact identities keep the FP64 work to about
-// K^3 / 6 multiply-adds per step:
-//  * C = chol(W*) without forming W* = (W*^-1)^-1: with J the reversal
-//    permutation and L_M = chol(J W*^-1 J), W*^-1 = (J L_M J)(J L_M J)^T with
-//    J L_M J upper triangular, so W* = (J L_M^-T J)(J L_M^-T J)^T and
-//    C = J L_M^-T J, i.e. C[i][j] = T[K-1-j][K-1-i] with T = L_M^-1
-//    (lower triangular with a positive diagonal, hence the Cholesky factor);
-//  * chol(beta* Lambda) = sqrt(beta*) B for B = C A (lower triangular with a
-//    positive diagonal and Lambda = B B^T), so mu = mu* + B^-T z / sqrt(beta*).
-// The Cholesky, the Bartlett draws and the back substitution for mu run in
-// one CTA; L_M^-1 runs one warp per column, and B = C A and Lambda = B B^T,
-// each K^3 / 6 multiply-adds with no chain between rows, one CTA per row.
-// Scratch (doubles): Mx | T | A | B (K*K each) | mu* (K) | ...; scr[5 K*K] = 1
-// once the factorisation succeeded (0: the later steps skip), followed by
-// 1 / diag(L_M) (K).
-
-// (3a) posterior, L_M, Bartlett A and mu*, by one CTA (T = L_M^-1 follows in
-// tri_inverse_cols).  The factorisation runs on a copy in shared memory with
-// an odd row stride (K + 1 doubles), so that the column reads of the trailing
-// update fall on different banks; the factor is then written to scratch.
-int wishart_factor_smem(int K) { return (int)sizeof(double) * K * (K + 1); }
-
-__global__ void __launch_bounds__(512) wishart_factor(HyperArgs a) {
-  extern __shared__ double s_mx[];  // J W*^-1 J, then L_M; row stride K + 1
-  __shared__ int bad;
-  const int K = a.K, KK = K * K, ld = K + 1;
-  double* Mx = a.scr;          // L_M
-  double* A = Mx + 2 * KK;     // Bartlett A (L_M^-1 goes between the two)
-  double* mus = A + 2 * KK;    // mu*
-  double* ok = a.scr + 5 * KK;
-  const double n = (double)a.n;
-  const double w = a.beta0 * n / (a.beta0 + n);
-  __shared__ double s_dm[kMaxK];  // mu0 - xbar
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    s_dm[k] = a.mu0[k] - a.xbar[k];
-    mus[k] = (a.beta0 * a.mu0[k] + n * a.xbar[k]) / (a.beta0 + n);
-  }
-  __syncthreads();
-  // (J W*^-1 J)[e / K][e % K] = W*^-1[K-1-e/K][K-1-e%K]; four loads of each
-  // matrix in flight per thread and pass
-  const int nt = blockDim.x;
-  for (int e0 = threadIdx.x; e0 < KK; e0 += 4 * nt) {
-    double wv[4], sv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * nt;
-      const int src = KK - 1 - e;  // (K-1-e/K) K + (K-1-e%K)
-      wv[u] = e < KK ? a.W0inv[src] : 0.0;
-      sv[u] = e < KK ? a.S[src] : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * nt;
-      if (e < KK) {
-        const int i = K - 1 - e / K, j = K - 1 - e % K;
-        s_mx[(e / K) * ld + e % K] = wv[u] + sv[u] + w * s_dm[i] * s_dm[j];
-      }
-    }
-  }
-  __syncthreads();
-  const double nu_s = a.nu0 + n;
-  const bool factored = cta_cholesky(s_mx, K, &bad, ok + 1, ld);
-  for (int e = threadIdx.x; e < KK; e += blockDim.x) Mx[e] = s_mx[(e / K) * ld + e % K];
-  if (!factored) {
-    if (threadIdx.x == 0) {
-      *ok = 0.0;
-      atomicOr(a.status, kStatusNotPD);
-    }
-    return;
-  }
-  cta_bartlett_A(A, K, nu_s, seed_key(a.seed), *a.tp, a.side, a.gamma_cap, a.status);
-  if (threadIdx.x == 0) *ok = 1.0;
-}
-
-// (3b) row i of B = C A (blockIdx.x = i), and its FP32 copy packed by rows:
-// B = chol(Lambda) for the rank-one row kernel
-__global__ void __launch_bounds__(128) wishart_b(HyperArgs a) {
-  const int K = a.K, KK = K * K, i = blockIdx.x;
-  if (a.scr[5 * KK] == 0.0) return;
-  const double* T = a.scr + KK;
-  const double* A = T + KK;
-  double* B = a.scr + 3 * KK;
-  for (int j = threadIdx.x; j < K; j += blockDim.x) {
-    // B[i][j] = sum over m = j .. i of C[i][m] A[m][j], C[i][m] = T[K-1-m][K-1-i]
-    const double v = j <= i ? dot4(T + (K - 1 - j) * K + (K - 1 - i), -K, A + j * K + j, K, i - j + 1)
-                            : 0.0;
-    B[i * K + j] = v;
-    if (j <= i) a.lchol[i * (i + 1) / 2 + j] = (float)v;
-  }
-}
-
-// (3c) row i of Lambda = B B^T (lower triangle, mirrored)
-__global__ void __launch_bounds__(128) wishart_lam(HyperArgs a) {
-  const int K = a.K, KK = K * K, i = blockIdx.x;
-  if (a.scr[5 * KK] == 0.0) return;
-  const double* B = a.scr + 3 * KK;
-  for (int j = threadIdx.x; j <= i; j += blockDim.x) {
-    const double v = dot4(B + i * K, 1, B + j * K, 1, j + 1);
-    a.lam[i * K + j] = v;
-    a.lam[j * K + i] = v;
-  }
-}
-
-// (3d) mu = mu* + B^-T z / sqrt(beta*) by one CTA: back substitution from the
-// bottom, each solved x_i subtracted from the remaining right-hand sides by
-// all threads; then the FP32 bordered copy
-int wishart_mu_smem(int K) { return (int)sizeof(double) * K * K; }
-
-__global__ void __launch_bounds__(128) wishart_mu(HyperArgs a) {
-  __shared__ double xs[kMaxK], zr[kMaxK], rd[kMaxK];
-  __shared__ double s_rb;
-  extern __shared__ double s_b[];  // B, K x K, so that the chain below waits on no global load
-  const int K = a.K, KK = K * K;
-  if (a.scr[5 * KK] == 0.0) return;
-  const double* B = a.scr + 3 * KK;
-  const double* mus = a.scr + 4 * KK;
-  const uint2 key = seed_key(a.seed);
-  const uint32_t t = *a.tp;
-  const uint32_t sw = stream_word(kStreamHyperMu, a.side);
-  for (int e = threadIdx.x; e < KK; e += blockDim.x) cp_async8(s_b + e, B + e);
-  cp_async_commit();
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    zr[k] = (double)normal_at_f32(key, 0u, t, sw, (uint32_t)k);
-    rd[k] = 1.0 / B[k * K + k];
-  }
-  if (threadIdx.x == 0) s_rb = 1.0 / sqrt(a.beta0 + (double)a.n);
-  cp_async_wait<0>();
-  __syncthreads();
-  // x = B^-T z from the bottom by warp 0, lane l holding z_k for
-  // k = l + 32 m: the owner of row i forms x_i and broadcasts it, every lane
-  // subtracts B[i][k] x_i from its rows k < i (each z_k sees the same updates
-  // in the same order as a serial back substitution); a group m is skipped
-  // once all its rows are at or past i
-  if (threadIdx.x < 32) {
-    constexpr int kNpl = kMaxK / 32;
-    const int lane = threadIdx.x;
-    double z[kNpl];
-#pragma unroll
-    for (int m = 0; m < kNpl; ++m) z[m] = lane + 32 * m < K ? zr[lane + 32 * m] : 0.0;
-    for (int i = K - 1; i >= 0; --i) {
-      const int mi = i >> 5;
-      double xi = 0.0;
-#pragma unroll
-      for (int m = 0; m < kNpl; ++m)
-        if (m == mi) xi = z[m] * rd[i];
-      xi = __shfl_sync(0xffffffffu, xi, i & 31);
-      if (lane == (i & 31)) xs[i] = xi;
-#pragma unroll
-      for (int m = 0; m < kNpl; ++m) {
-        if (32 * m >= i) continue;  // warp-uniform
-        const int k = lane + 32 * m;
-        if (k < i) z[m] = fma(-s_b[i * K + k], xi, z[m]);
-      }
-    }
-  }
-  __syncthreads();
-  const double rb = s_rb;
-  for (int k = threadIdx.x; k < K; k += blockDim.x) a.mu[k] = mus[k] + xs[k] * rb;
-  __syncthreads();
-  write_bordered(a.lam, a.mu, K, a.lamaug);
 }
 
 // Ainv = A^-1 for SPD A (used once for W0^-1); flags kStatusNotPD.
@@ -862,6 +567,7 @@ int launch_hyper(Handle* h, int s, cudaStream_t st, bool alt) {
   a.mu0 = h->mu0;
   a.beta0 = h->cfg.beta0;
   a.nu0 = h->cfg.nu0;
+  a.wmean = a.beta0 * (double)R / (a.beta0 + (double)R);
   a.W0inv = h->W0inv;
   a.seed = h->cfg.seed;
   a.tp = h->d_iter;
@@ -876,20 +582,7 @@ int launch_hyper(Handle* h, int s, cudaStream_t st, bool alt) {
   a.gamma_cap = h->gamma_cap;
   {
     PhaseTimer timer(h, BPMF_T_HYPER_DRAW, st);
-    const int smem = wishart_factor_smem(K);
-    BPMF_CUDA_CHECK(cudaFuncSetAttribute(wishart_factor, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    wishart_factor<<<1, 512, smem, st>>>(a);
-    const int tsmem = tri_inverse_smem(K);
-    BPMF_CUDA_CHECK(cudaFuncSetAttribute(tri_inverse_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, tsmem));
-    tri_inverse_cols<<<K, 32, tsmem, st>>>(a.scr, a.scr + 5 * K * K + 1, a.scr + K * K, K,
-                                       a.scr + 5 * K * K);
-    wishart_b<<<K, 128, 0, st>>>(a);
-    wishart_lam<<<K, 128, 0, st>>>(a);
-    const int msmem = wishart_mu_smem(K);
-    BPMF_CUDA_CHECK(cudaFuncSetAttribute(wishart_mu, cudaFuncAttributeMaxDynamicSharedMemorySize, msmem));
-    wishart_mu<<<1, 128, msmem, st>>>(a);
-    BPMF_CUDA_CHECK(cudaGetLastError());
-    h->kernels += 4;
+    BPMF_TRY(launch_wishart(a, st, &h->kernels));
   }
   sd.have_hyper = true;
   sd.have_stats = true;
