@@ -301,6 +301,7 @@ int time_sweep(Handle* h, int s, float* scratch, int reps, float* best_ms) {
     if (r > reps && (total >= kTuneMinMs || r > kTuneMaxReps)) break;
     SweepArgs a = make_sweep_args(h, s);
     a.X = scratch;
+    a.Xhi = a.Xlo = nullptr;
     if (cudaMemsetAsync(h->flag_count, 0, sizeof(int32_t), h->stream) != cudaSuccess ||
         cudaEventRecord(e0, h->stream) != cudaSuccess)
       rc = BPMF_ECUDA;

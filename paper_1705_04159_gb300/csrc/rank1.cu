@@ -521,7 +521,10 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
 #pragma unroll
         for (int m = 0; m < NPL; ++m) {
           const int i = lane + 32 * m;
-          if (i < K) out[i] = u[r][m];
+          if (i < K) {
+            out[i] = u[r][m];
+            write_shadow(a, row, i, u[r][m]);
+          }
         }
       }
     }

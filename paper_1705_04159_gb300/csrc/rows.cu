@@ -259,7 +259,10 @@ __global__ void __launch_bounds__(256) row_fp64(const SweepArgs a, const double*
         for (int k = i + 1; k < K; ++k) t -= A[k * K + i] * b[k];
         b[i] = t / A[i * K + i];
       }
-      for (int i = 0; i < K; ++i) a.X[(int64_t)row * K + i] = (float)b[i];
+      for (int i = 0; i < K; ++i) {
+        a.X[(int64_t)row * K + i] = (float)b[i];
+        write_shadow(a, row, i, (float)b[i]);
+      }
     }
   }
 }
@@ -348,6 +351,8 @@ SweepArgs make_sweep_args(Handle* h, int s) {
   a.work = sd.work;
   a.Vhi = od.Xhi;
   a.Vlo = od.Xlo;
+  a.Xhi = sd.Xhi;
+  a.Xlo = sd.Xlo;
   a.KS = od.KS;
   a.n_other = od.R;
   return a;
@@ -374,13 +379,10 @@ int launch_sweep(Handle* h, int s) {
       BPMF_TRY(launch_sweep_binned(h, s, a));
     }
   }
-  {
-    PhaseTimer timer(h, BPMF_T_FP64_REDO);
-    BPMF_TRY(launch_fp64_redo(h, s, a));
-    h->kernels += 1;
-  }
-  // the next half-sweep gathers this side's new rows from the shadow
-  return launch_refresh_shadow(h, s);
+  PhaseTimer timer(h, BPMF_T_FP64_REDO);
+  BPMF_TRY(launch_fp64_redo(h, s, a));
+  h->kernels += 1;
+  return BPMF_OK;
 }
 
 int launch_init_factors(Handle* h, int s) {

@@ -39,11 +39,28 @@ struct SweepArgs {
   // bf16 hi/lo shadow of the other side's factors, rows padded to KS (mixed path)
   const __nv_bfloat16* Vhi;
   const __nv_bfloat16* Vlo;
+  // that of this side's factors (written with X), or null
+  __nv_bfloat16* Xhi;
+  __nv_bfloat16* Xlo;
   int KS;
   int64_t n_other;      // rows of the other side (of Vo and its shadow)
   // per slot of the degree order: (row, first rating, one past the last, 0)
   const int4* work;
 };
+
+// x as the shadow's pair hi + lo
+__device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
+  hi = __float2bfloat16_rn(x);
+  lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+}
+// column i of a drawn row into the shadow
+__device__ __forceinline__ void write_shadow(const SweepArgs& a, int row, int i, float x) {
+  if (a.Xhi == nullptr) return;
+  __nv_bfloat16 h, l;
+  split_bf16(x, h, l);
+  a.Xhi[(int64_t)row * a.KS + i] = h;
+  a.Xlo[(int64_t)row * a.KS + i] = l;
+}
 
 SweepArgs make_sweep_args(Handle* h, int s);
 // whole rows row_begin..row_end of the row list, Gram from the ratings

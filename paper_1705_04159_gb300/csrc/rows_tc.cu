@@ -410,7 +410,7 @@ __device__ __forceinline__ bool tc_cholesky(const TileGeom& G, const TcSmem& s, 
 // thread above the block then subtracts the block's contribution.
 __device__ __forceinline__ void tc_backward_solve(const float* Lr, int LDS, int K,
                                                   const float* rinv, const float* zv, float* xs,
-                                                  float* __restrict__ xout) {
+                                                  const SweepArgs& a, int row) {
   const int i = threadIdx.x, warp = i >> 5;
   float w = i < K ? Lr[K * LDS + i] + zv[i] : 0.f;
   for (int b = (K + 15) / 16 - 1; b >= 0; --b) {
@@ -431,7 +431,10 @@ __device__ __forceinline__ void tc_backward_solve(const float* Lr, int LDS, int 
       w = t;
     }
   }
-  if (i < K) xout[i] = w;
+  if (i < K) {
+    a.X[(int64_t)row * K + i] = w;
+    write_shadow(a, row, i, w);
+  }
 }
 
 }  // namespace
@@ -470,7 +473,7 @@ __global__ void __launch_bounds__(kTcThreads) row_tc(const SweepArgs a, int* sta
     if (tid == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
     return;
   }
-  tc_backward_solve(s.Lr, G.LDS, a.K, s.rinv, s.zv, s.l11, a.X + (int64_t)row * a.K);
+  tc_backward_solve(s.Lr, G.LDS, a.K, s.rinv, s.zv, s.l11, a, row);
 }
 
 // Partial Gram of one piece of a split row on tensor cores, written as the

@@ -847,17 +847,29 @@ __global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
 }
 
 // bf16 hi/lo shadow of a factor matrix, rows padded to KS (a multiple of 8)
-__global__ void refresh_shadow_kernel(const float* __restrict__ X, int64_t R, int K, int KS,
-                                      __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-  const int64_t total = R * KS;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / KS;
-    const int c = (int)(e - r * KS);
-    const float x = c < K ? X[r * K + c] : 0.f;
-    const __nv_bfloat16 h = __float2bfloat16_rn(x);
-    hi[e] = h;
-    lo[e] = __float2bfloat16_rn(x - __bfloat162float(h));
+// for factors that are set or initialised (a draw writes its own); a thread
+// converts eight columns, KS / 8 threads a row
+constexpr int kShadowThreads = 256;
+__global__ void __launch_bounds__(kShadowThreads) refresh_shadow_kernel(const float* __restrict__ X, int64_t R,
+                                                                        int K, int KS,
+                                                                        __nv_bfloat16* __restrict__ hi,
+                                                                        __nv_bfloat16* __restrict__ lo) {
+  const int Q = KS >> 3, per = kShadowThreads / Q;
+  const int q = threadIdx.x % Q, rr = threadIdx.x / Q, c = 8 * q;
+  if (rr >= per) return;
+  for (int64_t r = (int64_t)blockIdx.x * per + rr; r < R; r += (int64_t)gridDim.x * per) {
+    float x[8];
+    if ((K & 3) == 0 && c + 8 <= K) {
+      ld8(X + r * K + c, x);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) x[k] = c + k < K ? X[r * K + c + k] : 0.f;
+    }
+    __align__(16) __nv_bfloat16 h[8], l[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) split_bf16(x[k], h[k], l[k]);
+    *reinterpret_cast<uint4*>(hi + r * KS + c) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(lo + r * KS + c) = *reinterpret_cast<const uint4*>(l);
   }
 }
 
@@ -985,10 +997,9 @@ int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross
 int launch_refresh_shadow(Handle* h, int s) {
   SideDev& sd = h->side[s];
   if (!sd.Xhi || sd.R == 0) return BPMF_OK;
-  const int64_t total = sd.R * sd.KS;
-  int64_t g = (total + 255) / 256;
-  if (g > 16LL * h->num_sms) g = 16LL * h->num_sms;
-  refresh_shadow_kernel<<<(unsigned)g, 256, 0, h->stream>>>(sd.X, sd.R, h->K, sd.KS, sd.Xhi, sd.Xlo);
+  const int per = kShadowThreads / (sd.KS >> 3);
+  const int64_t g = std::min<int64_t>((sd.R + per - 1) / per, 16LL * h->num_sms);
+  refresh_shadow_kernel<<<(unsigned)g, kShadowThreads, 0, h->stream>>>(sd.X, sd.R, h->K, sd.KS, sd.Xhi, sd.Xlo);
   BPMF_CUDA_CHECK(cudaGetLastError());
   h->kernels += 1;
   return BPMF_OK;

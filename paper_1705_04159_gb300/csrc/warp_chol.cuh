@@ -232,8 +232,10 @@ __device__ __forceinline__ bool warp_cholesky(int g, float* T, const float* thr_
 // solves the 8 x 8 system, and each subtracts the block's part from its
 // columns.  The next block's diagonal tile is loaded a step ahead; the other
 // tiles are not, which would take 32 registers more.
-__device__ __forceinline__ void warp_back(int K, const float* T, const float* rinv, const float* zv,
-                                          int lane, float* out) {
+__device__ __forceinline__ void warp_back(const SweepArgs& a, const float* T, const float* rinv,
+                                          const float* zv, int row, int lane) {
+  const int K = a.K;
+  float* out = a.X + (int64_t)row * K;
   const int J = lane >> 1, h4 = (lane & 1) << 2;
   const int IK = K >> 3, pk = K & 7;
   float v[4];
@@ -291,11 +293,27 @@ __device__ __forceinline__ void warp_back(int K, const float* T, const float* ri
   }
   const int c0 = 8 * J + h4;
   if ((K & 3) == 0) {  // the row of X starts on a 16-byte boundary
-    if (c0 < K) *reinterpret_cast<float4*>(out + c0) = make_float4(v[0], v[1], v[2], v[3]);
+    if (c0 < K) {
+      *reinterpret_cast<float4*>(out + c0) = make_float4(v[0], v[1], v[2], v[3]);
+      if (a.Xhi != nullptr) {
+        __nv_bfloat16 h[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) split_bf16(v[k], h[k], l[k]);
+        __nv_bfloat162* hi = reinterpret_cast<__nv_bfloat162*>(a.Xhi + (int64_t)row * a.KS + c0);
+        __nv_bfloat162* lo = reinterpret_cast<__nv_bfloat162*>(a.Xlo + (int64_t)row * a.KS + c0);
+        hi[0] = __nv_bfloat162(h[0], h[1]);
+        hi[1] = __nv_bfloat162(h[2], h[3]);
+        lo[0] = __nv_bfloat162(l[0], l[1]);
+        lo[1] = __nv_bfloat162(l[2], l[3]);
+      }
+    }
   } else {
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      if (c0 + k < K) out[c0 + k] = v[k];
+      if (c0 + k < K) {
+        out[c0 + k] = v[k];
+        write_shadow(a, row, c0 + k, v[k]);
+      }
   }
 }
 
@@ -325,7 +343,7 @@ __device__ __forceinline__ void row_draw(const SweepArgs& a, int g, float* T, co
     *reinterpret_cast<float4*>(zv + 4 * q) =
         normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)q, a.sw), a.key));
   const bool ok = warp_cholesky(g, T, thr, rinv, lane);
-  if (ok) warp_back(a.K, T, rinv, zv, lane, a.X + (int64_t)row * a.K);
+  if (ok) warp_back(a, T, rinv, zv, row, lane);
   else if (lane == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
 }
 
