@@ -59,31 +59,65 @@ void free_handle(Handle* h) {
   if (h->ev_join2) cudaEventDestroy(h->ev_join2);
   for (int s = 0; s < 2; ++s) {
     SideDev& sd = h->side[s];
-    dfree(sd.ptr); dfree(sd.idx); dfree(sd.val); dfree(sd.perm); dfree(sd.X); dfree(sd.Xhi);
-    dfree(sd.Xlo); dfree(sd.work);
-    dfree(sd.lam); dfree(sd.mu); dfree(sd.lamaug); dfree(sd.lchol); dfree(sd.linvT); dfree(sd.tiny_pre); dfree(sd.xbar); dfree(sd.S);
-    dfree(sd.piece_row); dfree(sd.piece_e0); dfree(sd.piece_e1); dfree(sd.hub_piece0);
+    dfree(sd.tiny_pre);
+    if (sd.piece_own) dfree(sd.piece_mem);
   }
-  dfree(h->mu0); dfree(h->W0inv); dfree(h->red); dfree(h->wscr); dfree(h->red2); dfree(h->wscr2);
-  dfree(h->status);
-  dfree(h->flag_rows); dfree(h->flag_count); dfree(h->trow); dfree(h->tcol); dfree(h->tval);
-  dfree(h->tsum); dfree(h->terr); dfree(h->hub_part); dfree(h->d_iter); dfree(h->d_navg);
-  dfree(h->ws_counter);
+  dfree(h->block); dfree(h->tblock); dfree(h->hub_part);
   delete h;
 }
 
-// Copies n elements to a fresh device buffer unless they already live there.
+// n elements on the device: where they live already, or a copy in space taken
+// from c (which only adds up bytes as long as it has no block).
 template <typename T>
-int to_device(const T* src, int64_t n, bool devptr, T** dst, bool* owned, cudaStream_t st) {
-  if (devptr || n == 0) {
-    *dst = const_cast<T*>(src);
-    *owned = false;
-    return BPMF_OK;
-  }
-  BPMF_TRY(dalloc(dst, n));
-  *owned = true;
-  BPMF_CUDA_CHECK(cudaMemcpyAsync(*dst, src, sizeof(T) * n, cudaMemcpyHostToDevice, st));
+int to_device(const T* src, int64_t n, bool devptr, T** dst, Carve& c, cudaStream_t st) {
+  *dst = const_cast<T*>(src);
+  if (devptr || n == 0) return BPMF_OK;
+  *dst = c.take<T>(n);
+  if (*dst) BPMF_CUDA_CHECK(cudaMemcpyAsync(*dst, src, sizeof(T) * n, cudaMemcpyHostToDevice, st));
   return BPMF_OK;
+}
+
+constexpr int64_t kPieceBlock = 8192;  // bytes of a side's pieces in the sampler's block
+
+// The sampler's arrays of fixed size; the words that start at zero are
+// consecutive, from status to d_navg.
+void carve_handle(Handle* h, Carve& c) {
+  const int64_t K = h->K, KK = K * K, KP = (K + 31) & ~31;
+  for (SideDev& sd : h->side) {
+    sd.ptr = c.take<int64_t>(sd.R + 1);
+    sd.idx = c.take<int32_t>(h->nnz);
+    sd.val = c.take<float>(h->nnz);
+    sd.perm = c.take<int32_t>(sd.R);
+    sd.work = c.take<int4>(sd.R);
+    sd.X = c.take<float>(sd.R * K);
+    sd.lam = c.take<double>(KK);
+    sd.mu = c.take<double>(K);
+    sd.lamaug = c.take<float>((K + 1) * (K + 1));
+    sd.lchol = c.take<float>(KK);
+    sd.linvT = c.take<float>(KP * (KP + 4));
+    if (h->cfg.path == BPMF_PATH_MIXED) {
+      sd.KS = (int)((K + 7) & ~7);
+      sd.Xhi = c.take<__nv_bfloat16>(sd.R * sd.KS);
+      sd.Xlo = c.take<__nv_bfloat16>(sd.R * sd.KS);
+    }
+    sd.xbar = c.take<double>(K);
+    sd.S = c.take<double>(KK);
+    sd.piece_mem = c.take<char>(kPieceBlock);
+    sd.piece_bytes = kPieceBlock;
+  }
+  h->red = c.take<double>(h->red_len);
+  h->wscr = c.take<double>(6 * KK + 8 * K);
+  h->red2 = c.take<double>(h->red_len);
+  h->wscr2 = c.take<double>(6 * KK + 8 * K);
+  h->mu0 = c.take<double>(K);
+  h->W0inv = c.take<double>(KK);
+  h->flag_rows = c.take<int32_t>(std::max(h->M, h->N));
+  h->terr = c.take<double>(2);
+  h->flag_count = c.take<int32_t>(1);
+  h->ws_counter = c.take<int>(1);
+  h->status = c.take<int>(1);
+  h->d_iter = c.take<uint32_t>(1);
+  h->d_navg = c.take<int64_t>(1);
 }
 
 }  // namespace
@@ -337,7 +371,7 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
   int rc = BPMF_OK;
   int32_t *d_row = nullptr, *d_col = nullptr;
   float* d_val = nullptr;
-  bool own_r = false, own_c = false, own_v = false;
+  char* scratch = nullptr;
   do {
     if (cudaGetDevice(&h->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device) !=
@@ -359,48 +393,17 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
     h->side[BPMF_USERS].R = M;
     h->side[BPMF_MOVIES].R = N;
     const int64_t KK = (int64_t)K * K;
-    for (int s = 0; s < 2 && rc == BPMF_OK; ++s) {
-      SideDev& sd = h->side[s];
-      if ((rc = dalloc(&sd.ptr, sd.R + 1))) break;
-      if ((rc = dalloc(&sd.idx, nnz))) break;
-      if ((rc = dalloc(&sd.val, nnz))) break;
-      if ((rc = dalloc(&sd.perm, sd.R))) break;
-      if ((rc = dalloc(&sd.X, sd.R * K))) break;
-      if ((rc = dalloc(&sd.lam, KK))) break;
-      if ((rc = dalloc(&sd.mu, K))) break;
-      if ((rc = dalloc(&sd.lamaug, (int64_t)(K + 1) * (K + 1)))) break;
-      if ((rc = dalloc(&sd.lchol, KK))) break;
-      {
-        const int64_t KP = (K + 31) & ~31;
-        if ((rc = dalloc(&sd.linvT, KP * (KP + 4)))) break;
-      }
-      if (cfg->path == BPMF_PATH_MIXED) {
-        sd.KS = (K + 7) & ~7;
-        if ((rc = dalloc(&sd.Xhi, sd.R * sd.KS))) break;
-        if ((rc = dalloc(&sd.Xlo, sd.R * sd.KS))) break;
-      }
-      if ((rc = dalloc(&sd.xbar, K))) break;
-      if ((rc = dalloc(&sd.S, KK))) break;
-    }
-    if (rc) break;
     h->red_len = std::max<int64_t>({2LL * h->num_sms * KK, 2LL * h->num_sms * K,
                                     16LL * h->num_sms + 1024, 4096});
-    if ((rc = dalloc(&h->red, h->red_len))) break;
-    if ((rc = dalloc(&h->wscr, 6 * KK + 8 * K))) break;
-    if ((rc = dalloc(&h->red2, h->red_len))) break;
-    if ((rc = dalloc(&h->wscr2, 6 * KK + 8 * K))) break;
-    if ((rc = dalloc(&h->mu0, K))) break;
-    if ((rc = dalloc(&h->W0inv, KK))) break;
-    if ((rc = dalloc(&h->status, 1))) break;
-    if ((rc = dalloc(&h->flag_count, 1))) break;
-    if ((rc = dalloc(&h->flag_rows, std::max(M, N)))) break;
-    if ((rc = dalloc(&h->terr, 2))) break;
-    if ((rc = dalloc(&h->d_iter, 1))) break;
-    if ((rc = dalloc(&h->d_navg, 1))) break;
-    if ((rc = dalloc(&h->ws_counter, 1))) break;
-    if (cudaMemsetAsync(h->status, 0, sizeof(int), h->stream) != cudaSuccess ||
-        cudaMemsetAsync(h->d_iter, 0, sizeof(uint32_t), h->stream) != cudaSuccess ||
-        cudaMemsetAsync(h->d_navg, 0, sizeof(int64_t), h->stream) != cudaSuccess) {
+    {
+      Carve size, c;
+      carve_handle(h, size);
+      if ((rc = dalloc(&h->block, (int64_t)size.bytes))) break;
+      c.base = h->block;
+      carve_handle(h, c);
+    }
+    if (cudaMemsetAsync(h->status, 0, reinterpret_cast<char*>(h->d_navg + 1) - reinterpret_cast<char*>(h->status),
+                        h->stream) != cudaSuccess) {
       rc = BPMF_ECUDA;
       break;
     }
@@ -435,10 +438,22 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
       break;
     }
     // ratings
-    if ((rc = to_device(row, nnz, dev, &d_row, &own_r, h->stream))) break;
-    if ((rc = to_device(col, nnz, dev, &d_col, &own_c, h->stream))) break;
-    if ((rc = to_device(val, nnz, dev, &d_val, &own_v, h->stream))) break;
-    if ((rc = build_structure(h, d_row, d_col, d_val))) break;
+    // scratch: the ratings if they come from the host, then what the structure
+    // takes or, after it, the factors of the autotuner's sweeps
+    const size_t work = std::max(structure_bytes(nnz, M, N),
+                                 cfg->autotune ? sizeof(float) * (size_t)(std::max(M, N) * K) : 0);
+    char* ws = nullptr;
+    for (int pass = 0; pass < 2 && rc == BPMF_OK; ++pass) {
+      Carve c;
+      c.base = scratch;
+      if ((rc = to_device(row, nnz, dev, &d_row, c, h->stream))) break;
+      if ((rc = to_device(col, nnz, dev, &d_col, c, h->stream))) break;
+      if ((rc = to_device(val, nnz, dev, &d_val, c, h->stream))) break;
+      ws = c.take<char>((int64_t)work);
+      if (pass == 0) rc = dalloc(&scratch, (int64_t)c.bytes);
+    }
+    if (rc) break;
+    if ((rc = build_structure(h, d_row, d_col, d_val, ws))) break;
     if ((rc = setup_bins(h, BPMF_USERS))) break;
     if ((rc = setup_bins(h, BPMF_MOVIES))) break;
     if ((rc = launch_init_factors(h, BPMF_USERS))) break;
@@ -446,12 +461,8 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
     if ((rc = launch_refresh_shadow(h, BPMF_USERS))) break;
     if ((rc = launch_refresh_shadow(h, BPMF_MOVIES))) break;
     if (cfg->autotune) {
-      float* scratch = nullptr;
-      if ((rc = dalloc(&scratch, std::max(M, N) * K))) break;
-      rc = autotune_bins(h, BPMF_USERS, scratch);
-      if (rc == BPMF_OK) rc = autotune_bins(h, BPMF_MOVIES, scratch);
-      cudaStreamSynchronize(h->stream);
-      dfree(scratch);
+      rc = autotune_bins(h, BPMF_USERS, reinterpret_cast<float*>(ws));
+      if (rc == BPMF_OK) rc = autotune_bins(h, BPMF_MOVIES, reinterpret_cast<float*>(ws));
       if (rc == BPMF_OK) rc = check_status(h, "bpmf_init (autotune)");
       if (rc) break;
     }
@@ -461,9 +472,10 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
       break;
     }
   } while (0);
-  if (own_r) cudaFree(d_row);
-  if (own_c) cudaFree(d_col);
-  if (own_v) cudaFree(d_val);
+  if (scratch) {
+    cudaStreamSynchronize(h->stream);
+    dfree(scratch);
+  }
   if (rc != BPMF_OK) {
     free_handle(h);
     return rc;
@@ -484,7 +496,8 @@ int bpmf_set_test(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col,
   drop_graph(h);  // the captured iteration holds the old test arrays
   BPMF_CUDA_CHECK(cudaMemsetAsync(h->d_navg, 0, sizeof(int64_t), st));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  dfree(h->trow); dfree(h->tcol); dfree(h->tval); dfree(h->tsum);
+  dfree(h->tblock);
+  h->tblock = nullptr;
   h->trow = h->tcol = nullptr;
   h->tval = nullptr;
   h->tsum = nullptr;
@@ -494,24 +507,28 @@ int bpmf_set_test(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col,
   if (n == 0) return BPMF_OK;
   int32_t *d_row = nullptr, *d_col = nullptr;
   float* d_val = nullptr;
-  bool own_r = false, own_c = false, own_v = false;
+  char *scratch = nullptr, *ws = nullptr;
   int rc = BPMF_OK;
-  uint32_t *keys = nullptr, *keys_sorted = nullptr;
-  int32_t *ids = nullptr, *src = nullptr;
   do {
-    if ((rc = to_device(row, n, dev, &d_row, &own_r, st))) break;
-    if ((rc = to_device(col, n, dev, &d_col, &own_c, st))) break;
-    if ((rc = to_device(val, n, dev, &d_val, &own_v, st))) break;
-    if ((rc = dalloc(&h->trow, n))) break;
-    if ((rc = dalloc(&h->tcol, n))) break;
-    if ((rc = dalloc(&h->tval, n))) break;
-    if ((rc = dalloc(&h->tsum, n))) break;
-    if ((rc = dalloc(&keys, n))) break;
-    if ((rc = dalloc(&keys_sorted, n))) break;
-    if ((rc = dalloc(&ids, n))) break;
-    if ((rc = dalloc(&src, n))) break;
+    for (int pass = 0; pass < 2 && rc == BPMF_OK; ++pass) {
+      Carve c;  // scratch
+      c.base = scratch;
+      if ((rc = to_device(row, n, dev, &d_row, c, st))) break;
+      if ((rc = to_device(col, n, dev, &d_col, c, st))) break;
+      if ((rc = to_device(val, n, dev, &d_val, c, st))) break;
+      ws = c.take<char>((int64_t)test_sort_bytes(n));
+      Carve k;  // kept
+      k.base = h->tblock;
+      h->trow = k.take<int32_t>(n);
+      h->tcol = k.take<int32_t>(n);
+      h->tval = k.take<float>(n);
+      h->tsum = k.take<float2>(n);
+      if (pass == 0 && (rc = dalloc(&scratch, (int64_t)c.bytes)) == BPMF_OK)
+        rc = dalloc(&h->tblock, (int64_t)k.bytes);
+    }
+    if (rc) break;
     // validate, then sort by user (stable) for gather locality
-    rc = sort_test_set(h, d_row, d_col, d_val, n, keys, keys_sorted, ids, src);
+    rc = sort_test_set(h, d_row, d_col, d_val, n, ws);
     if (rc) break;
     if (cudaMemsetAsync(h->tsum, 0, sizeof(float2) * n, st) != cudaSuccess) {
       rc = BPMF_ECUDA;
@@ -520,10 +537,10 @@ int bpmf_set_test(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col,
     h->n_test = n;
     rc = check_status(h, "bpmf_set_test");
   } while (0);
-  if (own_r) cudaFree(d_row);
-  if (own_c) cudaFree(d_col);
-  if (own_v) cudaFree(d_val);
-  dfree(keys); dfree(keys_sorted); dfree(ids); dfree(src);
+  if (scratch) {
+    cudaStreamSynchronize(st);
+    dfree(scratch);
+  }
   if (rc != BPMF_OK) h->n_test = 0;
   return rc;
 }
@@ -588,14 +605,20 @@ int bpmf_predict(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col, 
   if (n == 0) return BPMF_OK;
   const bool dev = (flags & BPMF_DEVPTR) != 0;
   int32_t *d_row = nullptr, *d_col = nullptr;
-  float* d_out = nullptr;
-  bool own_r = false, own_c = false;
+  float* d_out = dev ? out : nullptr;
+  char* scratch = nullptr;
   int rc = BPMF_OK;
   do {
-    if ((rc = to_device(row, n, dev, &d_row, &own_r, h->stream))) break;
-    if ((rc = to_device(col, n, dev, &d_col, &own_c, h->stream))) break;
-    if (dev) d_out = out;
-    else if ((rc = dalloc(&d_out, n))) break;
+    for (int pass = 0; pass < 2 && rc == BPMF_OK; ++pass) {
+      Carve c;
+      c.base = scratch;
+      if ((rc = to_device(row, n, dev, &d_row, c, h->stream))) break;
+      if ((rc = to_device(col, n, dev, &d_col, c, h->stream))) break;
+      if (dev) break;
+      d_out = c.take<float>(n);
+      if (pass == 0) rc = dalloc(&scratch, (int64_t)c.bytes);
+    }
+    if (rc) break;
     if ((rc = validate_pairs(h, d_row, d_col, n))) break;
     if ((rc = launch_predict(h, n, d_row, d_col, d_out))) break;
     if (!dev && cudaMemcpyAsync(out, d_out, sizeof(float) * n, cudaMemcpyDeviceToHost,
@@ -605,9 +628,10 @@ int bpmf_predict(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col, 
     }
     rc = check_status(h, "bpmf_predict");
   } while (0);
-  if (own_r) cudaFree(d_row);
-  if (own_c) cudaFree(d_col);
-  if (!dev) dfree(d_out);
+  if (scratch) {
+    cudaStreamSynchronize(h->stream);
+    dfree(scratch);
+  }
   return rc;
 }
 

@@ -179,20 +179,26 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
   }
   hub0.push_back((int32_t)prow.size());
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  cudaFree(sd.piece_row);
-  cudaFree(sd.piece_e0);
-  cudaFree(sd.piece_e1);
-  cudaFree(sd.hub_piece0);
-  sd.piece_row = nullptr;
-  sd.piece_e0 = sd.piece_e1 = nullptr;
-  sd.hub_piece0 = nullptr;
   sd.n_hub = n_hub;
   sd.n_pieces = (int64_t)prow.size();
-  const int64_t np = std::max<int64_t>(1, sd.n_pieces);
-  BPMF_CUDA_CHECK(cudaMalloc(&sd.piece_row, sizeof(int32_t) * np));
-  BPMF_CUDA_CHECK(cudaMalloc(&sd.piece_e0, sizeof(int64_t) * np));
-  BPMF_CUDA_CHECK(cudaMalloc(&sd.piece_e1, sizeof(int64_t) * np));
-  BPMF_CUDA_CHECK(cudaMalloc(&sd.hub_piece0, sizeof(int32_t) * (n_hub + 1)));
+  auto carve = [&](Carve& c) {
+    sd.piece_row = c.take<int32_t>(sd.n_pieces);
+    sd.piece_e0 = c.take<int64_t>(sd.n_pieces);
+    sd.piece_e1 = c.take<int64_t>(sd.n_pieces);
+    sd.hub_piece0 = c.take<int32_t>(n_hub + 1);
+  };
+  Carve size, c;
+  carve(size);
+  if ((int64_t)size.bytes > sd.piece_bytes) {
+    if (sd.piece_own) cudaFree(sd.piece_mem);
+    sd.piece_mem = nullptr;
+    sd.piece_bytes = 0;
+    sd.piece_own = true;
+    BPMF_CUDA_CHECK(cudaMalloc(&sd.piece_mem, size.bytes));
+    sd.piece_bytes = (int64_t)size.bytes;
+  }
+  c.base = sd.piece_mem;
+  carve(c);
   if (sd.n_pieces > 0) {
     BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_row, prow.data(), sizeof(int32_t) * sd.n_pieces,
                                     cudaMemcpyHostToDevice, st));
@@ -238,9 +244,6 @@ int setup_bins(Handle* h, int s) {
     sd.deg_h[q] = sd.ptr_h[r + 1] - sd.ptr_h[r];
     work[q] = make_int4(r, (int)sd.ptr_h[r], (int)sd.ptr_h[r + 1], 0);
   }
-  cudaFree(sd.work);
-  sd.work = nullptr;
-  BPMF_CUDA_CHECK(cudaMalloc(&sd.work, sizeof(int4) * work.size()));
   BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.work, work.data(), sizeof(int4) * work.size(),
                                   cudaMemcpyHostToDevice, st));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));

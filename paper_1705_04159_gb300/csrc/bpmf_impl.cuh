@@ -41,6 +41,21 @@ constexpr int kStatusValue = 16;   // an input rating is not finite
 // degree bins
 enum Bin { kBinTiny = 0, kBinLight = 1, kBinHeavy = 2, kBinHub = 3, kNumBins = 4 };
 
+// Arrays laid out one after the other in a block of device memory (256-byte
+// aligned); without a block it only adds up their bytes.  A device allocation
+// costs 53 us here whatever its size and a free 37 or more, so a sampler's arrays are
+// one allocation and the scratch of a call another.
+struct Carve {
+  char* base = nullptr;
+  size_t bytes = 0;
+  template <typename T>
+  T* take(int64_t n) {
+    T* p = base ? reinterpret_cast<T*>(base + bytes) : nullptr;
+    bytes += (sizeof(T) * (size_t)(n > 0 ? n : 1) + 255) & ~(size_t)255;
+    return p;
+  }
+};
+
 struct SideDev {
   int64_t R = 0;          // rows of this side
   int64_t* ptr = nullptr;
@@ -61,6 +76,9 @@ struct SideDev {
   float* linvT = nullptr;  // KP x (KP + 4), KP = K rounded up to 32: (L_s^-1)^T (tiny-row kernel)
   // split rows (hubs): pieces of at most kPiece ratings, in degree order
   int64_t n_hub = 0, n_pieces = 0;
+  char* piece_mem = nullptr;        // the four arrays below: piece_bytes of the sampler's block,
+  int64_t piece_bytes = 0;          // or, if they outgrew it, an allocation of their own
+  bool piece_own = false;
   int32_t* piece_row = nullptr;     // [n_pieces] row id
   int64_t* piece_e0 = nullptr;      // [n_pieces] first rating
   int64_t* piece_e1 = nullptr;      // [n_pieces] one past the last rating
@@ -91,6 +109,7 @@ struct Handle {
   int num_sms = 0;
   double mean = 0.0;
   SideDev side[2];
+  char* block = nullptr;    // the arrays of fixed size, here and in side[]
   double* mu0 = nullptr;    // K
   double* W0inv = nullptr;  // K*K
   // scratch
@@ -107,6 +126,7 @@ struct Handle {
   int32_t* flag_count = nullptr;
   // test set (sorted by user for gather locality)
   int64_t n_test = 0;
+  char* tblock = nullptr;    // the four arrays below
   int32_t* trow = nullptr;
   int32_t* tcol = nullptr;
   float* tval = nullptr;
@@ -241,16 +261,18 @@ __host__ __device__ __forceinline__ uint32_t stream_word(uint32_t stream, int si
 
 // ------------------------------------------------------------ launchers --
 // structure.cu
-int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val);
+// ws: structure_bytes(nnz, M, N) bytes of scratch
+size_t structure_bytes(int64_t nnz, int64_t M, int64_t N);
+int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val, void* ws);
 // stable LSD radix sort of (key, value) pairs by key into keys_out / vals_out;
 // keys_io / vals_io hold the input and serve as the other half of the
 // ping-pong pair (their contents are lost)
 int sort_pairs_u32(uint32_t* keys_io, int32_t* vals_io, uint32_t* keys_out, int32_t* vals_out,
-                   int64_t n, uint32_t max_key, cudaStream_t st);
-int order_rows_by_degree(Handle* h, int s);
+                   int64_t n, uint32_t max_key, Carve ws, cudaStream_t st);
 double device_mean(const float* d_val, int64_t n, double* d_red, cudaStream_t st, int* err);
-int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val,
-                  int64_t n, uint32_t* keys, uint32_t* keys_sorted, int32_t* ids, int32_t* src);
+size_t test_sort_bytes(int64_t n);  // scratch ws of sort_test_set
+int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val, int64_t n,
+                  void* ws);
 int validate_pairs(Handle* h, const int32_t* d_row, const int32_t* d_col, int64_t n);
 int setup_bins(Handle* h, int s);
 int autotune_bins(Handle* h, int s, float* scratch);  // binned.cu

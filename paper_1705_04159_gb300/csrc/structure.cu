@@ -131,23 +131,27 @@ __global__ void scan_add(int32_t* __restrict__ out, int64_t n, const int32_t* __
   }
 }
 
-int exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, cudaStream_t st) {
+// the block totals of each level, before and after their own scan
+void take_scan(Carve& c, int64_t n) {
+  for (; n > 1; ) {
+    n = (n + kScanTile - 1) / kScanTile;
+    c.take<int32_t>(n);
+    c.take<int32_t>(n);
+  }
+}
+
+int exclusive_scan_i32(const int32_t* in, int32_t* out, int64_t n, Carve ws, cudaStream_t st) {
   if (n <= 0) return BPMF_OK;
   const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-  int32_t* sums = nullptr;
-  int32_t* sums_scanned = nullptr;
-  BPMF_CUDA_CHECK(cudaMallocAsync(&sums, sizeof(int32_t) * tiles, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&sums_scanned, sizeof(int32_t) * tiles, st));
+  int32_t* sums = ws.take<int32_t>(tiles);
+  int32_t* sums_scanned = ws.take<int32_t>(tiles);
   scan_tiles<<<(unsigned)tiles, kScanThreads, 0, st>>>(in, out, n, sums);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (tiles > 1) {
-    int rc = exclusive_scan_i32(sums, sums_scanned, tiles, st);
-    if (rc != BPMF_OK) return rc;
+    BPMF_TRY(exclusive_scan_i32(sums, sums_scanned, tiles, ws, st));
     scan_add<<<(unsigned)tiles, kScanThreads, 0, st>>>(out, n, sums_scanned);
     BPMF_CUDA_CHECK(cudaGetLastError());
   }
-  BPMF_CUDA_CHECK(cudaFreeAsync(sums, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(sums_scanned, st));
   return BPMF_OK;
 }
 
@@ -257,24 +261,31 @@ unsigned grid_for(int64_t n, int threads) {
 
 }  // namespace
 
+// scratch of sort_pairs_u32 for n pairs
+void take_sort(Carve& c, int64_t n) {
+  const int64_t m = (int64_t)kRadix * ((n + kSortTile - 1) / kSortTile);
+  c.take<int32_t>(m);
+  c.take<int32_t>(m);
+  take_scan(c, m);
+}
+
 // Stable sort of (key, value) pairs by key, LSD with 8-bit digits; passes
 // stop once every key bit up to max_key has been consumed.
 int sort_pairs_u32(uint32_t* keys_io, int32_t* vals_io, uint32_t* keys_out, int32_t* vals_out,
-                   int64_t n, uint32_t max_key, cudaStream_t st) {
+                   int64_t n, uint32_t max_key, Carve ws, cudaStream_t st) {
   if (n <= 0) return BPMF_OK;
   int bits = 0;
   while (bits < 32 && (max_key >> bits) != 0u) ++bits;
   const int passes = bits == 0 ? 1 : (bits + 7) / 8;
   const int tiles = (int)((n + kSortTile - 1) / kSortTile);
   uint32_t *ka = keys_io, *kb = keys_out;
-  int32_t *va = vals_io, *vb = vals_out, *counts = nullptr, *offs = nullptr;
-  BPMF_CUDA_CHECK(cudaMallocAsync(&counts, sizeof(int32_t) * (int64_t)kRadix * tiles, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&offs, sizeof(int32_t) * (int64_t)kRadix * tiles, st));
+  int32_t *va = vals_io, *vb = vals_out;
+  int32_t* counts = ws.take<int32_t>((int64_t)kRadix * tiles);
+  int32_t* offs = ws.take<int32_t>((int64_t)kRadix * tiles);
   for (int p = 0; p < passes; ++p) {
     radix_hist<<<tiles, kSortThreads, 0, st>>>(ka, n, 8 * p, counts, tiles);
     BPMF_CUDA_CHECK(cudaGetLastError());
-    int rc = exclusive_scan_i32(counts, offs, (int64_t)kRadix * tiles, st);
-    if (rc != BPMF_OK) return rc;
+    BPMF_TRY(exclusive_scan_i32(counts, offs, (int64_t)kRadix * tiles, ws, st));
     radix_scatter<<<tiles, kSortThreads, 0, st>>>(ka, va, kb, vb, n, 8 * p, offs, tiles);
     BPMF_CUDA_CHECK(cudaGetLastError());
     std::swap(ka, kb);
@@ -285,8 +296,6 @@ int sort_pairs_u32(uint32_t* keys_io, int32_t* vals_io, uint32_t* keys_out, int3
     BPMF_CUDA_CHECK(cudaMemcpyAsync(keys_out, ka, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st));
     BPMF_CUDA_CHECK(cudaMemcpyAsync(vals_out, va, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st));
   }
-  BPMF_CUDA_CHECK(cudaFreeAsync(counts, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(offs, st));
   return BPMF_OK;
 }
 
@@ -305,37 +314,58 @@ double device_mean(const float* d_val, int64_t n, double* d_red, cudaStream_t st
   return m;
 }
 
-int order_rows_by_degree(Handle* h, int s) {
+namespace {
+
+int order_rows_by_degree(Handle* h, int s, Carve ws) {
   SideDev& sd = h->side[s];
   cudaStream_t st = h->stream;
   const int64_t R = sd.R;
-  unsigned long long* dmax = nullptr;
-  BPMF_CUDA_CHECK(cudaMallocAsync(&dmax, sizeof(unsigned long long), st));
+  unsigned long long* dmax = ws.take<unsigned long long>(1);
   BPMF_CUDA_CHECK(cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), st));
   max_degree<<<grid_for(R, 256), 256, 0, st>>>(sd.ptr, R, dmax);
   BPMF_CUDA_CHECK(cudaGetLastError());
   unsigned long long maxdeg = 0;
   BPMF_CUDA_CHECK(cudaMemcpyAsync(&maxdeg, dmax, sizeof(maxdeg), cudaMemcpyDeviceToHost, st));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(dmax, st));
   sd.max_deg = (int64_t)maxdeg;
-  uint32_t* keys = nullptr;
-  uint32_t* keys_sorted = nullptr;
-  int32_t* ids = nullptr;
-  BPMF_CUDA_CHECK(cudaMallocAsync(&keys, sizeof(uint32_t) * R, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&keys_sorted, sizeof(uint32_t) * R, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&ids, sizeof(int32_t) * R, st));
+  uint32_t* keys = ws.take<uint32_t>(R);
+  uint32_t* keys_sorted = ws.take<uint32_t>(R);
+  int32_t* ids = ws.take<int32_t>(R);
   degree_keys<<<grid_for(R, 256), 256, 0, st>>>(sd.ptr, R, (uint32_t)maxdeg, keys);
   iota_i32<<<grid_for(R, 256), 256, 0, st>>>(ids, R);
   BPMF_CUDA_CHECK(cudaGetLastError());
-  BPMF_TRY(sort_pairs_u32(keys, ids, keys_sorted, sd.perm, R, (uint32_t)maxdeg, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(keys, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(keys_sorted, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(ids, st));
-  return BPMF_OK;
+  return sort_pairs_u32(keys, ids, keys_sorted, sd.perm, R, (uint32_t)maxdeg, ws, st);
 }
 
-int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val) {
+struct EntrySort {
+  uint32_t *keys, *keys_sorted;
+  int32_t *ids, *src;
+};
+EntrySort take_entries(Carve& c, int64_t n) {
+  EntrySort e;
+  e.keys = c.take<uint32_t>(n);
+  e.keys_sorted = c.take<uint32_t>(n);
+  e.ids = c.take<int32_t>(n);
+  e.src = c.take<int32_t>(n);
+  return e;
+}
+
+}  // namespace
+
+size_t structure_bytes(int64_t nnz, int64_t M, int64_t N) {
+  // the entries, then the sort of either the entries or a side's rows
+  const int64_t R = std::max(M, N);
+  Carve a, b;
+  take_sort(a, nnz);
+  b.take<unsigned long long>(1);
+  for (int i = 0; i < 3; ++i) b.take<uint32_t>(R);
+  take_sort(b, R);
+  Carve c;
+  take_entries(c, nnz);
+  return c.bytes + std::max(a.bytes, b.bytes);
+}
+
+int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val, void* mem) {
   cudaStream_t st = h->stream;
   const int64_t nnz = h->nnz;
   if (nnz > 0) {
@@ -356,36 +386,26 @@ int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const
   h->mean = device_mean(d_val, nnz, h->red, st, &err);
   if (err != BPMF_OK) return err;
 
-  uint32_t* keys = nullptr;
-  uint32_t* keys_sorted = nullptr;
-  int32_t* ids = nullptr;
-  int32_t* src = nullptr;
-  const int64_t n_alloc = nnz > 0 ? nnz : 1;
-  BPMF_CUDA_CHECK(cudaMallocAsync(&keys, sizeof(uint32_t) * n_alloc, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&keys_sorted, sizeof(uint32_t) * n_alloc, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&ids, sizeof(int32_t) * n_alloc, st));
-  BPMF_CUDA_CHECK(cudaMallocAsync(&src, sizeof(int32_t) * n_alloc, st));
+  Carve ws;
+  ws.base = static_cast<char*>(mem);
+  const EntrySort t = take_entries(ws, nnz);
   for (int s = 0; s < 2; ++s) {
     SideDev& sd = h->side[s];
     const int32_t* key = s == BPMF_USERS ? d_row : d_col;
     const int32_t* other = s == BPMF_USERS ? d_col : d_row;
     if (nnz > 0) {
-      gather_keys<<<grid_for(nnz, 256), 256, 0, st>>>(key, keys, nnz);
-      iota_i32<<<grid_for(nnz, 256), 256, 0, st>>>(ids, nnz);
+      gather_keys<<<grid_for(nnz, 256), 256, 0, st>>>(key, t.keys, nnz);
+      iota_i32<<<grid_for(nnz, 256), 256, 0, st>>>(t.ids, nnz);
       BPMF_CUDA_CHECK(cudaGetLastError());
-      BPMF_TRY(sort_pairs_u32(keys, ids, keys_sorted, src, nnz, (uint32_t)(sd.R - 1), st));
-      gather_entries<<<grid_for(nnz, 256), 256, 0, st>>>(src, other, d_val, h->mean, sd.idx,
+      BPMF_TRY(sort_pairs_u32(t.keys, t.ids, t.keys_sorted, t.src, nnz, (uint32_t)(sd.R - 1), ws, st));
+      gather_entries<<<grid_for(nnz, 256), 256, 0, st>>>(t.src, other, d_val, h->mean, sd.idx,
                                                           sd.val, nnz);
       BPMF_CUDA_CHECK(cudaGetLastError());
     }
-    row_pointers<<<grid_for(sd.R + 1, 256), 256, 0, st>>>(keys_sorted, nnz, sd.R, sd.ptr);
+    row_pointers<<<grid_for(sd.R + 1, 256), 256, 0, st>>>(t.keys_sorted, nnz, sd.R, sd.ptr);
     BPMF_CUDA_CHECK(cudaGetLastError());
-    BPMF_TRY(order_rows_by_degree(h, s));
+    BPMF_TRY(order_rows_by_degree(h, s, ws));
   }
-  BPMF_CUDA_CHECK(cudaFreeAsync(keys, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(keys_sorted, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(ids, st));
-  BPMF_CUDA_CHECK(cudaFreeAsync(src, st));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
   return BPMF_OK;
 }
@@ -417,8 +437,18 @@ int validate_pairs(Handle* h, const int32_t* d_row, const int32_t* d_col, int64_
   return BPMF_OK;
 }
 
-int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val,
-                  int64_t n, uint32_t* keys, uint32_t* keys_sorted, int32_t* ids, int32_t* src) {
+size_t test_sort_bytes(int64_t n) {
+  Carve c;
+  take_entries(c, n);
+  take_sort(c, n);
+  return c.bytes;
+}
+
+int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val, int64_t n,
+                  void* mem) {
+  Carve ws;
+  ws.base = static_cast<char*>(mem);
+  const EntrySort t = take_entries(ws, n);
   cudaStream_t st = h->stream;
   BPMF_TRY(validate_pairs(h, d_row, d_col, n));
   check_finite<<<grid_for(n, 256), 256, 0, st>>>(d_val, n, h->status);
@@ -432,11 +462,11 @@ int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const f
                                   : "bpmf_set_test: a test rating is not finite");
     return BPMF_EINVAL;
   }
-  gather_keys<<<grid_for(n, 256), 256, 0, st>>>(d_row, keys, n);
-  iota_i32<<<grid_for(n, 256), 256, 0, st>>>(ids, n);
+  gather_keys<<<grid_for(n, 256), 256, 0, st>>>(d_row, t.keys, n);
+  iota_i32<<<grid_for(n, 256), 256, 0, st>>>(t.ids, n);
   BPMF_CUDA_CHECK(cudaGetLastError());
-  BPMF_TRY(sort_pairs_u32(keys, ids, keys_sorted, src, n, (uint32_t)(h->M - 1), st));
-  gather_test<<<grid_for(n, 256), 256, 0, st>>>(src, d_row, d_col, d_val, h->trow, h->tcol,
+  BPMF_TRY(sort_pairs_u32(t.keys, t.ids, t.keys_sorted, t.src, n, (uint32_t)(h->M - 1), ws, st));
+  gather_test<<<grid_for(n, 256), 256, 0, st>>>(t.src, d_row, d_col, d_val, h->trow, h->tcol,
                                                  h->tval, n);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
