@@ -695,8 +695,7 @@ int bpmf_set_state(bpmf_t* hh, const float* U, const float* V, const double* hyp
                                       cudaMemcpyHostToDevice, h->stream));
       BPMF_CUDA_CHECK(cudaMemcpyAsync(h->side[s].mu, base + KK, sizeof(double) * K,
                                       cudaMemcpyHostToDevice, h->stream));
-      BPMF_TRY(launch_check_spd_f64(h->side[s].lam, K, h->wscr, h->status, h->side[s].lchol,
-                                    h->stream));
+      BPMF_TRY(launch_check_spd_f64(h->side[s].lam, K, h->status, h->side[s].lchol, h->stream));
       BPMF_TRY(launch_hyper_to_f32(h, s));
     }
     const int rc = check_status(h, "bpmf_set_state");

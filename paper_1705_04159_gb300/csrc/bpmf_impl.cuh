@@ -284,8 +284,7 @@ int set_thresholds(Handle* h, int s, const int64_t t[5]);  // binned.cu
 int launch_hyper(Handle* h, int s, cudaStream_t st = nullptr, bool alt = false);
 int launch_spd_inverse_f64(const double* A, double* Ainv, int K, double* scratch, int* status,
                            cudaStream_t st);
-int launch_check_spd_f64(const double* A, int K, double* scratch, int* status, float* lout,
-                         cudaStream_t st);
+int launch_check_spd_f64(const double* A, int K, int* status, float* lout, cudaStream_t st);
 int launch_hyper_to_f32(Handle* h, int s);
 int launch_stats_into(const float* X, int64_t R, int K, double* part, int blocks, double* xbar,
                       double* S, float* xbarf, cudaStream_t st);

@@ -314,112 +314,6 @@ __global__ void __launch_bounds__(32 * kFinalWarps) scatter_final(
   }
 }
 
-// ---- FP64 dense algebra by one CTA on row-major K x K matrices in global
-// scratch, for the prior and for hyperparameters that are set.  Every helper
-// starts and ends with the block synchronised.
-
-// In-place lower Cholesky (upper part zeroed), right-looking by columns.
-// Returns false (to all threads) if a pivot is not positive.  FP64 roots and
-// divisions are long chains of FP64 instructions, so each pivot takes one
-// reciprocal square root r = piv^-1/2 (L_kk = piv r, the column is scaled by
-// r) by one thread, and it is taken ahead: in the trailing update of column
-// k, warp 0 first updates A[k+1][k+1] (the only entry of row k + 1 that
-// column k changes) and its lane 0 forms the next pivot while the other warps
-// update the remaining rows.  Two barriers per column.
-__device__ bool cta_cholesky(double* A, int K, int* bad) {
-  __shared__ double s_rd[2];
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nt >> 5;
-  auto pivot = [&](int k) {  // one thread
-    const double piv = A[k * K + k];
-    const bool ok = piv > 0.0;
-    const double r = ok ? rsqrt(piv) : 1.0;
-    if (!ok) *bad = 1;
-    A[k * K + k] = ok ? piv * r : 1.0;
-    s_rd[k & 1] = r;
-  };
-  if (tid == 0) {
-    *bad = 0;
-    if (K > 0) pivot(0);
-  }
-  __syncthreads();
-  // warp 0 takes the last row of each round of the trailing update
-  const int slot = (w + nw - 1) % nw;
-  for (int k = 0; k < K; ++k) {
-    const double rd = s_rd[k & 1];
-    for (int i = k + 1 + tid; i < K; i += nt) A[i * K + k] *= rd;
-    __syncthreads();
-    if (w == 0 && k + 1 < K) {
-      if (lane == 0) {
-        const double l = A[(k + 1) * K + k];
-        A[(k + 1) * K + k + 1] = fma(-l, l, A[(k + 1) * K + k + 1]);
-        pivot(k + 1);
-      }
-      __syncwarp();
-    }
-    // the rest of the trailing update of the lower triangle, a warp per row
-    for (int i = k + 2 + slot; i < K; i += nw) {
-      const double aik = A[i * K + k];
-      for (int j = k + 1 + lane; j <= i; j += 32)
-        A[i * K + j] = fma(-aik, A[j * K + k], A[i * K + j]);
-    }
-    __syncthreads();
-  }
-  for (int e = tid; e < K * K; e += nt) {
-    const int i = e / K, j = e % K;
-    if (j > i) A[i * K + j] = 0.0;
-  }
-  __syncthreads();
-  const bool ok = *bad == 0;
-  __syncthreads();
-  return ok;
-}
-
-// Four-way split sum of p[k] q[k] (strides sp, sq) over k = 0 .. n-1: four
-// independent chains instead of one.
-__device__ __forceinline__ double dot4(const double* p, int sp, const double* q, int sq, int n) {
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-  int k = 0;
-  for (; k + 4 <= n; k += 4) {
-    s0 = fma(p[k * sp], q[k * sq], s0);
-    s1 = fma(p[(k + 1) * sp], q[(k + 1) * sq], s1);
-    s2 = fma(p[(k + 2) * sp], q[(k + 2) * sq], s2);
-    s3 = fma(p[(k + 3) * sp], q[(k + 3) * sq], s3);
-  }
-  for (; k < n; ++k) s0 = fma(p[k * sp], q[k * sq], s0);
-  return (s0 + s1) + (s2 + s3);
-}
-
-// Linv = L^-1 for lower-triangular L: thread j solves column j by forward
-// substitution.
-__device__ void cta_tri_inverse(const double* L, double* Linv, int K) {
-  __shared__ double rdiag[kMaxK];  // 1 / L_ii, one division per row
-  for (int i = threadIdx.x; i < K; i += blockDim.x) rdiag[i] = 1.0 / L[i * K + i];
-  __syncthreads();
-  for (int j = threadIdx.x; j < K; j += blockDim.x) {
-    for (int i = 0; i < K; ++i) {
-      double v;
-      if (i < j) v = 0.0;
-      else {
-        const double t = (i == j ? 1.0 : 0.0) - dot4(L + i * K + j, 1, Linv + j * K + j, K, i - j);
-        v = t * rdiag[i];
-      }
-      Linv[i * K + j] = v;
-    }
-  }
-  __syncthreads();
-}
-
-// C = A^T A (symmetric)
-__device__ void cta_ata(const double* A, double* C, int K) {
-  for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-    const int i = e / K, j = e % K;
-    double s = 0.0;
-    for (int k = 0; k < K; ++k) s += A[k * K + i] * A[k * K + j];
-    C[e] = s;
-  }
-  __syncthreads();
-}
-
 // FP32 copy of Lambda bordered by b0 = Lambda mu: the (K+1) x (K+1) matrix
 // [[Lambda, b0], [b0^T, 0]] that the row kernels add alpha times the
 // rating-augmented Gram to.
@@ -460,40 +354,6 @@ __device__ void write_bordered(const double* lam, const double* mu, int K, float
   }
   if (threadIdx.x == 0) out[K * KA + K] = 0.f;
   __syncthreads();
-}
-
-// Ainv = A^-1 for SPD A (used once for W0^-1); flags kStatusNotPD.
-__global__ void __launch_bounds__(512) spd_inverse_kernel(const double* A, double* Ainv, int K,
-                                                          double* scr, int* status) {
-  __shared__ int bad;
-  const int KK = K * K;
-  double* L = scr;
-  double* Li = scr + KK;
-  for (int e = threadIdx.x; e < KK; e += blockDim.x) L[e] = A[e];
-  __syncthreads();
-  if (!cta_cholesky(L, K, &bad)) {
-    if (threadIdx.x == 0) atomicOr(status, kStatusNotPD);
-    return;
-  }
-  cta_tri_inverse(L, Li, K);
-  cta_ata(Li, Ainv, K);
-}
-
-// Checks that A is SPD; on success writes chol(A) in FP32 to lout (lower
-// triangle packed by rows: element (i, j) at i (i + 1) / 2 + j).
-__global__ void __launch_bounds__(512) spd_check_kernel(const double* A, int K, double* scr,
-                                                        int* status, float* lout) {
-  __shared__ int bad;
-  for (int e = threadIdx.x; e < K * K; e += blockDim.x) scr[e] = A[e];
-  __syncthreads();
-  if (!cta_cholesky(scr, K, &bad)) {
-    if (threadIdx.x == 0) atomicOr(status, kStatusNotPD);
-    return;
-  }
-  for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-    const int i = e / K, j = e % K;
-    if (j <= i) lout[i * (i + 1) / 2 + j] = (float)scr[e];
-  }
 }
 
 // float copies of a side's hyperparameters (after bpmf_set_state)
@@ -600,20 +460,6 @@ int launch_stats_into(const float* X, int64_t R, int K, double* part, int blocks
   BPMF_TRY(launch_scatter(X, R, K, xbarf, part, blocks, st));
   scatter_final<<<(K * K + kFinalWarps - 1) / kFinalWarps, 32 * kFinalWarps, 0, st>>>(part, blocks,
                                                                                      K, S);
-  BPMF_CUDA_CHECK(cudaGetLastError());
-  return BPMF_OK;
-}
-
-int launch_spd_inverse_f64(const double* A, double* Ainv, int K, double* scratch, int* status,
-                           cudaStream_t st) {
-  spd_inverse_kernel<<<1, 512, 0, st>>>(A, Ainv, K, scratch, status);
-  BPMF_CUDA_CHECK(cudaGetLastError());
-  return BPMF_OK;
-}
-
-int launch_check_spd_f64(const double* A, int K, double* scratch, int* status, float* lout,
-                         cudaStream_t st) {
-  spd_check_kernel<<<1, 512, 0, st>>>(A, K, scratch, status, lout);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
 }
