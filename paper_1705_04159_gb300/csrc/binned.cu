@@ -238,15 +238,10 @@ int setup_bins(Handle* h, int s) {
   BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.perm_h.data(), sd.perm, sizeof(int32_t) * R,
                                   cudaMemcpyDeviceToHost, st));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  std::vector<int4> work(R > 0 ? R : 1);
   for (int64_t q = 0; q < R; ++q) {
     const int32_t r = sd.perm_h[q];
     sd.deg_h[q] = sd.ptr_h[r + 1] - sd.ptr_h[r];
-    work[q] = make_int4(r, (int)sd.ptr_h[r], (int)sd.ptr_h[r + 1], 0);
   }
-  BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.work, work.data(), sizeof(int4) * work.size(),
-                                  cudaMemcpyHostToDevice, st));
-  BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
   sd.hub_min = 0;  // forces the pieces to be built
   sd.heavy_tc = h->cfg.heavy_kernel == 2 && tc_supported(h->K);
   sd.ws_nb = ws_stage_neighbours(R > 0 ? sd.ptr_h[R] : 0, R);

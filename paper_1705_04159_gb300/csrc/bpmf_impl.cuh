@@ -269,7 +269,6 @@ int build_structure(Handle* h, const int32_t* d_row, const int32_t* d_col, const
 // ping-pong pair (their contents are lost)
 int sort_pairs_u32(uint32_t* keys_io, int32_t* vals_io, uint32_t* keys_out, int32_t* vals_out,
                    int64_t n, uint32_t max_key, Carve ws, cudaStream_t st);
-double device_mean(const float* d_val, int64_t n, double* d_red, cudaStream_t st, int* err);
 size_t test_sort_bytes(int64_t n);  // scratch ws of sort_test_set
 int sort_test_set(Handle* h, const int32_t* d_row, const int32_t* d_col, const float* d_val, int64_t n,
                   void* ws);
