@@ -619,7 +619,6 @@ int bpmf_predict(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col, 
       if (pass == 0) rc = dalloc(&scratch, (int64_t)c.bytes);
     }
     if (rc) break;
-    if ((rc = validate_pairs(h, d_row, d_col, n))) break;
     if ((rc = launch_predict(h, n, d_row, d_col, d_out))) break;
     if (!dev && cudaMemcpyAsync(out, d_out, sizeof(float) * n, cudaMemcpyDeviceToHost,
                                 h->stream) != cudaSuccess) {

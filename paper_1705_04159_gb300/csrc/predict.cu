@@ -1,16 +1,21 @@
 // predict.cu -- test predictions (Algorithm 1, "for all test points:
 // predict rating and compute RMSE").
 //
-// r_hat = u_row . v_col + mean.  A warp takes 32 pairs at a time, G lanes per
-// pair (4 for K <= 64, else 8) in G rounds of 32 / G pairs: lane l of a group
-// reads the 16-byte chunks l, l + G, .. of both factor rows, so each row is
-// read by coalesced requests, and the partial sums meet in a butterfly of
-// shuffles; lane L then takes the product of pair L, so that the per-pair
-// arithmetic after the dot product runs on every lane.  The registered test
-// set is sorted by user at registration, so neighbouring pairs share the user
-// row through L1.  The squared errors of the latest sample and of the
-// running mean of predictions are summed per lane in FP32, per block in FP64
-// and combined in block order (deterministic).
+// r_hat = u_row . v_col + mean.  A warp takes 32 pairs at a time, a lane
+// loading the ids of each, then G lanes per pair (4 for K <= 64, else 8) in G
+// rounds of 32 / G pairs: lane l of a group reads the 16-byte chunks l, l + G,
+// .. of both factor rows, so each row is read by coalesced requests, and the
+// partial sums meet in a butterfly of shuffles; lane L then takes the product
+// of pair L, so that the per-pair arithmetic after the dot product runs on
+// every lane.  The registered test set is sorted by user at registration, so
+// neighbouring pairs share the user row through L1.  The squared errors of the
+// latest sample and of the running mean of predictions are summed per lane in
+// FP32, per block in FP64 and combined in block order (deterministic).
+// What bounds it: the rows' way from L2 to the SMs, 800 bytes a pair at K = 100.
+// 4,000,000 random pairs of 480,189 x 17,770: 478 us with the ids loaded in
+// each round; 264 with two rounds' loads in flight and registers cut for four
+// CTAs an SM (three 311, five 304, six 442; one round 268, four 281); 246,
+// 13 TB/s, with the range check in the kernel instead of a pass of its own.
 #include <cuda_runtime.h>
 
 #include "bpmf_impl.cuh"
@@ -25,58 +30,53 @@ constexpr int kPredWarps = kPredThreads / 32;
 int pred_group(int K) { return K <= 64 ? 4 : 8; }
 
 // u . v over the group of G lanes holding `sub` = lane % G; every lane of the
-// warp must call it (the shuffles span the warp); lanes with !ok read nothing
-// and add zero.  Rows are 16-byte aligned when K % 4 == 0 (VEC).
+// warp must call it (the shuffles span the warp).  Rows are 16-byte aligned
+// when K % 4 == 0 (VEC).
 template <int G, bool VEC>
 __device__ __forceinline__ float pair_dot(const float* __restrict__ u, const float* __restrict__ v,
-                                          int K, int sub, bool ok) {
+                                          int K, int sub) {
   float s = 0.f;
-  if (ok) {
-    if (VEC) {
-      const float4* a = reinterpret_cast<const float4*>(u);
-      const float4* b = reinterpret_cast<const float4*>(v);
-      const int nc = K >> 2;
-      float4 x[4], y[4];
+  if (VEC) {
+    const float4* a = reinterpret_cast<const float4*>(u);
+    const float4* b = reinterpret_cast<const float4*>(v);
+    const int nc = K >> 2;
+    float4 x[4], y[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int c = sub + i * G;
-        x[i] = c < nc ? __ldg(a + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        y[i] = c < nc ? __ldg(b + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        s = fmaf(x[i].x, y[i].x, s);
-        s = fmaf(x[i].y, y[i].y, s);
-        s = fmaf(x[i].z, y[i].z, s);
-        s = fmaf(x[i].w, y[i].w, s);
-      }
-    } else {
-      for (int k = sub; k < K; k += G) s = fmaf(__ldg(u + k), __ldg(v + k), s);
+    for (int i = 0; i < 4; ++i) {
+      const int c = sub + i * G;
+      x[i] = c < nc ? __ldg(a + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+      y[i] = c < nc ? __ldg(b + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s = fmaf(x[i].x, y[i].x, s);
+      s = fmaf(x[i].y, y[i].y, s);
+      s = fmaf(x[i].z, y[i].z, s);
+      s = fmaf(x[i].w, y[i].w, s);
+    }
+  } else {
+    for (int k = sub; k < K; k += G) s = fmaf(__ldg(u + k), __ldg(v + k), s);
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
 }
 
-// u_row . v_col of pairs p0 .. p0 + 31 by one warp; lane L returns that of
-// pair p0 + L (0 past n).  Pair p0 + L is done in round L / P by group L % P,
-// all of whose lanes hold the total after the butterfly.
+// u_r . v_c of 32 pairs by one warp, lane L holding the ids r, c of pair L (any
+// row if it has none: its product is not used); lane L returns its product.
+// Pair L is done in round L / P by group L % P, all of whose lanes hold the
+// total after the butterfly.
 template <int G, bool VEC>
 __device__ __forceinline__ float warp_dots(const float* __restrict__ U, const float* __restrict__ V,
-                                           int K, const int32_t* __restrict__ row,
-                                           const int32_t* __restrict__ col, int64_t p0, int64_t n,
-                                           int lane) {
+                                           int K, int r, int c, int lane) {
   constexpr int P = 32 / G;
   const int sub = lane & (G - 1), grp = lane / G;
   float mine = 0.f;
-#pragma unroll
+#pragma unroll 2
   for (int round = 0; round < G; ++round) {
-    const int64_t p = p0 + round * P + grp;
-    const bool ok = p < n;
-    const float* u = ok ? U + (int64_t)row[p] * K : U;
-    const float* v = ok ? V + (int64_t)col[p] * K : V;
-    const float s = pair_dot<G, VEC>(u, v, K, sub, ok);
+    const int rr = __shfl_sync(0xffffffffu, r, round * P + grp);
+    const int cc = __shfl_sync(0xffffffffu, c, round * P + grp);
+    const float s = pair_dot<G, VEC>(U + (int64_t)rr * K, V + (int64_t)cc * K, K, sub);
     const float t = __shfl_sync(0xffffffffu, s, (lane % P) * G);
     if (lane / P == round) mine = t;
   }
@@ -84,16 +84,23 @@ __device__ __forceinline__ float warp_dots(const float* __restrict__ U, const fl
 }
 
 template <int G, bool VEC>
-__global__ void __launch_bounds__(kPredThreads) predict_pairs(
-    const float* __restrict__ U, const float* __restrict__ V, int K, double mean,
+__global__ void __launch_bounds__(kPredThreads, 4) predict_pairs(
+    const float* __restrict__ U, const float* __restrict__ V, int M, int N, int K, double mean,
     const int32_t* __restrict__ row, const int32_t* __restrict__ col, int64_t n,
-    float* __restrict__ out) {
+    float* __restrict__ out, int* __restrict__ status) {
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t p0 = w0 * 32; p0 < n; p0 += nw * 32) {
-    const float s = warp_dots<G, VEC>(U, V, K, row, col, p0, n, lane);
-    if (p0 + lane < n) out[p0 + lane] = (float)((double)s + mean);
+    const int64_t p = p0 + lane;
+    const bool ok = p < n;
+    int i = ok ? __ldg(row + p) : 0, j = ok ? __ldg(col + p) : 0;
+    if ((unsigned)i >= (unsigned)M || (unsigned)j >= (unsigned)N) {
+      atomicOr(status, kStatusIndex);
+      i = j = 0;
+    }
+    const float s = warp_dots<G, VEC>(U, V, K, i, j, lane);
+    if (ok) out[p] = (float)((double)s + mean);
   }
 }
 
@@ -110,7 +117,7 @@ __device__ __forceinline__ float2 pair_add(float2 s, float x) {
 }
 
 template <int G, bool VEC>
-__global__ void __launch_bounds__(kPredThreads) test_errors(
+__global__ void __launch_bounds__(kPredThreads, 4) test_errors(
     const float* __restrict__ U, const float* __restrict__ V, int K, double mean,
     const int32_t* __restrict__ row, const int32_t* __restrict__ col,
     const float* __restrict__ truth, int64_t n, float2* __restrict__ sum,
@@ -128,14 +135,15 @@ __global__ void __launch_bounds__(kPredThreads) test_errors(
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t p0 = w0 * 32; p0 < n; p0 += nw * 32) {
-    const float s = warp_dots<G, VEC>(U, V, K, row, col, p0, n, lane);
     const int64_t p = p0 + lane;
-    if (p < n) {
+    const bool ok = p < n;
+    const float t = ok ? truth[p] : 0.f;
+    float2 acc = ok ? sum[p] : make_float2(0.f, 0.f);
+    const float s = warp_dots<G, VEC>(U, V, K, ok ? __ldg(row + p) : 0, ok ? __ldg(col + p) : 0, lane);
+    if (ok) {
       const float pred = s + meanf;
-      const float t = truth[p];
       const float d = pred - t;
       f1 = fmaf(d, d, f1);
-      float2 acc = sum[p];
       if (accumulate) {
         acc = pair_add(acc, pred);
         sum[p] = acc;
@@ -206,13 +214,9 @@ int launch_predict(Handle* h, int64_t n, const int32_t* r, const int32_t* c, flo
   const float* U = h->side[BPMF_USERS].X;
   const float* V = h->side[BPMF_MOVIES].X;
   const bool vec = (K & 3) == 0;
-  if (g == 4) {
-    if (vec) predict_pairs<4, true><<<b, kPredThreads, 0, h->stream>>>(U, V, K, h->mean, r, c, n, out);
-    else predict_pairs<4, false><<<b, kPredThreads, 0, h->stream>>>(U, V, K, h->mean, r, c, n, out);
-  } else {
-    if (vec) predict_pairs<8, true><<<b, kPredThreads, 0, h->stream>>>(U, V, K, h->mean, r, c, n, out);
-    else predict_pairs<8, false><<<b, kPredThreads, 0, h->stream>>>(U, V, K, h->mean, r, c, n, out);
-  }
+  auto kern = g == 4 ? (vec ? predict_pairs<4, true> : predict_pairs<4, false>)
+                     : (vec ? predict_pairs<8, true> : predict_pairs<8, false>);
+  kern<<<b, kPredThreads, 0, h->stream>>>(U, V, (int)h->M, (int)h->N, K, h->mean, r, c, n, out, h->status);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
 }
