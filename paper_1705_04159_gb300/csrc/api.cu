@@ -113,9 +113,12 @@ void carve_handle(Handle* h, Carve& c) {
   h->W0inv = c.take<double>(KK);
   h->flag_rows = c.take<int32_t>(std::max(h->M, h->N));
   h->terr = c.take<double>(2);
-  h->flag_count = c.take<int32_t>(1);
-  h->ws_counter = c.take<int>(1);
   h->status = c.take<int>(1);
+  h->flag_count = c.take<int32_t>(1);
+  h->redo_count = c.take<int32_t>(1);
+  h->redo_ticket = c.take<int>(1);
+  h->test_ticket = c.take<int>(1);
+  h->ws_counter = c.take<int>(1);
   h->d_iter = c.take<uint32_t>(1);
   h->d_navg = c.take<int64_t>(1);
 }
@@ -168,7 +171,7 @@ int sweep_one(Handle* h, int s) {
 
 int read_fp64_rows(Handle* h, int s) {
   int32_t n = 0;
-  BPMF_CUDA_CHECK(cudaMemcpyAsync(&n, h->flag_count, sizeof(int32_t), cudaMemcpyDeviceToHost,
+  BPMF_CUDA_CHECK(cudaMemcpyAsync(&n, h->redo_count, sizeof(int32_t), cudaMemcpyDeviceToHost,
                                   h->stream));
   BPMF_CUDA_CHECK(cudaStreamSynchronize(h->stream));
   h->side[s].fp64_rows = n;
@@ -205,8 +208,7 @@ int step_body(Handle* h) {
   }
   if (rc != BPMF_OK) return rc;
   BPMF_TRY(sweep_one(h, second));
-  BPMF_TRY(launch_test_step(h));
-  return launch_advance_iter(h);
+  return h->n_test > 0 ? launch_test_step(h) : launch_advance_iter(h);
 }
 
 // Records step_body into an executable graph.  The capture runs on a private

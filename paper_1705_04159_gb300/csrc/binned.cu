@@ -300,14 +300,14 @@ int time_sweep(Handle* h, int s, float* scratch, int reps, float* best_ms) {
     SweepArgs a = make_sweep_args(h, s);
     a.X = scratch;
     a.Xhi = a.Xlo = nullptr;
-    if (cudaMemsetAsync(h->flag_count, 0, sizeof(int32_t), h->stream) != cudaSuccess ||
-        cudaEventRecord(e0, h->stream) != cudaSuccess)
-      rc = BPMF_ECUDA;
+    if (cudaEventRecord(e0, h->stream) != cudaSuccess) rc = BPMF_ECUDA;
     if (rc == BPMF_OK) {
       if (h->cfg.path == BPMF_PATH_PLAIN) rc = launch_rows_fp32(a, h->stream, &h->kernels);
       else rc = launch_sweep_binned(h, s, a);
     }
     if (rc == BPMF_OK && cudaEventRecord(e1, h->stream) != cudaSuccess) rc = BPMF_ECUDA;
+    const int cleared = clear_sweep_counts(h);
+    if (rc == BPMF_OK) rc = cleared;
     if (rc == BPMF_OK && cudaEventSynchronize(e1) != cudaSuccess) rc = BPMF_ECUDA;
     float ms = 0.f;
     if (rc == BPMF_OK && cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) rc = BPMF_ECUDA;

@@ -123,7 +123,10 @@ struct Handle {
   double* wscr2 = nullptr;
   int* status = nullptr;    // device status word
   int32_t* flag_rows = nullptr;  // rows flagged for the FP64 redo (max R over sides)
-  int32_t* flag_count = nullptr;
+  int32_t* flag_count = nullptr;  // zero between sweeps (the redo takes it back)
+  int32_t* redo_count = nullptr;  // rows the last sweep redid
+  int* redo_ticket = nullptr;     // blocks of the redo, and of the test step, that have
+  int* test_ticket = nullptr;     // arrived; zero between launches
   // test set (sorted by user for gather locality)
   int64_t n_test = 0;
   char* tblock = nullptr;    // the four arrays below
@@ -290,6 +293,7 @@ int launch_stats_into(const float* X, int64_t R, int K, double* part, int blocks
 
 // rows.cu
 int launch_sweep(Handle* h, int s);
+int clear_sweep_counts(Handle* h);  // after a sweep whose FP64 redo was not launched
 int launch_init_factors(Handle* h, int s);
 int launch_refresh_shadow(Handle* h, int s);
 

@@ -121,9 +121,10 @@ __global__ void __launch_bounds__(kPredThreads, 4) test_errors(
     const float* __restrict__ U, const float* __restrict__ V, int K, double mean,
     const int32_t* __restrict__ row, const int32_t* __restrict__ col,
     const float* __restrict__ truth, int64_t n, float2* __restrict__ sum,
-    const uint32_t* __restrict__ tp, int64_t burnin, const int64_t* __restrict__ navg,
-    double* __restrict__ part) {
+    uint32_t* __restrict__ tp, int64_t burnin, int64_t* __restrict__ navg,
+    double* __restrict__ part, double* __restrict__ out, int* __restrict__ ticket) {
   __shared__ double es[kPredWarps], em[kPredWarps];
+  __shared__ bool s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // samples after burn-in enter the running mean; the count is read on the
   // device so that one captured iteration serves every iteration
@@ -171,19 +172,22 @@ __global__ void __launch_bounds__(kPredThreads, 4) test_errors(
     }
     part[2 * blockIdx.x] = a;
     part[2 * blockIdx.x + 1] = b;
+    __threadfence();
+    s_last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
   }
-}
-
-__global__ void test_final(const double* __restrict__ part, int blocks, int64_t n,
-                           double* __restrict__ out, const uint32_t* __restrict__ tp,
-                           int64_t burnin, int64_t* __restrict__ navg) {
-  // lane l sums blocks l, l + 32, ..; the 32 partial sums are combined by a
-  // fixed shuffle tree, so the order never depends on timing
-  const int lane = threadIdx.x;
+  __syncthreads();
+  if (!s_last || warp != 0) return;
+  // The last block to arrive (every block has read the iteration and the
+  // count by then) finishes and advances both: lane l sums blocks l, l + 32,
+  // ..; the 32 partial sums are combined by a fixed shuffle tree, so the order
+  // never depends on timing.
+  __threadfence();
+  const int blocks = gridDim.x;
   double a = 0.0, b = 0.0;
+#pragma unroll 4
   for (int i = lane; i < blocks; i += 32) {
-    a += part[2 * i];
-    b += part[2 * i + 1];
+    a += __ldcg(part + 2 * i);
+    b += __ldcg(part + 2 * i + 1);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -191,7 +195,9 @@ __global__ void test_final(const double* __restrict__ part, int blocks, int64_t 
     b += __shfl_down_sync(0xffffffffu, b, o);
   }
   if (lane == 0) {
-    if ((int64_t)*tp >= burnin) *navg += 1;
+    *navg = n_avg;
+    *tp += 1u;
+    *ticket = 0;
     out[0] = n > 0 ? sqrt(a / (double)n) : 0.0;
     out[1] = n > 0 ? sqrt(b / (double)n) : 0.0;
   }
@@ -221,20 +227,18 @@ int launch_predict(Handle* h, int64_t n, const int32_t* r, const int32_t* c, flo
   return BPMF_OK;
 }
 
+// with a test set also the iteration's end (launch_advance_iter)
 int launch_test_step(Handle* h) {
-  if (h->n_test <= 0) return BPMF_OK;
   const int blocks = pred_blocks(h, h->n_test);
   PhaseTimer timer(h, BPMF_T_PREDICT);
-  h->kernels += 2;
+  h->kernels += 1;
   const int K = h->K, g = pred_group(K);
   const bool vec = (K & 3) == 0;
   auto kern = g == 4 ? (vec ? test_errors<4, true> : test_errors<4, false>)
                      : (vec ? test_errors<8, true> : test_errors<8, false>);
   kern<<<blocks, kPredThreads, 0, h->stream>>>(
       h->side[BPMF_USERS].X, h->side[BPMF_MOVIES].X, K, h->mean, h->trow, h->tcol, h->tval,
-      h->n_test, h->tsum, h->d_iter, h->cfg.burnin, h->d_navg, h->red);
-  test_final<<<1, 32, 0, h->stream>>>(h->red, blocks, h->n_test, h->terr, h->d_iter,
-                                      h->cfg.burnin, h->d_navg);
+      h->n_test, h->tsum, h->d_iter, h->cfg.burnin, h->d_navg, h->red, h->terr, h->test_ticket);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
 }

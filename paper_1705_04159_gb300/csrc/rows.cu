@@ -196,8 +196,11 @@ __global__ void __launch_bounds__(160) piece_fp32(const SweepArgs a) {
 // FP64 redo of flagged rows: one CTA per row, Lambda* and b rebuilt in FP64
 // from the FP64 hyperparameters, Cholesky and solves in FP64 in shared
 // memory, normals in FP64.  A failed FP64 pivot flags kStatusNotPD.
+// The last block to have read the count publishes it and zeroes it and the
+// persistent kernel's row counter for the next sweep.
 __global__ void __launch_bounds__(256) row_fp64(const SweepArgs a, const double* __restrict__ lam,
-                                                const double* __restrict__ mu, int* status) {
+                                                const double* __restrict__ mu, int* status,
+                                                int32_t* redo_count, int* ticket, int* ws_counter) {
   extern __shared__ double dsm[];
   const int K = a.K;
   double* A = dsm;            // K*K
@@ -205,6 +208,16 @@ __global__ void __launch_bounds__(256) row_fp64(const SweepArgs a, const double*
   double* y = b + K;          // K
   __shared__ int bad;
   const int nflag = *a.flag_count;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(ticket, 1) == (int)gridDim.x - 1) {
+      *redo_count = nflag;
+      *a.flag_count = 0;
+      *ws_counter = 0;
+      *ticket = 0;
+    }
+  }
   for (int f = blockIdx.x; f < nflag; f += gridDim.x) {
     const int row = a.flag_rows[f];
     const int64_t p0 = a.ptr[row], p1 = a.ptr[row + 1];
@@ -362,22 +375,33 @@ int launch_fp64_redo(Handle* h, int s, const SweepArgs& a) {
   const size_t smem = sizeof(double) * ((size_t)h->K * h->K + 2 * h->K);
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sizeof(double) * (kMaxK * kMaxK + 2 * kMaxK))));
-  row_fp64<<<h->num_sms, 256, smem, h->stream>>>(a, h->side[s].lam, h->side[s].mu, h->status);
+  row_fp64<<<h->num_sms, 256, smem, h->stream>>>(a, h->side[s].lam, h->side[s].mu, h->status,
+                                                   h->redo_count, h->redo_ticket, h->ws_counter);
   BPMF_CUDA_CHECK(cudaGetLastError());
+  return BPMF_OK;
+}
+
+int clear_sweep_counts(Handle* h) {
+  BPMF_CUDA_CHECK(cudaMemsetAsync(h->flag_count, 0, sizeof(int32_t), h->stream));
+  BPMF_CUDA_CHECK(cudaMemsetAsync(h->ws_counter, 0, sizeof(int), h->stream));
   return BPMF_OK;
 }
 
 int launch_sweep(Handle* h, int s) {
   cudaStream_t st = h->stream;
-  BPMF_CUDA_CHECK(cudaMemsetAsync(h->flag_count, 0, sizeof(int32_t), st));
   SweepArgs a = make_sweep_args(h, s);
+  int rc = BPMF_OK;
   {
     PhaseTimer timer(h, s == BPMF_USERS ? BPMF_T_ROWS_USERS : BPMF_T_ROWS_MOVIES);
     if (h->cfg.path == BPMF_PATH_PLAIN) {
-      BPMF_TRY(launch_rows_fp32(a, st, &h->kernels));
+      rc = launch_rows_fp32(a, st, &h->kernels);
     } else {
-      BPMF_TRY(launch_sweep_binned(h, s, a));
+      rc = launch_sweep_binned(h, s, a);
     }
+  }
+  if (rc != BPMF_OK) {  // the redo will not take these back
+    clear_sweep_counts(h);
+    return rc;
   }
   PhaseTimer timer(h, BPMF_T_FP64_REDO);
   BPMF_TRY(launch_fp64_redo(h, s, a));

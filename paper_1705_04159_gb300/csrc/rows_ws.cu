@@ -983,7 +983,6 @@ int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross
   const int smem = ws_smem_bytes(G, S, C, nb, cross);
   auto kern = nb == 32 ? row_ws<32, false> : cross ? row_ws<64, true> : row_ws<64, false>;
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  BPMF_CUDA_CHECK(cudaMemsetAsync(counter, 0, sizeof(int), st));
   const int grid = (int)std::min<int64_t>(num_sms, nrows);
   CUtensorMap map_hi, map_lo;
   BPMF_TRY(encode_shadow_map(a.Vhi, a.n_other, a.KS, &map_hi));
