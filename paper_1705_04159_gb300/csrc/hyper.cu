@@ -120,33 +120,42 @@ __global__ void __launch_bounds__(32 * kFinalWarps) colsum_final(
   }
 }
 
-// ---- (2) centred scatter S = sum (x - xbar)(x - xbar)^T.  The lower triangle
-// is cut into T = g (g + 1) / 2 tiles of TM x TM (g = ceil(K / TM)), and a
-// block's threads are (tile, subset) pairs: thread t takes tile q = t % T
-// and, if r = t / T < S, rows r, r + S, .. of every chunk of rows.  Chunks
-// are copied by cp.async into a ring of kScatStages shared-memory stages
-// (rows zero padded to g TM columns), so that three chunks are in flight
-// while one is used; each landed chunk is centred in place before use.  The
-// FP32 tile sums of the S subsets are added in shared memory in the order
-// r = 1, 2, .. into subset 0, which moves them into the block's FP64 partial:
-// at the end, and often enough that no FP32 accumulator sums more than
-// kScatFlushRows rows.
-constexpr int kScatThreads = 288;
+// ---- (2) centred scatter S = sum (x - xbar)(x - xbar)^T.  With g = ceil(K / 8)
+// and the features in two halves of 4 g, group I is features 4 I .. 4 I + 3 of
+// both halves, and the lower triangle is cut into T = g (g + 1) / 2 tiles, the
+// 8 x 8 products of group I with group J <= I; a block's threads are (tile,
+// subset) pairs: thread t takes tile t % T and, if r = t / T < S, rows r, r + S,
+// .. of every chunk.  Neighbouring groups then lie 16 bytes apart and a
+// warp's 16-byte loads fall on different banks.  Chunks are copied by cp.async
+// into a ring of kScatStages stages; a thread centres what it copied itself
+// (always the same columns, so it keeps their means) before the one barrier of
+// the chunk.  The S subsets' FP32 sums meet in shared memory, in the order r = 0,
+// 1, .., and go to the block's FP64 partial: at the end, and often enough that
+// no FP32 accumulator sums more than kScatFlushRows rows.
+// What bounds it: the FP32 multiply-adds, with their shared-memory loads close
+// behind.  480,189 rows by 64 blocks, K = 64: 552 us with 4 x 4 tiles, a
+// centring pass with a division an element and two barriers a chunk, 287 now
+// (chunks of 32 rows 330, and 361 with 288 threads in 96 registers);
+// by 26 blocks, K = 100: 2,078 (8 x 8 tiles) -> 1,528.  TF32 tensor-core products,
+// split in two and summed in FP32 every eight rows, took 205 us at K = 64 but
+// their truncated sums doubled the error (2.8e-8 rms of the scale, here 1.5e-8).
 constexpr int kScatStages = 4;
-constexpr int kScatFlushRows = 1024;
-// rows per chunk, for every tile size (the 8 x 8 tiles measured 10% faster
-// at 32 than at 16, and the same at 64)
-constexpr int kScatRows = 32;
+constexpr int kScatFlushRows = 512;
+constexpr int kScatRows = 64;  // rows per chunk
 
-int scatter_tm(int K) { return K > 64 ? 8 : K > 16 ? 4 : K > 4 ? 2 : 1; }
-__host__ __device__ inline int scatter_tiles(int K, int TM) {
-  const int g = (K + TM - 1) / TM;
-  return g * (g + 1) / 2;
-}
-int scatter_smem(int K, int TM) {
-  const int g = (K + TM - 1) / TM;
-  return (int)sizeof(float) * (kScatStages * kScatRows * g * TM + scatter_tiles(K, TM) * TM * TM);
-}
+struct ScatGeom {
+  int g, KP, T, S;
+  __host__ __device__ ScatGeom(int K, int threads) {
+    g = (K + 7) / 8;
+    KP = 8 * g;
+    T = g * (g + 1) / 2;
+    S = threads / T;
+  }
+  __host__ __device__ int floats() const {
+    const int ring = kScatStages * kScatRows * KP, sums = S * T * 64;
+    return ring > sums ? ring : sums;
+  }
+};
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -163,12 +172,174 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// VEC: K % 4 == 0 and X 16-byte aligned (16-byte copies), else 4-byte copies
+template <int NT, bool VEC>
+__global__ void __launch_bounds__(NT, 2) scatter_partial(const float* __restrict__ X, int64_t R, int K,
+                                                                   const float* __restrict__ xbarf,
+                                                                   double* __restrict__ part) {
+  constexpr int W = VEC ? 4 : 1;
+  extern __shared__ __align__(16) float xs[];  // [kScatStages][kScatRows][KP]; sums [S][16][T][4]
+  const ScatGeom G(K, NT);
+  const int KP = G.KP, T = G.T, S = G.S, H = 4 * G.g, stage_f = kScatRows * KP;
+  const int tid = threadIdx.x;
+  const int q = tid % T, r = tid / T;
+  const bool active = r < S;
+  int I = 0;
+  while ((I + 1) * (I + 2) / 2 <= q) ++I;
+  const int J = q - I * (I + 1) / 2;
+  const int64_t per = (R + gridDim.x - 1) / gridDim.x;
+  const int64_t r0 = min(R, (int64_t)blockIdx.x * per);
+  const int64_t r1 = min(R, r0 + per);
+  const int64_t nchunks = (r1 - r0 + kScatRows - 1) / kScatRows;
+  // this thread's pieces of a chunk: columns W cc .. of rows cr, cr + cstep, ..
+  const int P = K / W, cstep = NT / P, cc = tid % P, cr = tid / P < cstep ? tid / P : kScatRows;
+  float mean[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) mean[w] = xbarf[W * cc + w];
+  // the padding columns K .. KP - 1 are never copied: zeroed here, and after the sums have met
+  auto zero_padding = [&]() {
+    for (int e = tid; e < kScatStages * kScatRows; e += NT)
+      for (int k = K; k < KP; ++k) xs[e * KP + k] = 0.f;
+  };
+  zero_padding();
+  auto issue = [&](int64_t c) {
+    if (c < nchunks) {
+      const int64_t c0 = r0 + c * kScatRows;
+      const int cnt = (int)min((int64_t)kScatRows, r1 - c0);
+      float* dst = xs + (int)(c % kScatStages) * stage_f + W * cc;
+      const float* src = X + c0 * K + W * cc;
+      for (int rr = cr; rr < cnt; rr += cstep) {
+        if (VEC) cp_async16(dst + rr * KP, src + (int64_t)rr * K);
+        else cp_async4(dst + rr * KP, src + (int64_t)rr * K);
+      }
+    }
+    cp_async_commit();  // one group per chunk index, empty past the end
+  };
+  float acc[8][8];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+  double* out = part + (int64_t)blockIdx.x * K * K;
+  bool first = true;
+  // the block's sums so far to its partial; acc back to zero
+  auto flush = [&]() {
+    float4* sums = reinterpret_cast<float4*>(xs);
+    if (active) {
+#pragma unroll
+      for (int v = 0; v < 16; ++v)
+        sums[(r * 16 + v) * T + q] = make_float4(acc[v >> 1][4 * (v & 1)], acc[v >> 1][4 * (v & 1) + 1],
+                                                 acc[v >> 1][4 * (v & 1) + 2], acc[v >> 1][4 * (v & 1) + 3]);
+    }
+#pragma unroll
+    for (int a = 0; a < 8; ++a)
+#pragma unroll
+      for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+    __syncthreads();
+    for (int e = tid; e < 16 * T; e += NT) {
+      float4 s = sums[e];
+#pragma unroll 4
+      for (int k = 1; k < S; ++k) {
+        const float4 x = sums[k * 16 * T + e];
+        s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+      }
+      const int v = e / T, p = v >> 1, t = e - v * T;
+      int ti = 0;
+      while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+      const int tj = t - ti * (ti + 1) / 2;
+      const int i = (p < 4 ? 4 * ti + p : H + 4 * ti + p - 4), j0 = 4 * tj + (v & 1 ? H : 0);
+      const float x[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        // past the diagonal: the mirrored entry, which no other tile holds
+        // unless the groups are the same
+        const int j = j0 + w, hi = max(i, j), lo = min(i, j);
+        if (hi < K && (j <= i || ti != tj))
+          out[hi * K + lo] = first ? (double)x[w] : out[hi * K + lo] + (double)x[w];
+      }
+    }
+    first = false;
+  };
+  const int64_t flush_chunks = max(1, kScatFlushRows * S / kScatRows);
+  for (int c = 0; c < kScatStages - 1; ++c) issue(c);
+  for (int64_t c = 0; c < nchunks; ++c) {
+    cp_async_wait<kScatStages - 2>();  // chunk c has landed (this thread's copies)
+    const int cnt = (int)min((int64_t)kScatRows, r1 - r0 - c * kScatRows);
+    float* xb = xs + (int)(c % kScatStages) * stage_f;
+    for (int rr = cr; rr < cnt; rr += cstep) {
+      float* x = xb + rr * KP + W * cc;
+      if constexpr (VEC) {
+        float4 v = *reinterpret_cast<float4*>(x);
+        v.x -= mean[0]; v.y -= mean[1]; v.z -= mean[2]; v.w -= mean[3];
+        *reinterpret_cast<float4*>(x) = v;
+      } else {
+        x[0] -= mean[0];
+      }
+    }
+    __syncthreads();             // everyone's pieces; chunk c - 1 is no longer read
+    issue(c + kScatStages - 1);  // into the stage chunk c - 1 used
+    if (active) {
+      const float *ai = xb + 4 * I, *bj = xb + 4 * J;
+#pragma unroll 2
+      for (int rr = r; rr < cnt; rr += S) {
+        float a[8], b[8];
+        *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(ai + rr * KP);
+        *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(ai + rr * KP + H);
+        *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(bj + rr * KP);
+        *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(bj + rr * KP + H);
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+#pragma unroll
+          for (int p2 = 0; p2 < 8; ++p2) acc[p][p2] = fmaf(a[p], b[p2], acc[p][p2]);
+      }
+    }
+    if ((c + 1) % flush_chunks == 0 && c + 1 < nchunks) {
+      // the sums meet in the ring's memory: the copies in flight land first
+      // and are made again
+      cp_async_wait<0>();
+      __syncthreads();
+      flush();
+      __syncthreads();
+      zero_padding();
+      __syncthreads();
+      for (int k = 1; k < kScatStages; ++k) issue(c + k);
+    }
+  }
+  cp_async_wait<0>();
+  __syncthreads();
+  flush();
+}
+
+// The same for K <= 32, where tiles of eight would leave few of them (K = 10, 8
+// iterations of a job: 836 us instead of 807).  The lower triangle is cut into T = g (g + 1) / 2 tiles of TM x TM (g = ceil(K / TM)), and a
+// block's threads are (tile, subset) pairs: thread t takes tile q = t % T
+// and, if r = t / T < S, rows r, r + S, .. of every chunk of rows.  Chunks
+// are copied by cp.async into a ring of kScatStages shared-memory stages
+// (rows zero padded to g TM columns), so that three chunks are in flight
+// while one is used; each landed chunk is centred in place before use.  The
+// FP32 tile sums of the S subsets are added in shared memory in the order
+// r = 1, 2, .. into subset 0, which moves them into the block's FP64 partial:
+// at the end, and often enough that no FP32 accumulator sums more than
+// kSmallFlushRows rows.
+constexpr int kSmallThreads = 288;
+constexpr int kSmallFlushRows = 1024;
+// rows per chunk
+constexpr int kSmallRows = 32;
+
+constexpr int kSmallScatK = 32;
+int scatter_tm(int K) { return K > 16 ? 4 : K > 4 ? 2 : 1; }
+__host__ __device__ inline int scatter_tiles(int K, int TM) {
+  const int g = (K + TM - 1) / TM;
+  return g * (g + 1) / 2;
+}
+int scatter_smem(int K, int TM) {
+  const int g = (K + TM - 1) / TM;
+  return (int)sizeof(float) * (kScatStages * kSmallRows * g * TM + scatter_tiles(K, TM) * TM * TM);
+}
+
 template <int TM>
 __device__ __forceinline__ void ld_tm(const float* p, float (&x)[TM]) {
-  if constexpr (TM == 8) {
-    const float4 u = reinterpret_cast<const float4*>(p)[0], v = reinterpret_cast<const float4*>(p)[1];
-    x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
-  } else if constexpr (TM == 4) {
+  if constexpr (TM == 4) {
     const float4 u = *reinterpret_cast<const float4*>(p);
     x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
   } else if constexpr (TM == 2) {
@@ -181,13 +352,13 @@ __device__ __forceinline__ void ld_tm(const float* p, float (&x)[TM]) {
 
 // VEC: K % 4 == 0 and X 16-byte aligned (16-byte copies), else 4-byte copies
 template <int TM, bool VEC>
-__global__ void __launch_bounds__(kScatThreads, TM == 8 ? 1 : 2) scatter_partial(const float* __restrict__ X, int64_t R,
+__global__ void __launch_bounds__(kSmallThreads, 2) scatter_small(const float* __restrict__ X, int64_t R,
                                                                 int K, const float* __restrict__ xbarf,
                                                                 double* __restrict__ part) {
-  constexpr int ROWS = kScatRows;
+  constexpr int ROWS = kSmallRows;
   extern __shared__ float sbuf[];
   const int g = (K + TM - 1) / TM, KP = g * TM, T = g * (g + 1) / 2;
-  const int S = kScatThreads / T > 1 ? kScatThreads / T : 1;
+  const int S = kSmallThreads / T > 1 ? kSmallThreads / T : 1;
   const int stage_f = ROWS * KP;
   float* xs = sbuf;                            // [kScatStages][ROWS][KP]
   float* cmb = sbuf + kScatStages * stage_f;   // [T][TM * TM]
@@ -207,7 +378,7 @@ __global__ void __launch_bounds__(kScatThreads, TM == 8 ? 1 : 2) scatter_partial
 #pragma unroll
     for (int b = 0; b < TM; ++b) acc[a][b] = 0.f;
   // the padding columns K .. KP - 1 are never copied: zero them once
-  for (int e = tid; e < kScatStages * stage_f; e += kScatThreads) xs[e] = 0.f;
+  for (int e = tid; e < kScatStages * stage_f; e += kSmallThreads) xs[e] = 0.f;
   __syncthreads();
   auto issue = [&](int64_t c) {
     if (c < nchunks) {
@@ -217,12 +388,12 @@ __global__ void __launch_bounds__(kScatThreads, TM == 8 ? 1 : 2) scatter_partial
       const float* src = X + c0 * K;
       if (VEC) {
         const int q4 = K >> 2;  // 16-byte pieces per row
-        for (int e = tid; e < cnt * q4; e += kScatThreads) {
+        for (int e = tid; e < cnt * q4; e += kSmallThreads) {
           const int rr = e / q4, cc = e - rr * q4;
           cp_async16(dst + rr * KP + 4 * cc, src + (int64_t)rr * K + 4 * cc);
         }
       } else {
-        for (int e = tid; e < cnt * K; e += kScatThreads) {
+        for (int e = tid; e < cnt * K; e += kSmallThreads) {
           const int rr = e / K, cc = e - rr * K;
           cp_async4(dst + rr * KP + cc, src + (int64_t)rr * K + cc);
         }
@@ -263,7 +434,7 @@ __global__ void __launch_bounds__(kScatThreads, TM == 8 ? 1 : 2) scatter_partial
 #pragma unroll
       for (int b = 0; b < TM; ++b) acc[a][b] = 0.f;
   };
-  const int flush_chunks = max(1, kScatFlushRows * S / ROWS);
+  const int flush_chunks = max(1, kSmallFlushRows * S / ROWS);
   for (int c = 0; c < kScatStages - 1; ++c) issue(c);
   int nchunk = 0;
   for (int64_t c = 0; c < nchunks; ++c) {
@@ -273,7 +444,7 @@ __global__ void __launch_bounds__(kScatThreads, TM == 8 ? 1 : 2) scatter_partial
     const int64_t c0 = r0 + c * ROWS;
     const int cnt = (int)min((int64_t)ROWS, r1 - c0);
     float* xb = xs + (int)(c % kScatStages) * stage_f;
-    for (int e = tid; e < cnt * K; e += kScatThreads) {
+    for (int e = tid; e < cnt * K; e += kSmallThreads) {
       const int rr = e / K, k = e - rr * K;
       xb[rr * KP + k] -= xbarf[k];
     }
@@ -366,8 +537,8 @@ int launch_scatter_tm(const float* X, int64_t R, int K, const float* xbarf, doub
                       cudaStream_t st) {
   const int smem = scatter_smem(K, TM);
   BPMF_CUDA_CHECK(
-      cudaFuncSetAttribute(scatter_partial<TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  scatter_partial<TM, VEC><<<blocks, kScatThreads, smem, st>>>(X, R, K, xbarf, part);
+      cudaFuncSetAttribute(scatter_small<TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  scatter_small<TM, VEC><<<blocks, kSmallThreads, smem, st>>>(X, R, K, xbarf, part);
   return BPMF_OK;
 }
 
@@ -377,16 +548,24 @@ bool rows_vec(const float* X, int K) { return (K & 3) == 0 && (reinterpret_cast<
 int launch_scatter(const float* X, int64_t R, int K, const float* xbarf, double* part, int blocks,
                    cudaStream_t st) {
   const bool v = rows_vec(X, K);
-  switch (scatter_tm(K)) {
-    case 8: return v ? launch_scatter_tm<8, true>(X, R, K, xbarf, part, blocks, st)
-                     : launch_scatter_tm<8, false>(X, R, K, xbarf, part, blocks, st);
-    case 4: return v ? launch_scatter_tm<4, true>(X, R, K, xbarf, part, blocks, st)
-                     : launch_scatter_tm<4, false>(X, R, K, xbarf, part, blocks, st);
-    case 2: return v ? launch_scatter_tm<2, true>(X, R, K, xbarf, part, blocks, st)
-                     : launch_scatter_tm<2, false>(X, R, K, xbarf, part, blocks, st);
-    default: return v ? launch_scatter_tm<1, true>(X, R, K, xbarf, part, blocks, st)
-                      : launch_scatter_tm<1, false>(X, R, K, xbarf, part, blocks, st);
+  if (K <= kSmallScatK) {
+    switch (scatter_tm(K)) {
+      case 4: return v ? launch_scatter_tm<4, true>(X, R, K, xbarf, part, blocks, st)
+                       : launch_scatter_tm<4, false>(X, R, K, xbarf, part, blocks, st);
+      case 2: return v ? launch_scatter_tm<2, true>(X, R, K, xbarf, part, blocks, st)
+                       : launch_scatter_tm<2, false>(X, R, K, xbarf, part, blocks, st);
+      default: return v ? launch_scatter_tm<1, true>(X, R, K, xbarf, part, blocks, st)
+                        : launch_scatter_tm<1, false>(X, R, K, xbarf, part, blocks, st);
+    }
   }
+  // up to 36 tiles leave 252 or more of 256 threads busy; 91 and 136 want 288
+  const int threads = K <= 64 ? 256 : 288;
+  auto kern = K <= 64 ? (v ? scatter_partial<256, true> : scatter_partial<256, false>)
+                      : (v ? scatter_partial<288, true> : scatter_partial<288, false>);
+  const int smem = (int)sizeof(float) * ScatGeom(K, threads).floats();
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  kern<<<blocks, threads, smem, st>>>(X, R, K, xbarf, part);
+  return BPMF_OK;
 }
 
 int launch_colsum(const float* X, int64_t R, int K, double* part, int blocks, cudaStream_t st) {
