@@ -541,7 +541,10 @@ template <int NB, bool XO>
 __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S, uint32_t tmem,
                                        int hold) {
   const int lane = threadIdx.x & 31;
-  const uint32_t idesc = idesc_bf16_mn(128, G.NP);
+  // XO: the lo features follow the 128 hi features at the same block stride, so
+  // [h | l] is one operand of 128 + NP columns and h^T [h | l] one product: 32 +
+  // N / 4 cycles, 92 at K = 100 instead of 2 x 60.
+  const uint32_t idesc = idesc_bf16_mn(128, XO ? 128 + G.NP : G.NP);
   // operand tile of the first stage: the leading byte offset steps between
   // 64-feature blocks, the stride one between atoms
   const uint64_t desc0 = smem_desc_sw128(smem_u32(w.stages), WsNb<NB>::kBlk, kWsAtom);
@@ -577,7 +580,6 @@ __device__ __forceinline__ void ws_mma(const WsGeom& G, const WsShared& w, int S
           const uint32_t more = kk == 0 ? (m.flags & 1) ^ 1u : 1u;
           if (XO) {
             tc_mma_bf16(acc, h, h, idesc, more);
-            tc_mma_bf16(acc + kWsAccCols, h, l, idesc, more);
           } else {
             tc_mma_bf16(acc, h, h, idesc, more);
             tc_mma_bf16(acc, h, l, idesc, 1u);
