@@ -91,10 +91,11 @@ struct SideDev {
   std::vector<int64_t> ptr_h;   // host: row pointers
   std::vector<int32_t> perm_h;  // host: degree order
   int64_t max_deg = 0;
-  bool heavy_tc = false;
+  bool heavy_tc = false;  // heavy bin on the per-row tensor-core kernel instead of the persistent one
   int ws_cons = 0;        // consumer warps of the persistent kernel (0: automatic)
   int ws_nb = 32;         // neighbours per stage of the persistent kernel (32 or 64)
-  bool ws_cross = false;  // its 64-neighbour stages form the hi/lo cross term from one product  // heavy bin on the per-row tensor-core kernel instead of the persistent one
+  bool ws_cross = false;  // its 64-neighbour stages form the hi/lo cross term from one product
+  bool ws_wide = false;   // short rows of a large K: fewer stages, more consumers
   bool have_hyper = false;
   bool have_stats = false;
   int64_t fp64_rows = 0;

@@ -80,12 +80,14 @@ int launch_sweep_binned(Handle* h, int s, const SweepArgs& a);
 bool ws_supported(int K);
 // cons: consumer warps per CTA (0: automatic); nb: neighbours per stage (32 or 64);
 // cross: the cross term of the hi/lo split from one product (nb 64 only)
-int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross, int* counter,
-                   int* status, cudaStream_t st, int64_t* launches);
+// wide: a ring of four and as many consumers as fit, up to 11, if cons is 0
+int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross, bool wide,
+                   int* counter, int* status, cudaStream_t st, int64_t* launches);
 // neighbours per stage of the persistent kernel for a side with nnz ratings over R rows
 int ws_stage_neighbours(int64_t nnz, int64_t R);
 // whether that side's 64-neighbour stages form the cross term from one product
 bool ws_cross_once(int64_t nnz, int64_t R);
+bool ws_many_consumers(int K, int64_t nnz, int64_t R, int64_t max_degree);
 // whole rows by one warp each and pieces of split rows, FP32; 1 <= K <= 55
 // (rows_small.cu; launch_rows_fp32 and launch_pieces_fp32 take them where they can)
 bool small_supported(int K);

@@ -99,6 +99,20 @@ constexpr int kWsMaxAcc = 3;
 __host__ __device__ constexpr int ws_stage_bytes(int nb) { return 2 * 2 * nb * 128; }
 constexpr int kWsMaxStages = 16;
 constexpr int kWsMaxCons = 7;
+// The wide form: a ring of four stages instead of eight and as many consumers
+// as fit, up to 11 (past seven, 640 threads of 95 registers instead of 113), for
+// sides of K >= 64 without long rows, whose consumers set the pace: there
+// eight stages of K = 64 leave seven consumers, of K = 72 five, of K >= 80 three.
+// An iteration of 50,000 x 12,000 uniform cells with 2.5M ratings: K = 64 1,145
+// -> 1,075 us, K = 80 1,772 -> 1,434, K = 100 2,837 -> 2,156; with 0.5M 999 -> 902,
+// 1,705 -> 1,284 and 2,779 -> 2,079.  K = 56 gained 2% there and lost 4% with
+// 60,000 x 17,770 and 5M (83 and 281 ratings a row), K <= 48 lost up to 7%.  Below
+// K = 72 sides averaging kWsWideRow ratings or more lose (K = 64, 208 a row: 1%).  A
+// row much longer than the others is copied by one SM at the pace of its ring:
+// sides with one of more than kWsWideMax ratings keep eight stages
+// (ChEMBL-shaped, K = 64: 1,320 us against 1,328).
+constexpr int kWsWideCons = 11, kWsWideK = 64, kWsWideAllK = 72;
+constexpr int64_t kWsWideRow = 128, kWsWideMax = 1024;
 constexpr int kWsRecs = 32;          // row records in flight: >= stages + accumulators + 1
 constexpr int kWsGather = 128, kWsDrain = 128;
 constexpr int kWsMmaWarp = 8, kWsConsWarp0 = 9;
@@ -785,8 +799,8 @@ __device__ __forceinline__ void ws_consume(const SweepArgs& a, const WsGeom& G, 
   }
 }
 
-template <int NB, bool XO>
-__global__ void __launch_bounds__(512, 1) row_ws(const SweepArgs a,
+template <int NB, bool XO, int NT>
+__global__ void __launch_bounds__(NT, 1) row_ws(const SweepArgs a,
                                                  const __grid_constant__ CUtensorMap map_hi,
                                                  const __grid_constant__ CUtensorMap map_lo, int S,
                                                  int C, int* counter, int* status) {
@@ -887,16 +901,20 @@ int ws_stage_neighbours(int64_t nnz, int64_t R) {
 
 bool ws_cross_once(int64_t nnz, int64_t R) { return R > 0 && nnz >= kWsCrossRow * R; }
 
+bool ws_many_consumers(int K, int64_t nnz, int64_t R, int64_t max_degree) {
+  return K >= kWsWideK && R > 0 && max_degree <= kWsWideMax && (K >= kWsWideAllK || nnz < kWsWideRow * R);
+}
+
 bool ws_supported(int K) { return K >= 8 && K + 1 <= 128; }
 
 // Stages (a multiple of 4, one or more ring slots per gather warp) and
 // consumer warps for latent dimension K and nb neighbours per stage (cross:
 // with the base tiles in shared memory).  With
 // `cons` > 0 that many consumers (as many as fit, if fewer) and the deepest
-// ring up to kWsMaxStages that fits;
-// otherwise 8 stages if at least 3 consumers fit beside them, else 4 stages
-// and as many consumers as fit.
-int ws_config(int K, int cons, int nb, bool cross, int* S, int* C) {
+// ring up to kWsMaxStages that fits; otherwise 4 stages and as many consumers
+// as fit, up to kWsWideCons, if wide; else 8 stages if at least 3 consumers fit
+// beside them, or 4 stages and as many consumers as fit.
+int ws_config(int K, int cons, int nb, bool cross, bool wide, int* S, int* C) {
   const WsGeom G(K);
   int dev = 0, max_smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -904,8 +922,8 @@ int ws_config(int K, int cons, int nb, bool cross, int* S, int* C) {
     cudaGetLastError();
     return BPMF_ECUDA;
   }
-  auto fit_cons = [&](int s) {
-    int c = kWsMaxCons;
+  auto fit_cons = [&](int s, int most = kWsMaxCons) {
+    int c = most;
     while (c > 0 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) --c;
     return c;
   };
@@ -915,6 +933,9 @@ int ws_config(int K, int cons, int nb, bool cross, int* S, int* C) {
     s = kWsMaxStages;
     while (s > 4 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) s -= 4;
     while (c > 1 && ws_smem_bytes(G, s, c, nb, cross) > max_smem) --c;  // more than fit: cut
+  } else if (wide) {
+    s = 4;
+    c = fit_cons(s, kWsWideCons);
   } else {
     c = fit_cons(s);
     if (c < 3) {
@@ -973,17 +994,18 @@ int encode_shadow_map(const __nv_bfloat16* p, int64_t rows, int KS, CUtensorMap*
 
 }  // namespace
 
-int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross, int* counter,
-                   int* status, cudaStream_t st, int64_t* launches) {
+int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross, bool wide,
+                   int* counter, int* status, cudaStream_t st, int64_t* launches) {
   const int64_t nrows = a.row_end - a.row_begin;
   if (nrows <= 0) return BPMF_OK;
   if (nb != 32 && nb != 64) return BPMF_EINVAL;
   if (cross && nb != 64) return BPMF_EINVAL;
   int S = 0, C = 0;
-  BPMF_TRY(ws_config(a.K, cons, nb, cross, &S, &C));
+  BPMF_TRY(ws_config(a.K, cons, nb, cross, wide, &S, &C));
   const WsGeom G(a.K);
   const int smem = ws_smem_bytes(G, S, C, nb, cross);
-  auto kern = nb == 32 ? row_ws<32, false> : cross ? row_ws<64, true> : row_ws<64, false>;
+  auto kern = nb == 32 ? (C > kWsMaxCons ? row_ws<32, false, 640> : row_ws<32, false, 512>)
+              : cross  ? row_ws<64, true, 512> : row_ws<64, false, 512>;
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   const int grid = (int)std::min<int64_t>(num_sms, nrows);
   CUtensorMap map_hi, map_lo;
