@@ -369,12 +369,13 @@ __device__ __forceinline__ void ws_issue_stage(const WsGeom& G, const SweepArgs&
     }
   }
   if (split) {
-    // features 64 .. KA - 1 (chunks 0 .. c1 - 1 of the second block) by
+    // features 64 .. KS - 1 (chunks 0 .. c1 - 1 of the second block) by
     // 16-byte cp.async into their swizzled places, rows past cnt (up to the
-    // MMA's 16-neighbour step) zero-filled; the later chunks stay zero from
-    // the start of the kernel.  Every lane arrives on the stage's barrier
-    // once its copies have landed.
-    const int c1 = (G.KA - 64 + 7) >> 3;
+    // MMA's 16-neighbour step) zero-filled; the later chunks, among them the
+    // rating's where K is a multiple of eight, stay zero from the start of
+    // the kernel: a copy of them would read the next row, or past the last.
+    // Every lane arrives on the stage's barrier once its copies have landed.
+    const int c1 = (a.KS - 64) >> 3;
     const int kmax = 16 * ((cnt + 15) >> 4);
     const uint32_t base = smem_u32(stage) + (uint32_t)WsNb<NB>::kBlk;
 #pragma unroll
