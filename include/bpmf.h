@@ -89,7 +89,7 @@ typedef struct {
   int32_t light_max;  /* rows with degree <= light_max take the FP32 light-row kernel on the
                          BINNED and MIXED paths (one warp per row for K <= 55, else one CTA
                          per row); heavier rows take the heavy-row kernel (tensor-core Gram
-                         on MIXED, FP32 CTA per row on BINNED); -1: automatic */
+                         on MIXED, the FP32 light-row kernel on BINNED); -1: automatic */
   int32_t hub_min;    /* rows with degree >= hub_min are split across CTAs; -1: automatic */
   int32_t tiny_max;   /* rows with degree <= tiny_max take the tiny-row kernel, built from
                          chol(Lambda_s) and one rank-one term per rating (BINNED and MIXED
@@ -226,7 +226,7 @@ BPMF_API int bpmf_get_hyper_stats(bpmf_t *h, int side, double *xbar, double *S);
  * (tiny: degree <= tiny_max, chol(Lambda_s) and one rank-one term per
  * rating, one warp per row; light: degree <= light_max, FP32 Gram, one warp per row for
  * K <= 55, else one CTA per row; heavy: tensor-core Gram on the MIXED path,
- * FP32 CTA per row on BINNED; hub: degree >= hub_min, split across
+ * as light on BINNED; hub: degree >= hub_min, split across
  * CTAs) and the number of rows the last sweep redid in FP64 (paper Sec. III:
  * a cheap kernel for rows with few ratings, split tasks for rows with many).
  * Errors: EINVAL. */

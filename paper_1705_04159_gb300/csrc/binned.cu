@@ -8,10 +8,11 @@
 // slice of that order and, inside each launch, the heaviest rows start first
 // (CTAs are issued in index order: a longest-first greedy schedule):
 //   hub   (degree >= hub_min): split into pieces of min(kPiece, hub_min / 2)
-//         ratings; one CTA per piece computes a partial Gram, then one CTA per
-//         hub sums its partials in piece order (deterministic) and factorises;
-//   heavy (light_max < degree < hub_min): one CTA per row, tensor-core Gram
-//         on the MIXED path, FP32 Gram otherwise;
+//         ratings; a CTA (FP32, K <= 55: a warp) per piece computes a partial
+//         Gram, then one CTA per hub sums its partials in piece order
+//         (deterministic) and one of its warps draws;
+//   heavy (light_max < degree < hub_min): tensor-core Gram (persistent kernel
+//         or one CTA per row) on the MIXED path, as light otherwise;
 //   light (tiny_max < degree <= light_max): FP32 Gram; one warp per row for
 //         K <= 55 (rows_small.cu), else one CTA per row;
 //   tiny  (degree <= tiny_max, degree 0 included): one warp per row, rank-one
