@@ -19,9 +19,9 @@
 //   MMA (warp 8, one elected thread): per 16 neighbours hi.hi + hi.lo + lo.hi into
 //     one of three FP32 accumulators in tensor memory (G = X^T X with X the
 //     stage's neighbours x features; lo.lo, ~2^-16 relative, is dropped); on
-//     sides whose rows average 2048 ratings or more, hi.hi and hi.lo into two
-//     accumulators instead, and the drain adds hi.lo and its transpose (two
-//     products per step);
+//     sides whose rows average 2048 ratings or more, hi.[hi lo] as one wide
+//     product into two accumulators instead, and the drain adds hi.lo and its
+//     transpose;
 //   drain (warps 4-7, thread m = tensor-memory lane m = matrix row m):
 //     forms A = base + alpha G (base = bordered [[Lambda_s, b0], [b0^T, 0]],
 //     kept in tensor memory, or in shared memory where the accumulators take
@@ -33,7 +33,7 @@
 //     registers by every lane, the panel by forward substitution), then
 //     u = L^-T (y + z) by back substitution.
 // So the tensor cores, the gathers and the FP32 factorisations of up to
-// seven rows per SM overlap, with no CTA-wide barrier on the way.
+// eleven rows per SM overlap, with no CTA-wide barrier on the way.
 //
 // Every mbarrier wait polls with a wall-clock bound; on a timeout the CTA
 // records kStatusTimeout, every role leaves its loop, outstanding copies and
@@ -81,10 +81,11 @@ struct WsNb {
 
 // With XO ("cross once") the cross term h^T l + l^T h comes from one product:
 // h^T h and h^T l go to two accumulators and the drain adds h^T l and its
-// transpose (a second pass over the slot).  Two products per step instead of
-// three, which pays where rows are long enough for the tensor pipe to set
-// the pace (sides averaging kWsCrossRow ratings or more); where they are
-// shorter the drain's second pass costs more than the product it saves.
+// transpose (a second pass over the slot).  One wide product per step instead
+// of three (92 cycles against 180 at K = 100), which pays where rows are long
+// enough for the tensor pipe to set the pace (sides averaging kWsCrossRow
+// ratings or more); where they are shorter the drain's second pass costs more
+// than it saves.
 constexpr int64_t kWsCrossRow = 2048;
 template <bool XO>
 __host__ __device__ constexpr uint32_t ws_acc_stride() { return XO ? 256u : 128u; }  // TMEM columns per buffer
