@@ -253,7 +253,8 @@ BPMF_API int bpmf_get_thresholds(bpmf_t *h, int side, int64_t thresholds[5]);
  * shared memory are cut to what fits), else 0.  On the PLAIN path only the
  * values in effect are accepted.  Results are exact either way: the schedule
  * changes which kernel draws a row, not the conditional it draws from.
- * Errors: EINVAL (nothing changed), ECUDA. */
+ * Errors: EINVAL, ECUDA (among them: no memory for the pieces of split rows);
+ * the schedule in effect stays. */
 BPMF_API int bpmf_set_thresholds(bpmf_t *h, int side, const int64_t thresholds[5]);
 
 /* Failure-path limits (the paper has no counterpart; both default to values

@@ -54,6 +54,10 @@ int launch_sweep_binned(Handle* h, int s, const SweepArgs& a0) {
   const bool fork = sd.n_hub > 0 && others && h->aux != nullptr;
   cudaStream_t hs = fork ? h->aux : st;
   int rc = BPMF_OK;
+  if (sd.n_pieces * partial_floats_per_piece(h->K) > h->hub_part_len) {
+    set_error("launch_sweep_binned: no memory for the partial Grams of split rows");
+    return BPMF_ENOMEM;
+  }
   if (fork) {
     BPMF_CUDA_CHECK(cudaEventRecord(h->ev_fork, st));
     BPMF_CUDA_CHECK(cudaStreamWaitEvent(hs, h->ev_fork, 0));
@@ -120,7 +124,44 @@ int launch_other_bins(Handle* h, int s, const SweepArgs& a, cudaStream_t st) {
 
 namespace {
 
-// Row counts per bin and the pieces of the hubs for the given thresholds.
+// n bytes on the device; without them the error is cleared, so that the next
+// launch does not report it.
+int alloc_bytes(void** p, int64_t n) {
+  *p = nullptr;
+  const cudaError_t e = cudaMalloc(p, (size_t)n);
+  if (e == cudaSuccess) return BPMF_OK;
+  cudaGetLastError();
+  *p = nullptr;
+  set_error("cudaMalloc of %lld bytes for split rows: %s", (long long)n, cudaGetErrorString(e));
+  return BPMF_ECUDA;
+}
+
+// Room for `need` floats of partial Grams (one buffer serves both sides, whose
+// sweeps run one after the other).  The old buffer goes first only where both
+// do not fit, and is had again if the new one does not fit without it either.
+int grow_partials(Handle* h, int64_t need) {
+  if (need <= h->hub_part_len) return BPMF_OK;
+  void* p = nullptr;
+  int rc = alloc_bytes(&p, sizeof(float) * need);
+  if (rc != BPMF_OK && h->hub_part) {
+    cudaFree(h->hub_part);
+    h->hub_part = nullptr;
+    rc = alloc_bytes(&p, sizeof(float) * need);
+    if (rc != BPMF_OK) {
+      void* old = nullptr;
+      if (alloc_bytes(&old, sizeof(float) * h->hub_part_len) != BPMF_OK) h->hub_part_len = 0;
+      h->hub_part = static_cast<float*>(old);
+    }
+  }
+  if (rc != BPMF_OK) return rc;
+  cudaFree(h->hub_part);
+  h->hub_part = static_cast<float*>(p);
+  h->hub_part_len = need;
+  return BPMF_OK;
+}
+
+// Row counts per bin and the pieces of the hubs for the given thresholds.  Where
+// the pieces' memory cannot be had, the schedule in effect stays.
 int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hub_min) {
   SideDev& sd = h->side[s];
   cudaStream_t st = h->stream;
@@ -128,10 +169,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
   hub_min = std::max<int64_t>(1, hub_min);
   light_max = std::max(light_max, tiny_max);
   const bool new_hubs = hub_min != sd.hub_min || sd.hub_piece0 == nullptr;
-  sd.tiny_max = tiny_max;
-  sd.light_max = light_max;
-  sd.hub_min = hub_min;
-  for (int b = 0; b < kNumBins; ++b) sd.bin_count[b] = 0;
+  int64_t count[kNumBins] = {0, 0, 0, 0};
   int64_t n_hub = 0, tiny_ratings = 0;
   for (int64_t q = 0; q < R; ++q) {
     const int64_t d = sd.deg_h[q];
@@ -140,7 +178,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
     else if (d <= tiny_max) bin = kBinTiny;
     else if (d <= light_max) bin = kBinLight;
     else bin = kBinHeavy;
-    sd.bin_count[bin] += 1;
+    count[bin] += 1;
     if (bin == kBinTiny) tiny_ratings += d;
     if (bin == kBinHub) {
       // degree order puts every hub before every other row
@@ -151,7 +189,68 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
       ++n_hub;
     }
   }
-  const int64_t pre = rank1_pre_floats(h->K, h->side[1 - s].R, sd.bin_count[kBinTiny], tiny_ratings);
+  if (new_hubs) {
+    // piece length: half the hub threshold, at most kPiece ratings
+    const int64_t plen = std::max<int64_t>(1, std::min<int64_t>(kPiece, hub_min / 2));
+    std::vector<int32_t> prow, hub0;
+    std::vector<int64_t> pe0, pe1;
+    for (int64_t q = 0; q < n_hub; ++q) {
+      const int32_t r = sd.perm_h[q];
+      hub0.push_back((int32_t)prow.size());
+      for (int64_t e = sd.ptr_h[r]; e < sd.ptr_h[r + 1]; e += plen) {
+        prow.push_back(r);
+        pe0.push_back(e);
+        pe1.push_back(std::min(sd.ptr_h[r + 1], e + plen));
+      }
+    }
+    hub0.push_back((int32_t)prow.size());
+    const int64_t n_pieces = (int64_t)prow.size();
+    BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
+    int32_t *row = nullptr, *first = nullptr;
+    int64_t *e0 = nullptr, *e1 = nullptr;
+    auto carve = [&](Carve& c) {
+      row = c.take<int32_t>(n_pieces);
+      e0 = c.take<int64_t>(n_pieces);
+      e1 = c.take<int64_t>(n_pieces);
+      first = c.take<int32_t>(n_hub + 1);
+    };
+    Carve size, c;
+    carve(size);
+    // all the memory first: from here on nothing of the side changes unless all of it does
+    BPMF_TRY(grow_partials(h, n_pieces * partial_floats_per_piece(h->K)));
+    if ((int64_t)size.bytes > sd.piece_bytes) {
+      void* p = nullptr;
+      BPMF_TRY(alloc_bytes(&p, (int64_t)size.bytes));
+      if (sd.piece_own) cudaFree(sd.piece_mem);
+      sd.piece_mem = static_cast<char*>(p);
+      sd.piece_bytes = (int64_t)size.bytes;
+      sd.piece_own = true;
+    }
+    sd.n_hub = n_hub;
+    sd.n_pieces = n_pieces;
+    c.base = sd.piece_mem;
+    carve(c);
+    sd.piece_row = row;
+    sd.piece_e0 = e0;
+    sd.piece_e1 = e1;
+    sd.hub_piece0 = first;
+    if (sd.n_pieces > 0) {
+      BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_row, prow.data(), sizeof(int32_t) * sd.n_pieces,
+                                      cudaMemcpyHostToDevice, st));
+      BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_e0, pe0.data(), sizeof(int64_t) * sd.n_pieces,
+                                      cudaMemcpyHostToDevice, st));
+      BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_e1, pe1.data(), sizeof(int64_t) * sd.n_pieces,
+                                      cudaMemcpyHostToDevice, st));
+    }
+    BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.hub_piece0, hub0.data(), sizeof(int32_t) * (n_hub + 1),
+                                    cudaMemcpyHostToDevice, st));
+    BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
+  }
+  sd.tiny_max = tiny_max;
+  sd.light_max = light_max;
+  sd.hub_min = hub_min;
+  std::copy(count, count + kNumBins, sd.bin_count);
+  const int64_t pre = rank1_pre_floats(h->K, h->side[1 - s].R, count[kBinTiny], tiny_ratings);
   if (pre != sd.tiny_pre_len) {
     BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
     cudaFree(sd.tiny_pre);
@@ -163,61 +262,6 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
       sd.tiny_pre = nullptr;
     }
     if (sd.tiny_pre) sd.tiny_pre_len = pre;
-  }
-  if (!new_hubs) return BPMF_OK;
-  // piece length: half the hub threshold, at most kPiece ratings
-  const int64_t plen = std::max<int64_t>(1, std::min<int64_t>(kPiece, hub_min / 2));
-  std::vector<int32_t> prow, hub0;
-  std::vector<int64_t> pe0, pe1;
-  for (int64_t q = 0; q < n_hub; ++q) {
-    const int32_t r = sd.perm_h[q];
-    hub0.push_back((int32_t)prow.size());
-    for (int64_t e = sd.ptr_h[r]; e < sd.ptr_h[r + 1]; e += plen) {
-      prow.push_back(r);
-      pe0.push_back(e);
-      pe1.push_back(std::min(sd.ptr_h[r + 1], e + plen));
-    }
-  }
-  hub0.push_back((int32_t)prow.size());
-  BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  sd.n_hub = n_hub;
-  sd.n_pieces = (int64_t)prow.size();
-  auto carve = [&](Carve& c) {
-    sd.piece_row = c.take<int32_t>(sd.n_pieces);
-    sd.piece_e0 = c.take<int64_t>(sd.n_pieces);
-    sd.piece_e1 = c.take<int64_t>(sd.n_pieces);
-    sd.hub_piece0 = c.take<int32_t>(n_hub + 1);
-  };
-  Carve size, c;
-  carve(size);
-  if ((int64_t)size.bytes > sd.piece_bytes) {
-    if (sd.piece_own) cudaFree(sd.piece_mem);
-    sd.piece_mem = nullptr;
-    sd.piece_bytes = 0;
-    sd.piece_own = true;
-    BPMF_CUDA_CHECK(cudaMalloc(&sd.piece_mem, size.bytes));
-    sd.piece_bytes = (int64_t)size.bytes;
-  }
-  c.base = sd.piece_mem;
-  carve(c);
-  if (sd.n_pieces > 0) {
-    BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_row, prow.data(), sizeof(int32_t) * sd.n_pieces,
-                                    cudaMemcpyHostToDevice, st));
-    BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_e0, pe0.data(), sizeof(int64_t) * sd.n_pieces,
-                                    cudaMemcpyHostToDevice, st));
-    BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.piece_e1, pe1.data(), sizeof(int64_t) * sd.n_pieces,
-                                    cudaMemcpyHostToDevice, st));
-  }
-  BPMF_CUDA_CHECK(cudaMemcpyAsync(sd.hub_piece0, hub0.data(), sizeof(int32_t) * (n_hub + 1),
-                                  cudaMemcpyHostToDevice, st));
-  BPMF_CUDA_CHECK(cudaStreamSynchronize(st));
-  // one partial buffer serves both sides (the sweeps run one after the other)
-  const int64_t need = sd.n_pieces * partial_floats_per_piece(h->K);
-  if (need > h->hub_part_len) {
-    cudaFree(h->hub_part);
-    h->hub_part = nullptr;
-    BPMF_CUDA_CHECK(cudaMalloc(&h->hub_part, sizeof(float) * need));
-    h->hub_part_len = need;
   }
   return BPMF_OK;
 }
