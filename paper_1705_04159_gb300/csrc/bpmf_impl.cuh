@@ -319,6 +319,22 @@ int check_status(Handle* h, const char* where);  // waits for the stream, maps d
     }                                                                                  \
   } while (0)
 
+namespace gb {
+
+// Lets kern use up to `most` bytes of dynamic shared memory.  `most` is the
+// largest that any launch of this kernel asks for, not this launch's size: the
+// limit belongs to the kernel on its device, and a sampler of another latent
+// dimension on another host thread may set it between this call and the launch.
+// Kernels that never ask for more than 48 KB need no call.
+template <typename F>
+int allow_smem(F kern, size_t most) {
+  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+  return BPMF_OK;
+}
+constexpr size_t kSmemNoOptIn = 48 * 1024;
+
+}  // namespace gb
+
 #define BPMF_TRY(expr)      \
   do {                      \
     int rc_ = (expr);       \

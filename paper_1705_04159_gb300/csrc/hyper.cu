@@ -155,6 +155,10 @@ struct ScatGeom {
     const int ring = kScatStages * kScatRows * KP, sums = S * T * 64;
     return ring > sums ? ring : sums;
   }
+  // the most that any K up to max_k takes (S T <= threads)
+  static constexpr int max_floats(int max_k, int threads) {
+    return kScatStages * kScatRows * max_k > threads * 64 ? kScatStages * kScatRows * max_k : threads * 64;
+  }
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -328,14 +332,15 @@ constexpr int kSmallRows = 32;
 
 constexpr int kSmallScatK = 32;
 int scatter_tm(int K) { return K > 16 ? 4 : K > 4 ? 2 : 1; }
-__host__ __device__ inline int scatter_tiles(int K, int TM) {
+__host__ __device__ constexpr int scatter_tiles(int K, int TM) {
   const int g = (K + TM - 1) / TM;
   return g * (g + 1) / 2;
 }
-int scatter_smem(int K, int TM) {
+constexpr int scatter_smem(int K, int TM) {
   const int g = (K + TM - 1) / TM;
   return (int)sizeof(float) * (kScatStages * kSmallRows * g * TM + scatter_tiles(K, TM) * TM * TM);
 }
+static_assert(scatter_smem(kSmallScatK, 4) <= kSmemNoOptIn, "scatter_small takes no opt-in");
 
 template <int TM>
 __device__ __forceinline__ void ld_tm(const float* p, float (&x)[TM]) {
@@ -536,8 +541,6 @@ template <int TM, bool VEC>
 int launch_scatter_tm(const float* X, int64_t R, int K, const float* xbarf, double* part, int blocks,
                       cudaStream_t st) {
   const int smem = scatter_smem(K, TM);
-  BPMF_CUDA_CHECK(
-      cudaFuncSetAttribute(scatter_small<TM, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   scatter_small<TM, VEC><<<blocks, kSmallThreads, smem, st>>>(X, R, K, xbarf, part);
   return BPMF_OK;
 }
@@ -559,11 +562,12 @@ int launch_scatter(const float* X, int64_t R, int K, const float* xbarf, double*
     }
   }
   // up to 36 tiles leave 252 or more of 256 threads busy; 91 and 136 want 288
-  const int threads = K <= 64 ? 256 : 288;
-  auto kern = K <= 64 ? (v ? scatter_partial<256, true> : scatter_partial<256, false>)
+  constexpr int kNarrow = 64;
+  const int threads = K <= kNarrow ? 256 : 288;
+  auto kern = K <= kNarrow ? (v ? scatter_partial<256, true> : scatter_partial<256, false>)
                       : (v ? scatter_partial<288, true> : scatter_partial<288, false>);
   const int smem = (int)sizeof(float) * ScatGeom(K, threads).floats();
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(kern, sizeof(float) * ScatGeom::max_floats(K <= kNarrow ? kNarrow : kMaxK, threads)));
   kern<<<blocks, threads, smem, st>>>(X, R, K, xbarf, part);
   return BPMF_OK;
 }

@@ -66,6 +66,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kR1MaxWarps = 8;
 constexpr int kR1Rows = 4;  // rows of a group (they share the product with L_s^-T)
+constexpr size_t kR1Smem = 200 * 1024;  // dynamic shared memory of a CTA, at most
 
 __device__ __forceinline__ int tri(int i) { return (i * (i + 1)) >> 1; }
 
@@ -535,7 +536,7 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
 // CTAs of `kern` that fill the device, at most `need`
 template <typename F>
 int r1_grid(F kern, int threads, size_t smem, int64_t need, unsigned* grid) {
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  BPMF_TRY(allow_smem(kern, kR1Smem));
   int dev = 0, sms = 1, occ = 1;
   BPMF_CUDA_CHECK(cudaGetDevice(&dev));
   BPMF_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -547,8 +548,7 @@ int r1_grid(F kern, int threads, size_t smem, int64_t need, unsigned* grid) {
 template <int NPL>
 int launch_r1(const SweepArgs& a, const float* lchol, float* T, float* W, int D, cudaStream_t st) {
   constexpr int KP = 32 * NPL, LD = KP + 4;
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(linv_columns<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       linv_smem(a.K)));
+  BPMF_TRY(allow_smem(linv_columns<NPL>, linv_smem(KP)));
   linv_columns<NPL><<<KP, 32, linv_smem(a.K), st>>>(lchol, a.K, T);
   BPMF_CUDA_CHECK(cudaGetLastError());
   const size_t tbytes = sizeof(float) * KP * LD;
@@ -563,7 +563,7 @@ int launch_r1(const SweepArgs& a, const float* lchol, float* T, float* W, int D,
   }
   const size_t per = sizeof(float) * (size_t)r1_warp_floats(D, KP);
   int w = kR1MaxWarps;
-  while (w > 1 && tbytes + w * per > 200 * 1024) --w;
+  while (w > 1 && tbytes + w * per > kR1Smem) --w;
   const size_t smem = tbytes + w * per;
   const int64_t n = a.row_end - a.row_begin, per_cta = (int64_t)w * kR1Rows;
   auto kern = W != nullptr ? row_rank1<NPL, true> : row_rank1<NPL, false>;

@@ -294,22 +294,13 @@ __global__ void init_factors_kernel(float* X, int64_t R, int K, uint2 key, uint3
   }
 }
 
-namespace {
-
-int set_smem_attr(const void* fn, int bytes) {
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  return BPMF_OK;
-}
-
-}  // namespace
-
 int launch_rows_fp32(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
   if (small_supported(a.K)) return launch_rows_small(a, st, launches);
   const int64_t nrows = a.row_end - a.row_begin;
   if (nrows <= 0) return BPMF_OK;
   const TileGeom G(a.K, 8);
   const int smem = smem_bytes_fp32(G);
-  BPMF_TRY(set_smem_attr((const void*)row_fp32, smem));
+  BPMF_TRY(allow_smem(row_fp32, smem_bytes_fp32(TileGeom(kMaxK, 8))));
   for (int64_t off = 0; off < nrows; off += 1LL << 30) {
     SweepArgs b = a;
     b.row_begin = a.row_begin + off;
@@ -326,7 +317,7 @@ int launch_pieces_fp32(const SweepArgs& a, int64_t npieces, cudaStream_t st, int
   if (npieces <= 0) return BPMF_OK;
   const TileGeom G(a.K, 8);
   const int smem = (int)sizeof(float) * 2 * kChunk * G.KPs;
-  BPMF_TRY(set_smem_attr((const void*)piece_fp32, smem));
+  BPMF_TRY(allow_smem(piece_fp32, sizeof(float) * 2 * kChunk * TileGeom(kMaxK, 8).KPs));
   piece_fp32<<<(unsigned)npieces, G.nthreads, smem, st>>>(a);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;
@@ -373,8 +364,7 @@ SweepArgs make_sweep_args(Handle* h, int s) {
 
 int launch_fp64_redo(Handle* h, int s, const SweepArgs& a) {
   const size_t smem = sizeof(double) * ((size_t)h->K * h->K + 2 * h->K);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(sizeof(double) * (kMaxK * kMaxK + 2 * kMaxK))));
+  BPMF_TRY(allow_smem(row_fp64, sizeof(double) * (kMaxK * kMaxK + 2 * kMaxK)));
   row_fp64<<<h->num_sms, 256, smem, h->stream>>>(a, h->side[s].lam, h->side[s].mu, h->status,
                                                    h->redo_count, h->redo_ticket, h->ws_counter);
   BPMF_CUDA_CHECK(cudaGetLastError());

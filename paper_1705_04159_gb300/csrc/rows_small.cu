@@ -392,7 +392,7 @@ template <int g, bool B>
 int launch_small(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
   using S = SmGeom<g, B>;
   const int smem = (S::NT * kTileF + kSmWarps * S::kFloats) * (int)sizeof(float);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_small<g, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(row_small<g, B>, smem));
   const int64_t n = a.row_end - a.row_begin;
   for (int64_t off = 0; off < n; off += (int64_t)kSmWarps << 27) {
     SweepArgs b = a;
@@ -410,7 +410,7 @@ template <int g, bool B>
 int launch_small_pieces(const SweepArgs& a, int64_t npieces, cudaStream_t st, int64_t* launches) {
   using S = SmGeom<g, B>;
   const int smem = kSmWarps * S::kStage * (int)sizeof(float);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(piece_small<g, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(piece_small<g, B>, smem));
   piece_small<g, B><<<(unsigned)((npieces + kSmWarps - 1) / kSmWarps), 32 * kSmWarps, smem, st>>>(a, npieces);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;
@@ -461,9 +461,9 @@ int64_t partial_floats_per_piece(int K) {
 int launch_hub_draw(const SweepArgs& a, cudaStream_t st, int64_t* launches) {
   const int64_t n = a.row_end - a.row_begin;
   if (n <= 0) return BPMF_OK;
-  const int g = (a.K + 8) / 8;
-  const int smem = (g * (g + 1) / 2 * kTileF + 3 * 8 * g) * (int)sizeof(float);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(hub_draw, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  auto bytes = [](int g) { return (g * (g + 1) / 2 * kTileF + 3 * 8 * g) * sizeof(float); };
+  static_assert(bytes((kMaxK + 8) / 8) <= kSmemNoOptIn, "hub_draw takes no opt-in");
+  const size_t smem = bytes((a.K + 8) / 8);
   hub_draw<<<(unsigned)n, kHubThreads, smem, st>>>(a);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;

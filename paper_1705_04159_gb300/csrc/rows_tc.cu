@@ -48,6 +48,7 @@ namespace {
 
 constexpr int kTcStage = 32;                    // neighbours per stage
 constexpr int kTcM = 128;                       // accumulator rows (features, padded)
+constexpr int kTcMaxK = kTcM - 1;               // the rating takes a row
 constexpr int kTcLBO = 128;                     // bytes between core matrices along K
 constexpr int kTcSBO = 4 * 128 + 16;            // bytes between 8-row groups (Gram tiles)
 constexpr int kTcTile = 16 * kTcSBO;            // one Gram operand tile (128 rows x 32 k)
@@ -525,7 +526,7 @@ bool tc_supported(int K) {
   const TileGeom G(K, 8);
   // finish kernels of split rows use 8 x 8 FP32 tiles (K + 1 > 48); the
   // accumulator spans at most 128 rows and 128 columns
-  return K + 1 > 48 && G.KA <= kTcM && G.ntiles <= 160;
+  return K + 1 > 48 && K <= kTcMaxK && G.ntiles <= 160;
 }
 
 int launch_rows_tc(const SweepArgs& a, int* status, cudaStream_t st, int64_t* launches) {
@@ -533,7 +534,7 @@ int launch_rows_tc(const SweepArgs& a, int* status, cudaStream_t st, int64_t* la
   if (nrows <= 0) return BPMF_OK;
   const TileGeom G(a.K, 8);
   const int smem = tc_smem_bytes(G);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(row_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(row_tc, tc_smem_bytes(TileGeom(kTcMaxK, 8))));
   for (int64_t off = 0; off < nrows; off += 1LL << 30) {
     SweepArgs b = a;
     b.row_begin = a.row_begin + off;
@@ -550,7 +551,7 @@ int launch_pieces_tc(const SweepArgs& a, int64_t npieces, int* status, cudaStrea
   if (npieces <= 0) return BPMF_OK;
   const TileGeom G(a.K, 8);
   const int smem = tc_smem_bytes(G);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(piece_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(piece_tc, tc_smem_bytes(TileGeom(kTcMaxK, 8))));
   piece_tc<<<(unsigned)npieces, kTcThreads, smem, st>>>(a, status);
   BPMF_CUDA_CHECK(cudaGetLastError());
   if (launches) *launches += 1;

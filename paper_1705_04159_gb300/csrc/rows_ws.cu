@@ -916,7 +916,7 @@ bool ws_supported(int K) { return K >= 8 && K + 1 <= 128; }
 // ring up to kWsMaxStages that fits; otherwise 4 stages and as many consumers
 // as fit, up to kWsWideCons, if wide; else 8 stages if at least 3 consumers fit
 // beside them, or 4 stages and as many consumers as fit.
-int ws_config(int K, int cons, int nb, bool cross, bool wide, int* S, int* C) {
+int ws_config(int K, int cons, int nb, bool cross, bool wide, int* S, int* C, int* most) {
   const WsGeom G(K);
   int dev = 0, max_smem = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -948,6 +948,7 @@ int ws_config(int K, int cons, int nb, bool cross, bool wide, int* S, int* C) {
   if (c < 1 || ws_smem_bytes(G, s, c, nb, cross) > max_smem) return BPMF_EINVAL;
   *S = s;
   *C = c;
+  *most = max_smem;
   return BPMF_OK;
 }
 
@@ -1002,13 +1003,13 @@ int launch_rows_ws(const SweepArgs& a, int num_sms, int cons, int nb, bool cross
   if (nrows <= 0) return BPMF_OK;
   if (nb != 32 && nb != 64) return BPMF_EINVAL;
   if (cross && nb != 64) return BPMF_EINVAL;
-  int S = 0, C = 0;
-  BPMF_TRY(ws_config(a.K, cons, nb, cross, wide, &S, &C));
+  int S = 0, C = 0, most = 0;
+  BPMF_TRY(ws_config(a.K, cons, nb, cross, wide, &S, &C, &most));
   const WsGeom G(a.K);
   const int smem = ws_smem_bytes(G, S, C, nb, cross);
   auto kern = nb == 32 ? (C > kWsMaxCons ? row_ws<32, false, 640> : row_ws<32, false, 512>)
               : cross  ? row_ws<64, true, 512> : row_ws<64, false, 512>;
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(kern, most));
   const int grid = (int)std::min<int64_t>(num_sms, nrows);
   CUtensorMap map_hi, map_lo;
   BPMF_TRY(encode_shadow_map(a.Vhi, a.n_other, a.KS, &map_hi));

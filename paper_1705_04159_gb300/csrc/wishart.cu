@@ -586,7 +586,7 @@ namespace {
 template <typename... P, typename... A>
 int launch_cluster(void (*kern)(P...), int K, cudaStream_t st, A... args) {
   const int smem = wish_smem(K);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(kern, wish_smem(kMaxK)));
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)wish_ctas(K));
@@ -619,7 +619,7 @@ int launch_spd_inverse_f64(const double* A, double* Ainv, int K, double* scratch
 
 int launch_check_spd_f64(const double* A, int K, int* status, float* lout, cudaStream_t st) {
   const int smem = wish_smem(K);
-  BPMF_CUDA_CHECK(cudaFuncSetAttribute(spd_check, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  BPMF_TRY(allow_smem(spd_check, wish_smem(kMaxK)));
   spd_check<<<1, kWishThreads, smem, st>>>(A, K, status, lout);
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
