@@ -256,7 +256,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
     cudaFree(sd.tiny_pre);
     sd.tiny_pre = nullptr;
     sd.tiny_pre_len = 0;
-    // without the memory the products are formed row by row
+    // without the memory the products are formed row by row: the same draws, bit for bit
     if (pre > 0 && cudaMalloc(&sd.tiny_pre, sizeof(float) * pre) != cudaSuccess) {
       cudaGetLastError();
       sd.tiny_pre = nullptr;

@@ -71,7 +71,7 @@ struct SideDev {
   double* mu = nullptr;    // K
   float* lamaug = nullptr; // (K+1)^2: Lambda_s bordered by b0 = Lambda_s mu_s (row and column K)
   float* lchol = nullptr;  // K(K+1)/2: chol(Lambda_s), lower, packed by rows, FP32 (rank-one kernel)
-  float* tiny_pre = nullptr;  // L_s^-1 of the other side's rows (tiny-row kernel), or none
+  float* tiny_pre = nullptr;  // sqrt(alpha) L_s^-1 of the other side's rows (tiny-row kernel), or none
   int64_t tiny_pre_len = 0;   // its floats
   float* linvT = nullptr;  // KP x (KP + 4), KP = K rounded up to 32: (L_s^-1)^T (tiny-row kernel)
   // split rows (hubs): pieces of at most kPiece ratings, in degree order

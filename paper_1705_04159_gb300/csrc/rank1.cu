@@ -32,10 +32,13 @@
 // the other row kernels (L*_ii^2 against Lambda*_ii) still decides which rows
 // go to the FP64 redo.
 //
-// The w_t do not depend on the row: w_t = sqrt(alpha) L_s^-1 v_j, and
-// c = L_s^-1 b0 + alpha sum_t r_t L_s^-1 v_j.  Where the bin's ratings outnumber
-// the other side's rows, lower_rows forms L_s^-1 v_j for every j once per sweep
-// (PRE), and a row is left with the scans and the product with L_s^-T.
+// The w_t do not depend on the row but through the neighbour j: w_t = L_s^-1
+// sqrt(alpha) v_j, and c = L_s^-1 b0 + sqrt(alpha) sum_t r_t w_t.  Where the bin's
+// ratings outnumber the other side's rows, lower_rows forms them for every j once
+// per sweep (PRE), and a row is left with the scans and the product with L_s^-T.  The
+// other form takes the same products row by row and then the same steps, so a
+// row's draw is bitwise the same in both: which one runs depends on the other
+// rows of the bin and on the memory at hand.
 //
 // Layout.  linv_columns writes T = (L_s^-1)^T, KP x LD floats (KP = K rounded
 // up to 32, LD = KP + 4, zero outside the triangle), once per sweep, in FP64
@@ -299,11 +302,11 @@ __host__ __device__ __forceinline__ int r1_warp_floats(int D, int KP) {
   return (2 * D + 1 + kR1Rows) * KP;
 }
 
-// W row j = L_s^-1 (row j of V) for j < n, and row n = L_s^-1 b0: KP floats per
-// row, zero past K.  A warp takes four rows at a time.
+// W row j = L_s^-1 (sqrt(alpha) row j of V) for j < n, and row n = L_s^-1 b0: KP
+// floats per row, zero past K.  A warp takes four rows at a time.
 template <int NPL>
 __global__ void __launch_bounds__(32 * kR1MaxWarps)
-    lower_rows(const float* __restrict__ V, int64_t n, int K, const float* __restrict__ b0,
+    lower_rows(const float* __restrict__ V, int64_t n, int K, float alpha, const float* __restrict__ b0,
                const float* __restrict__ Tg, float* __restrict__ W) {
   constexpr int KP = 32 * NPL, LD = KP + 4;
   extern __shared__ __align__(16) float r1s[];
@@ -312,6 +315,7 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
     reinterpret_cast<float4*>(r1s)[e] = __ldg(reinterpret_cast<const float4*>(Tg) + e);
   __syncthreads();
   float* vec = r1s + KP * LD + warp * 4 * KP;
+  const float sa = sqrtf(alpha);
   const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5) * 4;
   for (int64_t j0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * 4; j0 <= n; j0 += stride) {
     __syncwarp();
@@ -321,7 +325,8 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
 #pragma unroll
       for (int m = 0; m < NPL; ++m) {
         const int i = lane + 32 * m;
-        vec[g * KP + i] = j0 + g <= n && i < K ? __ldg(v + i) : 0.f;
+        const float x = j0 + g <= n && i < K ? __ldg(v + i) : 0.f;
+        vec[g * KP + i] = j0 + g < n ? sa * x : x;
       }
     }
     __syncwarp();
@@ -335,7 +340,7 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
   }
 }
 
-// PRE: W holds L_s^-1 of the other side's rows and of b0 (lower_rows)
+// PRE: W holds sqrt(alpha) L_s^-1 of the other side's rows and L_s^-1 b0 (lower_rows)
 template <int NPL, bool PRE>
 __global__ void __launch_bounds__(32 * kR1MaxWarps)
     row_rank1(const SweepArgs a, const float* __restrict__ lchol, const float* __restrict__ Tg,
@@ -354,14 +359,22 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
   float* vec = T + KP * LD + warp * r1_warp_floats(D, KP);
   float* Bp = vec + (D + 1) * KP;
   float* zb = Bp + D * KP;  // [kR1Rows][KP]
-  // per-element constants: b0 = Lambda_s mu_s (the bordered hyper matrix's
-  // last row) or L_s^-1 b0, the diagonal of Lambda_s and that of L_s squared
-  const float* b0 = PRE ? W + a.n_other * KP : a.lamaug + (int64_t)K * (K + 1);
+  // per-element constants: L_s^-1 b0 (b0 = Lambda_s mu_s, the bordered hyper
+  // matrix's last row), the diagonal of Lambda_s and that of L_s squared
   float bs[NPL], ds[NPL], ls2[NPL];
+  if (!PRE) {
+#pragma unroll
+    for (int m = 0; m < NPL; ++m) {
+      const int i = lane + 32 * m;
+      vec[i] = i < K ? __ldg(a.lamaug + (int64_t)K * (K + 1) + i) : 0.f;
+    }
+    __syncwarp();
+    lower_times<NPL, 1>(T, vec, K, lane);
+  }
 #pragma unroll
   for (int m = 0; m < NPL; ++m) {
     const int i = lane + 32 * m;
-    bs[m] = i < K ? __ldg(b0 + i) : 0.f;
+    bs[m] = i < K ? (PRE ? __ldg(W + a.n_other * KP + i) : vec[i]) : 0.f;
     ds[m] = i < K ? __ldg(a.lamaug + (int64_t)i * (K + 1) + i) : 0.f;
     const float l = i < K ? __ldg(lchol + tri(i) + i) : 1.f;
     ls2[m] = l * l;
@@ -403,17 +416,20 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
         drop |= 1u << r;
         continue;
       }
-      // x_t = sqrt(alpha) v_t, b = b0 + alpha sum_t r_t v_t, Lambda*_ii; with
-      // PRE, of L_s^-1 v_t in place of v_t (but for Lambda*_ii)
+      // Lambda*_ii, then w_t = L_s^-1 x_t and c = L_s^-1 b0 + sum_t sqrt(alpha)
+      // r_t w_t: the same operations in the same order whether the w_t were
+      // formed before or are formed here
       float b[NPL], d0[NPL];
 #pragma unroll
       for (int m = 0; m < NPL; ++m) {
         b[m] = bs[m];
         d0[m] = ds[m];
       }
+      // the ratings of the second pass, a lane each (d <= 32)
+      const float rl = !PRE && lane < d ? sa * __ldg(a.val + p0 + lane) : 0.f;
       for (int t = 0; t < d; ++t) {
         const int32_t j = __ldg(a.idx + p0 + t);
-        const float ar = a.alpha * __ldg(a.val + p0 + t);
+        const float sr = PRE ? sa * __ldg(a.val + p0 + t) : 0.f;
         const float* vj = a.Vo + (int64_t)j * K;
         const float* wj = PRE ? W + (int64_t)j * KP : nullptr;
 #pragma unroll
@@ -422,18 +438,22 @@ __global__ void __launch_bounds__(32 * kR1MaxWarps)
           const float v = i < K ? __ldg(vj + i) : 0.f;
           const float x = sa * v;
           d0[m] = fmaf(x, x, d0[m]);
-          const float w = PRE ? __ldg(wj + i) : v;
-          vec[t * KP + i] = sa * w;
-          b[m] = fmaf(ar, w, b[m]);
+          const float w = PRE ? __ldg(wj + i) : x;
+          vec[t * KP + i] = w;
+          if (PRE) b[m] = fmaf(sr, w, b[m]);
+        }
+      }
+      if (!PRE) {
+        __syncwarp();
+        lower_times_n<NPL>(T, vec, d, K, lane);
+        for (int t = 0; t < d; ++t) {
+          const float sr = __shfl_sync(kFull, rl, t);
+#pragma unroll
+          for (int m = 0; m < NPL; ++m) b[m] = fmaf(sr, vec[t * KP + lane + 32 * m], b[m]);
         }
       }
 #pragma unroll
       for (int m = 0; m < NPL; ++m) vec[d * KP + lane + 32 * m] = b[m];
-      if (!PRE) {
-        __syncwarp();
-        // w_t = L_s^-1 x_t and c = L_s^-1 b
-        lower_times_n<NPL>(T, vec, d + 1, K, lane);
-      }
       // the factors: p_s, then M_s^-1 applied to w_{s+1} .. w_{d-1} and to c
       float pr[NPL];  // prod_s rho_s^2 = (L_s)_ii^2 / L*_ii^2
 #pragma unroll
@@ -557,7 +577,7 @@ int launch_r1(const SweepArgs& a, const float* lchol, float* T, float* W, int D,
     const size_t smem = tbytes + sizeof(float) * kR1MaxWarps * 4 * KP;
     BPMF_TRY(r1_grid(lower_rows<NPL>, 32 * kR1MaxWarps, smem,
                      (a.n_other + 4 * kR1MaxWarps) / (4 * kR1MaxWarps), &grid));
-    lower_rows<NPL><<<grid, 32 * kR1MaxWarps, smem, st>>>(a.Vo, a.n_other, a.K,
+    lower_rows<NPL><<<grid, 32 * kR1MaxWarps, smem, st>>>(a.Vo, a.n_other, a.K, a.alpha,
                                                           a.lamaug + (int64_t)a.K * (a.K + 1), T, W);
     BPMF_CUDA_CHECK(cudaGetLastError());
   }

@@ -96,7 +96,8 @@ int launch_pieces_small(const SweepArgs& a, int64_t npieces, cudaStream_t st, in
 // rows row_begin..row_end of degree <= max_degree (<= kTinyDegreeMax) from
 // chol(Lambda_s) (rank1.cu); linvT is scratch of KP x (KP + 4) floats that the
 // call fills with (L_s^-1)^T first, pre scratch of rank1_pre_floats floats for
-// L_s^-1 of the other side's rows (nullptr: formed row by row)
+// sqrt(alpha) L_s^-1 of the other side's rows (nullptr: formed row by row, the
+// same draws bit for bit)
 int launch_rows_rank1(const SweepArgs& a, const float* lchol, float* linvT, float* pre,
                       int max_degree, cudaStream_t st, int64_t* launches);
 // floats of that scratch for a bin of `rows` rows with `ratings` ratings in all;
