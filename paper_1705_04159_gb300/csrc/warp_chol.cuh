@@ -193,6 +193,7 @@ __device__ __forceinline__ bool warp_cholesky(int g, float* T, const float* thr_
 #pragma unroll
     for (int i = 0; i < 8; ++i) ld8(D + trow(i), d[i]);
     ld8(thr_s + 8 * J, thr);
+    __syncwarp();  // every lane has loaded the tile that every lane writes below
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       // A failed pivot leaves NaN or inf in the rest of the factorisation,
