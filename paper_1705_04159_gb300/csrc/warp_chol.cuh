@@ -1,7 +1,7 @@
 // warp_chol.cuh -- one row's factorisation and draw by one warp, on 8 x 8 FP32
 // tiles in shared memory.
 //
-// The bordered matrix [[Lambda*, b], [b^T, c]] ((K + 1) x (K + 1), padded with
+// The bordered matrix [[Lambda*, b], [b^T, inf]] ((K + 1) x (K + 1), padded with
 // the identity to 8 g, lower triangle) lies as tiles (I, J), J <= I < g, at
 // kTileF (I (I + 1) / 2 + J); its factor's row K is y = L^-1 b, and the draw is
 // u = L^-T (y + z).
@@ -171,9 +171,9 @@ __device__ __forceinline__ void warp_panel(int r0, int nr, int J, float* T, cons
 
 // Left-looking Cholesky of g x g tiles (lower triangle) by one warp.  Returns false if a
 // pivot met the pivot rule of tile_chol.cuh (at or below thr, formed from its
-// starting diagonal; -inf on the bordered row K and on the
-// padding, which are never tested: row K's starting diagonal is set far above
-// any y^T y, so that its pivot is a positive number).  The diagonals
+// starting diagonal; -inf on the bordered row K and on the padding: row K's
+// starting diagonal is infinite, so its pivot is too, whatever y^T y it loses, with
+// the reciprocal root 0, and the padding keeps its ones).  The diagonals
 // themselves are not stored; rinv holds their reciprocals.
 __device__ __forceinline__ bool warp_cholesky(int g, float* T, const float* thr_s, float* rinv,
                                               int lane) {
@@ -319,13 +319,13 @@ __device__ __forceinline__ void warp_back(const SweepArgs& a, const float* T, co
 }
 
 // Element (i, j) of the base matrix: the lower triangle of the bordered
-// [[Lambda_s, b0], [b0^T, c]], identity on the padding past row K.  The corner
-// c, which no draw reads, is large, so that the factorisation passes row K
-// with a positive pivot.
+// [[Lambda_s, b0], [b0^T, inf]], identity on the padding past row K.  No draw reads
+// the corner; a finite one, 1e30, sent rows with alpha sum r^2 past it to the FP64
+// redo, by the NaN that the root of a negative pivot leaves in the padding.
 __device__ __forceinline__ float row_base(const SweepArgs& a, int i, int j) {
   const int K = a.K, KA = K + 1;
   if (i >= KA || j >= KA) return i == j ? 1.f : 0.f;
-  return j > i ? 0.f : i == K && j == K ? 1e30f : __ldg(a.lamaug + i * KA + j);
+  return j > i ? 0.f : i == K && j == K ? INFINITY : __ldg(a.lamaug + i * KA + j);
 }
 
 // Element (i, j) of base + alpha G from the Gram's; what the Gram holds in the
