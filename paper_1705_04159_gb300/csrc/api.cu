@@ -433,7 +433,8 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
       rc = BPMF_ECUDA;
       break;
     }
-    if ((rc = launch_spd_inverse_f64(d_W0, h->W0inv, K, h->wscr, h->status, h->stream))) break;
+    if ((rc = wish_cluster(K, &h->wish_ctas))) break;
+    if ((rc = launch_spd_inverse_f64(d_W0, h->W0inv, K, h->wish_ctas, h->wscr, h->status, h->stream))) break;
     if ((rc = check_status(h, "bpmf_init (W0)"))) {
       set_error("bpmf_init: W0 is not symmetric positive definite");
       rc = BPMF_EINVAL;

@@ -117,6 +117,7 @@ struct Handle {
   double* red = nullptr;    // reduction partials
   int64_t red_len = 0;
   double* wscr = nullptr;   // FP64 Wishart scratch (6 K*K + 8 K)
+  int wish_ctas = 0;        // CTAs of the draw's cluster (wish_cluster)
   // a second set of both, for the hyperparameter draw of the side that runs
   // second in an iteration: it runs on aux2 beside the first side's draw and
   // sweep (it reads only its own side's factors, which neither changes)
@@ -285,7 +286,10 @@ int set_thresholds(Handle* h, int s, const int64_t t[5]);  // binned.cu
 // On stream st (the handle's stream if null) with the second scratch set if
 // alt (see Handle::red2).
 int launch_hyper(Handle* h, int s, cudaStream_t st = nullptr, bool alt = false);
-int launch_spd_inverse_f64(const double* A, double* Ainv, int K, double* scratch, int* status,
+// CTAs of the cluster that the draws and the inverse of dimension K run on here
+// (their results do not depend on it)
+int wish_cluster(int K, int* ctas);
+int launch_spd_inverse_f64(const double* A, double* Ainv, int K, int ctas, double* scratch, int* status,
                            cudaStream_t st);
 int launch_check_spd_f64(const double* A, int K, int* status, float* lout, cudaStream_t st);
 int launch_hyper_to_f32(Handle* h, int s);

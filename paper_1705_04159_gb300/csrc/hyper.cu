@@ -625,7 +625,7 @@ int launch_hyper(Handle* h, int s, cudaStream_t st, bool alt) {
   a.gamma_cap = h->gamma_cap;
   {
     PhaseTimer timer(h, BPMF_T_HYPER_DRAW, st);
-    BPMF_TRY(launch_wishart(a, st, &h->kernels));
+    BPMF_TRY(launch_wishart(a, h->wish_ctas, st, &h->kernels));
   }
   sd.have_hyper = true;
   sd.have_stats = true;

@@ -26,7 +26,7 @@ struct HyperArgs {
   int gamma_cap;  // Gamma rejection attempts per draw before kStatusRng
 };
 
-// the whole draw: one kernel, one cluster of CTAs
-int launch_wishart(const HyperArgs& a, cudaStream_t st, int64_t* launches);
+// the whole draw: one kernel, one cluster of `ctas` CTAs (wish_cluster)
+int launch_wishart(const HyperArgs& a, int ctas, cudaStream_t st, int64_t* launches);
 
 }  // namespace gb

@@ -44,8 +44,18 @@ constexpr int kWishThreads = 256, kWishWarps = kWishThreads / 32;
 constexpr int kNpl = kMaxK / 32;
 constexpr unsigned kFull = 0xffffffffu;
 
-// CTAs of the cluster: one column of T a quarter SM for K <= 64, two up to 128
+// CTAs of the cluster: one column of T a quarter SM for K <= 64, two up to 128.
+// Past eight the size is not portable, and a device whose GPCs offer fewer SMs (a
+// partition of one) takes the largest half that fits (wish_cluster); the warps then
+// take their columns in several rounds.
 int wish_ctas(int K) { return K <= 16 ? 4 : K <= 32 ? 8 : 16; }
+
+// The column of T that a warp begins with: one a quarter SM (warps 0 - 3), then
+// the rest in reverse order, a short column to a long one; 8 nc further in each
+// round.
+__device__ __forceinline__ int first_column(int cta, int nc, int warp) {
+  return warp < 4 ? cta + nc * warp : 8 * nc - 1 - (cta + nc * (warp - 4));
+}
 
 __host__ __device__ inline int wish_packed(int K) { return (K * (K + 1) / 2 + 1) & ~1; }
 // the matrix, then B; A, then B scaled; a row of C per warp; (row, column) of the packed elements
@@ -291,7 +301,7 @@ __global__ void __launch_bounds__(kWishThreads, 1) spd_inverse(const double* A, 
   double* cbuf = M + 2 * wish_packed(K) + warp * K;
   uint16_t* ij = reinterpret_cast<uint16_t*>(M + 2 * wish_packed(K) + kWishWarps * K);
   double *gL = scr, *gT = scr + K * K, *gD = gT + K * K, *gok = gD + K;
-  const int j = warp < 4 ? cta + nc * warp : 8 * nc - 1 - (cta + nc * (warp - 4));
+  const int j0 = first_column(cta, nc, warp);
   if (cta == 0) {
     load_lower(A, K, M, ij);
     __syncthreads();
@@ -308,7 +318,7 @@ __global__ void __launch_bounds__(kWishThreads, 1) spd_inverse(const double* A, 
   copy_in(M, gL, np);
   for (int k = tid; k < K; k += kWishThreads) s_rr[k] = rsqrt(__ldcg(gD + k));
   __syncthreads();
-  if (j < K) {
+  for (int j = j0; j < K; j += 8 * nc) {
     switch ((K - j + 31) >> 5) {
       case 1: unit_solve<1>(M, K, j, s_rr, cbuf, lane); break;
       case 2: unit_solve<2>(M, K, j, s_rr, cbuf, lane); break;
@@ -317,11 +327,12 @@ __global__ void __launch_bounds__(kWishThreads, 1) spd_inverse(const double* A, 
     }
     __syncwarp();
     for (int q = lane; q < K - j; q += 32) gT[col_off(K, j) + q] = cbuf[K - 1 - j - q];
+    __syncwarp();
   }
   cluster_sync();
   copy_in(M, gT, np);
   __syncthreads();
-  if (j < K) {
+  for (int j = j0; j < K; j += 8 * nc) {
     // row i = K - 1 - j: entry (i, l), l <= i, is sum over k >= i of T[k][i] T[k][l]
     const int i = K - 1 - j;
     const double* ti = M + col_off(K, i);
@@ -384,9 +395,8 @@ __global__ void __launch_bounds__(kWishThreads, 1) wishart_draw(const HyperArgs 
   double* gB = gA + KK;
   double* gD = gL + 4 * KK;
   double* gok = gL + 5 * KK;
-  // The warp's column of T, and row of B and Lambda (K - 1 - j): one a quarter
-  // SM (warps 0 - 3), then the rest in reverse order, a short column to a long one.
-  const int wj = warp < 4 ? cta + nc * warp : 8 * nc - 1 - (cta + nc * (warp - 4));
+  // the warp's columns j of T, and rows K - 1 - j of B and Lambda, start here
+  const int j0 = first_column(cta, nc, warp);
   const double n = (double)a.n;
   const uint2 key = seed_key(a.seed);
   const uint32_t t = *a.tp;
@@ -449,8 +459,8 @@ __global__ void __launch_bounds__(kWishThreads, 1) wishart_draw(const HyperArgs 
     s_mus[k] = (a.beta0 * a.mu0[k] + n * a.xbar[k]) / bstar;
   }
   __syncthreads();
-  if (wj < K) {
-    const int j = wj, len = K - j;
+  for (int j = j0; j < K; j += 8 * nc) {
+    const int len = K - j;
     switch ((len + 31) >> 5) {
       case 1: unit_solve<1>(M, K, j, s_rr, cbuf, lane); break;
       case 2: unit_solve<2>(M, K, j, s_rr, cbuf, lane); break;
@@ -542,7 +552,7 @@ __global__ void __launch_bounds__(kWishThreads, 1) wishart_draw(const HyperArgs 
     }
     if (lane == 0) a.lamaug[K * KA + K] = 0.f;
   }
-  if (wj < K) {
+  for (int wj = j0; wj < K; wj += 8 * nc) {
     const int i = K - 1 - wj;
     const double* bi = B + i * (i + 1) / 2;
     double b0 = 0.0;
@@ -582,23 +592,30 @@ __global__ void __launch_bounds__(kWishThreads, 1) wishart_draw(const HyperArgs 
 
 namespace {
 
-// kern on one cluster of wish_ctas(K) CTAs
-template <typename... P, typename... A>
-int launch_cluster(void (*kern)(P...), int K, cudaStream_t st, A... args) {
-  const int smem = wish_smem(K);
+// The launch of kern on one cluster of `ctas` CTAs.
+template <typename... P>
+int cluster_config(void (*kern)(P...), int K, int ctas, cudaStream_t st, cudaLaunchConfig_t* cfg,
+                   cudaLaunchAttribute* at) {
   BPMF_TRY(allow_smem(kern, wish_smem(kMaxK)));
   BPMF_CUDA_CHECK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)wish_ctas(K));
-  cfg.blockDim = dim3(kWishThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
+  *cfg = {};
+  cfg->gridDim = dim3((unsigned)ctas);
+  cfg->blockDim = dim3(kWishThreads);
+  cfg->dynamicSmemBytes = wish_smem(K);
+  cfg->stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = cfg->gridDim.x;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+  return BPMF_OK;
+}
+
+template <typename... P, typename... A>
+int launch_cluster(void (*kern)(P...), int K, int ctas, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cfg.gridDim.x;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  BPMF_TRY(cluster_config(kern, K, ctas, st, &cfg, &at));
   BPMF_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kern, args...));
   BPMF_CUDA_CHECK(cudaGetLastError());
   return BPMF_OK;
@@ -606,15 +623,31 @@ int launch_cluster(void (*kern)(P...), int K, cudaStream_t st, A... args) {
 
 }  // namespace
 
-int launch_wishart(const HyperArgs& a, cudaStream_t st, int64_t* launches) {
-  BPMF_TRY(launch_cluster(wishart_draw, a.K, st, a));
+int wish_cluster(int K, int* ctas) {
+  for (int n = wish_ctas(K); n >= 2; n /= 2) {  // a draw needs two: the factorisation's and Bartlett's
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    int fit = 0;
+    BPMF_TRY(cluster_config(wishart_draw, K, n, nullptr, &cfg, &at));
+    if (cudaOccupancyMaxActiveClusters(&fit, wishart_draw, &cfg) == cudaSuccess && fit > 0) {
+      *ctas = n;
+      return BPMF_OK;
+    }
+    cudaGetLastError();
+  }
+  set_error("wishart: the device holds no cluster of two CTAs for K = %d", K);
+  return BPMF_ECUDA;
+}
+
+int launch_wishart(const HyperArgs& a, int ctas, cudaStream_t st, int64_t* launches) {
+  BPMF_TRY(launch_cluster(wishart_draw, a.K, ctas, st, a));
   if (launches) *launches += 1;
   return BPMF_OK;
 }
 
-int launch_spd_inverse_f64(const double* A, double* Ainv, int K, double* scratch, int* status,
+int launch_spd_inverse_f64(const double* A, double* Ainv, int K, int ctas, double* scratch, int* status,
                            cudaStream_t st) {
-  return launch_cluster(spd_inverse, K, st, A, Ainv, K, scratch, status);
+  return launch_cluster(spd_inverse, K, ctas, st, A, Ainv, K, scratch, status);
 }
 
 int launch_check_spd_f64(const double* A, int K, int* status, float* lout, cudaStream_t st) {
