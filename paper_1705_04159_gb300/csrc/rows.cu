@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(160) row_fp32(const SweepArgs a) {
     }
   }
   __syncthreads();
-  if (tid < 32) row_draw(a, G.g, T, thr, thr + G.KP, thr + 2 * G.KP, row, tid);
+  if (tid < 32) row_draw<2>(a, G.g, T, thr, thr + G.KP, thr + 2 * G.KP, row, tid);
 }
 
 // Partial Gram of one piece of a split row, stored as raw tiles.

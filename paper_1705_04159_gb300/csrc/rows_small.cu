@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(kHubThreads) hub_draw(const SweepArgs a) {
     }
   }
   __syncthreads();
-  if (threadIdx.x < 32) row_draw(a, g, T, thr, rinv, zv, a.rows ? a.rows[slot] : (int)slot, threadIdx.x);
+  if (threadIdx.x < 32) row_draw<2>(a, g, T, thr, rinv, zv, a.rows ? a.rows[slot] : (int)slot, threadIdx.x);
 }
 
 template <int g, bool B>

@@ -9,9 +9,16 @@
 // The factorisation is left-looking by block columns J of eight columns:
 //   update: A_IJ -= sum_{p<J} L_Ip L_Jp^T for all row tiles I >= J, on the
 //     tensor cores by mma.m16n8k8 (two row tiles at a time) with FP32 operands
-//     split into two TF32 parts, x = h + l: h h^T in one FP32 accumulator and
-//     h l^T + l h^T in another (l l^T, at most 2^-22 relative, is dropped), so only
-//     the p-sums of like size meet in an accumulator;
+//     split into two TF32 parts, x = h + l: h h^T in one or two FP32 accumulators
+//     and h l^T + l h^T in another (l l^T, at most 2^-22 relative, is dropped), so
+//     only the p-sums of like size meet in an accumulator.  The tensor core's sums
+//     round towards zero: over the 16 steps of K = 128 one accumulator's bias put a
+//     draw up to 1.33 times as far from FP64 as FP32 multiply-adds (rms, K >= 88, 8 to
+//     64 ratings under a well-conditioned prior), two in turn, each of half the
+//     steps and half the size, at most 0.96 times.  K <= 55, where one stays within
+//     1.0 times, and the persistent kernel, whose bf16 Gram sets its error (1.00 times;
+//     rows without ratings 0.6 to 0.96), take one (W): with two there, 50,000 x 12,000
+//     with 2.5M ratings, K = 64, 2,309 -> 2,397 us for two iterations;
 //   diagonal tile: Cholesky in registers by every lane;
 //   panel: the rows below by substitution, a lane per row.
 // A tile is 8 rows of 8 floats (trow), and a lane's fragment of an operand or
@@ -86,12 +93,13 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
 }
 
 // A_IJ -= sum_{p<J} L_Ip L_Jp^T for the 2 NPR row tiles I = I0 .. (those below
-// g; pairs wholly past it compute on the last tile and store nothing).  The
-// next step's fragments are loaded as soon as the current ones are split, so
-// after the last step they are those of column J itself.
-template <int NPR>
+// g; pairs wholly past it compute on the last tile and store nothing), the
+// steps p taking W accumulators in turn.  The next step's fragments are loaded as
+// soon as the current ones are split, so after the last step they are those of
+// column J itself.
+template <int NPR, int W>
 __device__ __forceinline__ void warp_update(float* T, int g, int J, int I0, int fo) {
-  float acc[NPR][4], cross[NPR][4];
+  float acc[W][NPR][4], cross[NPR][4];
   float2 fu[NPR], fv[NPR];
   float *pu[NPR], *pv[NPR];
 #pragma unroll
@@ -102,44 +110,55 @@ __device__ __forceinline__ void warp_update(float* T, int g, int J, int I0, int 
     fu[i] = ldf2(pu[i]);
     fv[i] = ldf2(pv[i]);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[i][q] = cross[i][q] = 0.f;
+    for (int q = 0; q < 4; ++q) {
+      cross[i][q] = 0.f;
+#pragma unroll
+      for (int w = 0; w < W; ++w) acc[w][i][q] = 0.f;
+    }
   }
   const float* pb = T + tidx(J, 0) * kTileF + fo;
   float2 b = ldf2(pb);
   int off = 0;
 #pragma unroll 1
-  for (int p = 0; p < J; ++p) {
-    off += kTileF;
-    uint32_t bh0, bl0, bh1, bl1;
-    split_tf32(b.x, bh0, bl0);
-    split_tf32(b.y, bh1, bl1);
-    b = ldf2(pb + off);
-    uint32_t l[NPR][4];
+  for (int p = 0; p < J; p += W) {
 #pragma unroll
-    for (int i = 0; i < NPR; ++i) {
-      uint32_t h0, h1, h2, h3;
-      split_tf32(fu[i].x, h0, l[i][0]);
-      split_tf32(fv[i].x, h1, l[i][1]);
-      split_tf32(fu[i].y, h2, l[i][2]);
-      split_tf32(fv[i].y, h3, l[i][3]);
-      fu[i] = ldf2(pu[i] + off);
-      fv[i] = ldf2(pv[i] + off);
-      mma_tf32(acc[i], h0, h1, h2, h3, bh0, bh1);
-      mma_tf32(cross[i], h0, h1, h2, h3, bl0, bl1);
+    for (int w = 0; w < W; ++w) {
+      if (w > 0 && p + w >= J) break;
+      off += kTileF;
+      uint32_t bh0, bl0, bh1, bl1;
+      split_tf32(b.x, bh0, bl0);
+      split_tf32(b.y, bh1, bl1);
+      b = ldf2(pb + off);
+      uint32_t l[NPR][4];
+#pragma unroll
+      for (int i = 0; i < NPR; ++i) {
+        uint32_t h0, h1, h2, h3;
+        split_tf32(fu[i].x, h0, l[i][0]);
+        split_tf32(fv[i].x, h1, l[i][1]);
+        split_tf32(fu[i].y, h2, l[i][2]);
+        split_tf32(fv[i].y, h3, l[i][3]);
+        fu[i] = ldf2(pu[i] + off);
+        fv[i] = ldf2(pv[i] + off);
+        mma_tf32(acc[w][i], h0, h1, h2, h3, bh0, bh1);
+        mma_tf32(cross[i], h0, h1, h2, h3, bl0, bl1);
+      }
+#pragma unroll
+      for (int i = 0; i < NPR; ++i)
+        mma_tf32(cross[i], l[i][0], l[i][1], l[i][2], l[i][3], bh0, bh1);
     }
-#pragma unroll
-    for (int i = 0; i < NPR; ++i)
-      mma_tf32(cross[i], l[i][0], l[i][1], l[i][2], l[i][3], bh0, bh1);
   }
 #pragma unroll
   for (int i = 0; i < NPR; ++i) {
     const int I = I0 + 2 * i;
-    if (I < g)
-      *reinterpret_cast<float2*>(pu[i] + off) =
-          make_float2(fu[i].x - (acc[i][0] + cross[i][0]), fu[i].y - (acc[i][1] + cross[i][1]));
-    if (I + 1 < g)
-      *reinterpret_cast<float2*>(pv[i] + off) =
-          make_float2(fv[i].x - (acc[i][2] + cross[i][2]), fv[i].y - (acc[i][3] + cross[i][3]));
+    float s[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s[q] = cross[i][q];
+#pragma unroll
+      for (int w = W - 1; w >= 0; --w) s[q] = acc[w][i][q] + s[q];
+    }
+    if (I < g) *reinterpret_cast<float2*>(pu[i] + off) = make_float2(fu[i].x - s[0], fu[i].y - s[1]);
+    if (I + 1 < g) *reinterpret_cast<float2*>(pv[i] + off) = make_float2(fv[i].x - s[2], fv[i].y - s[3]);
   }
 }
 
@@ -175,6 +194,7 @@ __device__ __forceinline__ void warp_panel(int r0, int nr, int J, float* T, cons
 // starting diagonal is infinite, so its pivot is too, whatever y^T y it loses, with
 // the reciprocal root 0, and the padding keeps its ones).  The diagonals
 // themselves are not stored; rinv holds their reciprocals.
+template <int W>
 __device__ __forceinline__ bool warp_cholesky(int g, float* T, const float* thr_s, float* rinv,
                                               int lane) {
   bool fail = false;
@@ -184,8 +204,8 @@ __device__ __forceinline__ bool warp_cholesky(int g, float* T, const float* thr_
     if (J > 0) {
       int I0 = J;
 #pragma unroll 1
-      for (; g - I0 > 2; I0 += 4) warp_update<2>(T, g, J, I0, fo);
-      if (g - I0 > 0) warp_update<1>(T, g, J, I0, fo);
+      for (; g - I0 > 2; I0 += 4) warp_update<2, W>(T, g, J, I0, fo);
+      if (g - I0 > 0) warp_update<1, W>(T, g, J, I0, fo);
       __syncwarp();
     }
     float* D = T + tidx(J, J) * kTileF;
@@ -337,13 +357,14 @@ __device__ __forceinline__ float row_elem(const SweepArgs& a, int i, int j, floa
 
 // One warp factors the tiles and draws the row, or leaves it to the FP64 redo;
 // zv has room for K rounded up to 4.
+template <int W = 1>
 __device__ __forceinline__ void row_draw(const SweepArgs& a, int g, float* T, const float* thr,
                                          float* rinv, float* zv, int row, int lane) {
   const uint32_t tw = *a.tp;
   for (int q = lane; 4 * q < a.K; q += 32)
     *reinterpret_cast<float4*>(zv + 4 * q) =
         normal4_f32(philox(make_uint4((uint32_t)row, tw, (uint32_t)q, a.sw), a.key));
-  const bool ok = warp_cholesky(g, T, thr, rinv, lane);
+  const bool ok = warp_cholesky<W>(g, T, thr, rinv, lane);
   if (ok) warp_back(a, T, rinv, zv, row, lane);
   else if (lane == 0) a.flag_rows[atomicAdd(a.flag_count, 1)] = row;
 }
