@@ -16,7 +16,13 @@
 //     formed from zero and then added in FP32: the tensor core's accumulator
 //     rounds towards zero, which over many steps would add up to a bias (over
 //     1,024 neighbours 1e-5 of the sum; by the step 2.0e-7, FP32 multiply-adds
-//     one after the other 5.1e-7).  The staged row stride is an odd multiple of
+//     one after the other 5.1e-7).  The two parts keep 23 of an operand's 24 bits and
+//     l l is left out, which a row of a few ratings and a small K shows: its draw was
+//     up to 1.3 times as far from FP64 as with FP32 multiply-adds (rms; 1.0 times
+//     at 12 ratings, 0.6 at 100, any number at K >= 24).  So for K <= 23 rows of up
+//     to 16 ratings, and the pieces of a hub up to 64 for K <= 15 (they add up in
+//     FP32), take multiply-adds (sm_few): 100,000 rows of 14 ratings, K = 16, 273 ->
+//     292 us, of 6 ratings 268 -> 273.  The staged row stride is an odd multiple of
 //     eight floats, so the fragments (features 8 I + lane / 4 of neighbours
 //     lane % 4 and + 4) load without bank conflicts;
 //   the factorisation and the draw: warp_chol.cuh.
@@ -49,8 +55,9 @@ namespace gb {
 namespace {
 
 constexpr int kSmWarps = 4;   // warps (rows) per CTA
-// CTAs per SM the registers are cut for: 128 a thread, 168 where the Gram takes up to 76
-constexpr int sm_ctas(int g) { return g <= 5 ? 4 : 3; }
+// CTAs per SM the registers are cut for: 80 to 128 a thread without spills, 168
+// where the Gram takes up to 76
+constexpr int sm_ctas(int g) { return g <= 3 ? 6 : g == 4 ? 5 : g == 5 ? 4 : 3; }
 constexpr int kSmMaxG = 7;    // K <= 55
 
 // g tile rows, the last of them row K alone if B (K = 8 (g - 1)): the Gram's
@@ -68,6 +75,8 @@ struct SmGeom {
   // neighbours staged at a time; 32 of seven tile rows would leave the L1 32 KB
   // (K = 50: 744 us instead of 732, K = 32: 331 instead of 340)
   static constexpr int kChunk = G < 7 ? 32 : 16;
+  // up to so many neighbours of a row, and of a piece, by FP32 multiply-adds (sm_few)
+  static constexpr int kFew = g <= 3 ? 16 : 0, kFewPiece = g <= 2 ? 64 : kFew;
   static constexpr int kRows = 2 * kChunk * LDT;    // staged rows, then ratings if B
   static constexpr int kStage = kRows + (B ? 2 * kChunk : 0);
   // per warp: staging buffers, reused by the tiles; thresholds, 1 / diagonal, z
@@ -127,6 +136,41 @@ __device__ __forceinline__ void mma_tf32_zero(float (&d)[4], uint32_t a0, uint32
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
+// o += x x^T of n staged neighbours by FP32 multiply-adds, neighbour by
+// neighbour (X0: the first one's row, zeros past n up to a multiple of four); if
+// B, s as sm_step forms it
+template <int g, bool B>
+__device__ __forceinline__ void sm_few(const float* X0, const float* R, int n, int lane,
+                                       float (&o)[SmGeom<g, B>::NA][4], float (&s)[SmGeom<g, B>::G]) {
+  using S = SmGeom<g, B>;
+  const int t = lane & 3;
+  const float *xr = X0 + (lane >> 2), *xc = X0 + 2 * t;
+#pragma unroll 1
+  for (int e0 = 0; e0 < n; e0 += 4, xr += 4 * S::LDT, xc += 4 * S::LDT) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      float x[S::G];
+#pragma unroll
+      for (int I = 0; I < S::G; ++I) x[I] = xr[e * S::LDT + 8 * I];
+#pragma unroll
+      for (int J = 0; J < S::G; ++J) {
+        const float2 y = ldf2(xc + e * S::LDT + 8 * J);
+#pragma unroll
+        for (int I = J; I < S::G; ++I) {
+          float(&d)[4] = o[(I >> 1) * ((I >> 1) + 1) + J];
+          d[2 * (I & 1)] = fmaf(x[I], y.x, d[2 * (I & 1)]);
+          d[2 * (I & 1) + 1] = fmaf(x[I], y.y, d[2 * (I & 1) + 1]);
+        }
+      }
+      if (B && e == t) {  // a lane in four keeps the sum of a neighbour
+        const float r = R[e0];
+#pragma unroll
+        for (int I = 0; I < S::G; ++I) s[I] = fmaf(r, x[I], s[I]);
+      }
+    }
+  }
+}
+
 // o += sum over eight staged neighbours of x x^T (lower tiles, in pairs); if
 // B, s += their r x (R: their ratings; a lane's own two neighbours only)
 template <int g, bool B>
@@ -174,7 +218,7 @@ __device__ __forceinline__ void sm_step(const float* X, const float* R, float (&
 
 // o (and s) = sums over ratings [e0, e1)
 template <int g, bool B, int V>
-__device__ __forceinline__ void sm_gram_v(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int lane,
+__device__ __forceinline__ void sm_gram_v(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int few, int lane,
                                           float (&o)[SmGeom<g, B>::NA][4], float (&s)[SmGeom<g, B>::G]) {
   using S = SmGeom<g, B>;
   constexpr int kBuf = S::kChunk * S::LDT;
@@ -215,14 +259,18 @@ __device__ __forceinline__ void sm_gram_v(const SweepArgs& a, float* T, int64_t 
     __syncwarp();
     const float *Xb = X + buf * kBuf, *Rb = R + buf * S::kChunk;
     const int cnt = count(c0);
+    if (n <= few) {
+      sm_few<g, B>(T + buf * kBuf, Rb, cnt, lane, o, s);
+    } else {
 #pragma unroll 1
-    for (int k = 0; k < cnt; k += 8) sm_step<g, B>(Xb + k * S::LDT, Rb + k, o, s);
+      for (int k = 0; k < cnt; k += 8) sm_step<g, B>(Xb + k * S::LDT, Rb + k, o, s);
+    }
     __syncwarp();  // the buffer is refilled next
   }
 }
 
 template <int g, bool B>
-__device__ __forceinline__ void sm_gram(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int lane,
+__device__ __forceinline__ void sm_gram(const SweepArgs& a, float* T, int64_t e0, int64_t e1, int few, int lane,
                                         float (&o)[SmGeom<g, B>::NA][4], float (&s)[SmGeom<g, B>::G]) {
   using S = SmGeom<g, B>;
 #pragma unroll
@@ -232,7 +280,7 @@ __device__ __forceinline__ void sm_gram(const SweepArgs& a, float* T, int64_t e0
 #pragma unroll
   for (int i = 0; i < S::G; ++i) s[i] = 0.f;
   if constexpr (B) {
-    sm_gram_v<g, B, 4>(a, T, e0, e1, lane, o, s);
+    sm_gram_v<g, B, 4>(a, T, e0, e1, few, lane, o, s);
     // over the four lanes that share a feature
 #pragma unroll
     for (int i = 0; i < S::G; ++i) {
@@ -247,9 +295,9 @@ __device__ __forceinline__ void sm_gram(const SweepArgs& a, float* T, int64_t e0
         if (c > a.K) T[e * S::LDT + c] = 0.f;
     }
     __syncwarp();
-    if ((a.K & 3) == 0) sm_gram_v<g, B, 4>(a, T, e0, e1, lane, o, s);
-    else if ((a.K & 1) == 0) sm_gram_v<g, B, 2>(a, T, e0, e1, lane, o, s);
-    else sm_gram_v<g, B, 1>(a, T, e0, e1, lane, o, s);
+    if ((a.K & 3) == 0) sm_gram_v<g, B, 4>(a, T, e0, e1, few, lane, o, s);
+    else if ((a.K & 1) == 0) sm_gram_v<g, B, 2>(a, T, e0, e1, few, lane, o, s);
+    else sm_gram_v<g, B, 1>(a, T, e0, e1, few, lane, o, s);
   }
 }
 
@@ -273,7 +321,7 @@ __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) row_small(const Swe
   float* zv = rinv + S::KP;
   {
     float o[S::NA][4], s[S::G];
-    sm_gram<g, B>(a, T, a.ptr[row], a.ptr[row + 1], lane, o, s);
+    sm_gram<g, B>(a, T, a.ptr[row], a.ptr[row + 1], S::kFew, lane, o, s);
     // A = base + alpha G as tiles, over the staging buffers
     const int gr = lane >> 2, t2 = 2 * (lane & 3), fo = trow(gr) + t2;
 #pragma unroll
@@ -322,7 +370,7 @@ __global__ void __launch_bounds__(32 * kSmWarps, sm_ctas(g)) piece_small(const S
   const int64_t pc = (int64_t)blockIdx.x * kSmWarps + warp;
   if (pc >= npieces) return;
   float o[S::NA][4], s[S::G];
-  sm_gram<g, B>(a, ssm + warp * S::kStage, a.piece_e0[pc], a.piece_e1[pc], lane, o, s);
+  sm_gram<g, B>(a, ssm + warp * S::kStage, a.piece_e0[pc], a.piece_e1[pc], S::kFewPiece, lane, o, s);
   float* dst = a.part + pc * S::NT * 64 + 2 * lane;
 #pragma unroll
   for (int k = 0; k < S::NP; ++k)
