@@ -129,9 +129,9 @@ __global__ void __launch_bounds__(32 * kFinalWarps) colsum_final(
 // warp's 16-byte loads fall on different banks.  Chunks are copied by cp.async
 // into a ring of kScatStages stages; a thread centres what it copied itself
 // (always the same columns, so it keeps their means) before the one barrier of
-// the chunk.  The S subsets' FP32 sums meet in shared memory, in the order r = 0,
-// 1, .., and go to the block's FP64 partial: at the end, and often enough that
-// no FP32 accumulator sums more than kScatFlushRows rows.
+// the chunk.  The S subsets' FP32 sums are added in FP32 in shared memory, in the
+// order r = 0, 1, .., and go to the block's FP64 partial: at the end, and often
+// enough that no FP32 accumulator sums more than kScatFlushRows rows.
 // What bounds it: the FP32 multiply-adds, with their shared-memory loads close
 // behind.  480,189 rows by 64 blocks, K = 64: 552 us with 4 x 4 tiles, a
 // centring pass with a division an element and two barriers a chunk, 287 now
@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(NT, 2) scatter_partial(const float* __restrict
     }
     first = false;
   };
-  const int64_t flush_chunks = max(1, kScatFlushRows * S / kScatRows);
+  const int64_t flush_chunks = max(1, kScatFlushRows / ((kScatRows + S - 1) / S));  // rows of a subset a chunk
   for (int c = 0; c < kScatStages - 1; ++c) issue(c);
   for (int64_t c = 0; c < nchunks; ++c) {
     cp_async_wait<kScatStages - 2>();  // chunk c has landed (this thread's copies)
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) scatter_small(const float* _
 #pragma unroll
       for (int b = 0; b < TM; ++b) acc[a][b] = 0.f;
   };
-  const int flush_chunks = max(1, kSmallFlushRows * S / ROWS);
+  const int flush_chunks = max(1, kSmallFlushRows / ((ROWS + S - 1) / S));  // rows of a subset a chunk
   for (int c = 0; c < kScatStages - 1; ++c) issue(c);
   int nchunk = 0;
   for (int64_t c = 0; c < nchunks; ++c) {
