@@ -129,9 +129,11 @@ __global__ void __launch_bounds__(32 * kFinalWarps) colsum_final(
 // warp's 16-byte loads fall on different banks.  Chunks are copied by cp.async
 // into a ring of kScatStages stages; a thread centres what it copied itself
 // (always the same columns, so it keeps their means) before the one barrier of
-// the chunk.  The S subsets' FP32 sums are added in FP32 in shared memory, in the
-// order r = 0, 1, .., and go to the block's FP64 partial: at the end, and often
-// enough that no FP32 accumulator sums more than kScatFlushRows rows.
+// the chunk.  The S subsets' FP32 sums are added in FP32 in shared memory, in a
+// fixed order of four chains (one chain of the 17 subsets of K = 33 .. 40 put S up
+// to 1.2 times as far from FP64 as the six subsets of 4 x 4 tiles), and go to the
+// block's FP64 partial: at the end, and often enough that no FP32 accumulator sums
+// more than kScatFlushRows rows.
 // What bounds it: the FP32 multiply-adds, with their shared-memory loads close
 // behind.  480,189 rows by 64 blocks, K = 64: 552 us with 4 x 4 tiles, a
 // centring pass with a division an element and two barriers a chunk, 287 now
@@ -241,12 +243,20 @@ __global__ void __launch_bounds__(NT, 2) scatter_partial(const float* __restrict
       for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
     __syncthreads();
     for (int e = tid; e < 16 * T; e += NT) {
-      float4 s = sums[e];
-#pragma unroll 4
-      for (int k = 1; k < S; ++k) {
-        const float4 x = sums[k * 16 * T + e];
-        s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+      float4 s4[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) s4[u] = u < S ? sums[u * 16 * T + e] : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int k = 4; k < S; k += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (k + u < S) {
+            const float4 x = sums[(k + u) * 16 * T + e];
+            s4[u].x += x.x; s4[u].y += x.y; s4[u].z += x.z; s4[u].w += x.w;
+          }
+        }
       }
+      const float4 s = make_float4((s4[0].x + s4[1].x) + (s4[2].x + s4[3].x), (s4[0].y + s4[1].y) + (s4[2].y + s4[3].y),
+                                   (s4[0].z + s4[1].z) + (s4[2].z + s4[3].z), (s4[0].w + s4[1].w) + (s4[2].w + s4[3].w));
       const int v = e / T, p = v >> 1, t = e - v * T;
       int ti = 0;
       while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
