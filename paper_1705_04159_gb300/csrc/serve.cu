@@ -80,8 +80,9 @@ int64_t job_bytes(const Job& j, int num_sms) {
   b += j.n_test * (4 + 4 + 4 + 8);                  // test set and running sums
   b += (j.nnz / 2048 + 16) * (K + 8) * (K + 8) * 4; // split-row partial Grams
   b += j.nnz * 32 + (j.M + j.N) * 16;               // sort and copy buffers of bpmf_init
-  for (const int64_t n : {j.M, j.N})                // L^-1 of the other side's rows (tiny rows)
-    b += rank1_pre_floats((int)K, n, j.M + j.N - n, j.nnz) * 4;
+  // L^-1 of the other side's rows, where a row with ratings can be in the tiny bin
+  if (j.cfg.path != BPMF_PATH_PLAIN && (j.cfg.tiny_max > 0 || (j.cfg.tiny_max < 0 && j.cfg.autotune)))
+    for (const int64_t n : {j.M, j.N}) b += rank1_pre_floats((int)K, n, j.M + j.N - n, j.nnz) * 4;
   return b + (8LL << 20);
 }
 
