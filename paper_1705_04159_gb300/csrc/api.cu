@@ -123,7 +123,62 @@ void carve_handle(Handle* h, Carve& c) {
   h->d_navg = c.take<int64_t>(1);
 }
 
+// Doubles of the reduction partials.
+int64_t red_length(int K, int num_sms) {
+  return std::max<int64_t>({2LL * num_sms * K * K, 2LL * num_sms * K, 16LL * num_sms + 1024, 4096});
+}
+
+// The test set's arrays.
+void carve_test(Handle* h, int64_t n, Carve& k) {
+  h->trow = k.take<int32_t>(n);
+  h->tcol = k.take<int32_t>(n);
+  h->tval = k.take<float>(n);
+  h->tsum = k.take<float2>(n);
+}
+
+// Scratch of bpmf_init beside the ratings from the host: what the structure
+// takes or, after it, the factors of the autotuner's sweeps.
+size_t init_work_bytes(int64_t M, int64_t N, int64_t nnz, const bpmf_config& cfg) {
+  return std::max(structure_bytes(nnz, M, N),
+                  cfg.autotune ? sizeof(float) * (size_t)(std::max(M, N) * cfg.K) : 0);
+}
+
 }  // namespace
+
+int64_t sampler_bytes(int64_t M, int64_t N, int64_t nnz, int64_t n_test, const bpmf_config& cfg, int num_sms) {
+  Handle h;
+  h.M = M;
+  h.N = N;
+  h.nnz = nnz;
+  h.K = cfg.K;
+  h.cfg = cfg;
+  h.side[BPMF_USERS].R = M;
+  h.side[BPMF_MOVIES].R = N;
+  h.red_len = red_length(cfg.K, num_sms);
+  Carve held, init, test;
+  carve_handle(&h, held);
+  if (n_test > 0) carve_test(&h, n_test, held);
+  // pieces of both sides and the partials of one: at most a piece per plen
+  // ratings and one more per hub
+  const int64_t hub = cfg.hub_min >= 0 ? std::max(1, cfg.hub_min) : cfg.autotune ? kTuneHubMin : 2 * kPiece;
+  const int64_t pieces = nnz / piece_length(hub) + nnz / hub + 1;
+  for (int s = 0; s < 2; ++s) {
+    held.take<int64_t>(2 * pieces);
+    held.take<int32_t>(2 * pieces);
+  }
+  held.take<float>(nnz >= hub ? pieces * partial_floats_per_piece(cfg.K) : 0);
+  // L^-1 of the other side's rows, where a row with ratings can be in the tiny bin
+  if (cfg.path != BPMF_PATH_PLAIN && (cfg.tiny_max > 0 || (cfg.tiny_max < 0 && cfg.autotune)))
+    for (const int64_t n : {M, N}) held.take<float>(rank1_pre_floats(cfg.K, n, M + N - n, nnz));
+  // scratch, released before the call returns
+  for (int i = 0; i < 3; ++i) {
+    init.take<int32_t>(nnz);
+    test.take<int32_t>(n_test);
+  }
+  init.take<char>((int64_t)init_work_bytes(M, N, nnz, cfg));
+  test.take<char>((int64_t)test_sort_bytes(n_test));
+  return (int64_t)(held.bytes + std::max(init.bytes, test.bytes));
+}
 
 // Reads and clears the device status word; maps bits to a status code.
 int check_status(Handle* h, const char* where) {
@@ -395,8 +450,7 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
     h->side[BPMF_USERS].R = M;
     h->side[BPMF_MOVIES].R = N;
     const int64_t KK = (int64_t)K * K;
-    h->red_len = std::max<int64_t>({2LL * h->num_sms * KK, 2LL * h->num_sms * K,
-                                    16LL * h->num_sms + 1024, 4096});
+    h->red_len = red_length(K, h->num_sms);
     {
       Carve size, c;
       carve_handle(h, size);
@@ -441,10 +495,7 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
       break;
     }
     // ratings
-    // scratch: the ratings if they come from the host, then what the structure
-    // takes or, after it, the factors of the autotuner's sweeps
-    const size_t work = std::max(structure_bytes(nnz, M, N),
-                                 cfg->autotune ? sizeof(float) * (size_t)(std::max(M, N) * K) : 0);
+    const size_t work = init_work_bytes(M, N, nnz, *cfg);
     char* ws = nullptr;
     for (int pass = 0; pass < 2 && rc == BPMF_OK; ++pass) {
       Carve c;
@@ -522,10 +573,7 @@ int bpmf_set_test(bpmf_t* hh, int64_t n, const int32_t* row, const int32_t* col,
       ws = c.take<char>((int64_t)test_sort_bytes(n));
       Carve k;  // kept
       k.base = h->tblock;
-      h->trow = k.take<int32_t>(n);
-      h->tcol = k.take<int32_t>(n);
-      h->tval = k.take<float>(n);
-      h->tsum = k.take<float2>(n);
+      carve_test(h, n, k);
       if (pass == 0 && (rc = dalloc(&scratch, (int64_t)c.bytes)) == BPMF_OK)
         rc = dalloc(&h->tblock, (int64_t)k.bytes);
     }

@@ -190,8 +190,7 @@ int apply_bins(Handle* h, int s, int64_t tiny_max, int64_t light_max, int64_t hu
     }
   }
   if (new_hubs) {
-    // piece length: half the hub threshold, at most kPiece ratings
-    const int64_t plen = std::max<int64_t>(1, std::min<int64_t>(kPiece, hub_min / 2));
+    const int64_t plen = piece_length(hub_min);
     std::vector<int32_t> prow, hub0;
     std::vector<int64_t> pe0, pe1;
     for (int64_t q = 0; q < n_hub; ++q) {
@@ -448,8 +447,8 @@ int autotune_bins(Handle* h, int s, float* scratch) {
   const bool tune_cons = !sd.heavy_tc && h->cfg.path == BPMF_PATH_MIXED && ws_supported(h->K) && sd.Xhi;
   const int64_t maxdeg = sd.deg_h.empty() ? 0 : sd.deg_h[0];
   std::vector<int64_t> hubs;
-  if (h->cfg.hub_min < 0 && maxdeg >= 2048) {
-    for (int64_t v : {(int64_t)2048, (int64_t)4096, (int64_t)8192, (int64_t)16384, (int64_t)1 << 40})
+  if (h->cfg.hub_min < 0 && maxdeg >= kTuneHubMin) {
+    for (int64_t v : {kTuneHubMin, (int64_t)4096, (int64_t)8192, (int64_t)16384, (int64_t)1 << 40})
       if (v == (int64_t)1 << 40 || v <= maxdeg) hubs.push_back(v);
   } else {
     hubs.push_back(sd.hub_min);

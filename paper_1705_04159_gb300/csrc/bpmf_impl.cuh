@@ -309,6 +309,8 @@ int launch_advance_iter(Handle* h);
 
 // api.cu
 void set_error(const char* fmt, ...);
+// Device bytes of a sampler while it is built and while it runs: an upper estimate
+int64_t sampler_bytes(int64_t M, int64_t N, int64_t nnz, int64_t n_test, const bpmf_config& cfg, int num_sms);
 int step_async(Handle* h);          // one iteration queued on h->stream, no wait
 int check_status(Handle* h, const char* where);  // waits for the stream, maps device status
 

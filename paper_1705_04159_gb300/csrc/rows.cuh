@@ -8,7 +8,13 @@
 namespace gb {
 
 constexpr int kChunk = 32;          // neighbour rows staged per pipeline step
-constexpr int64_t kPiece = 4096;    // ratings per piece of a split (hub) row
+constexpr int64_t kPiece = 4096;    // ratings per piece of a split (hub) row, at most
+constexpr int64_t kTuneHubMin = 2048;  // least hub threshold that the autotuner tries
+// ratings per piece: half the hub threshold
+inline int64_t piece_length(int64_t hub_min) {
+  const int64_t half = hub_min / 2;
+  return half < 1 ? 1 : half < kPiece ? half : kPiece;
+}
 
 struct SweepArgs {
   const int64_t* ptr;   // row pointers of this side

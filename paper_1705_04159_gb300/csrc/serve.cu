@@ -33,7 +33,6 @@
 #include <vector>
 
 #include "bpmf_impl.cuh"
-#include "rows.cuh"
 
 namespace gb {
 namespace {
@@ -66,24 +65,10 @@ struct Job {
   bpmf_job_result res{};
 };
 
-// Device bytes a job holds while resident (structure, factors, hyper state,
-// scratch, test set) plus the transient peak of its initialisation.
+// Device bytes a job holds while resident and at the transient peak of its
+// initialisation, with some room for its graph and events.
 int64_t job_bytes(const Job& j, int num_sms) {
-  const int64_t K = j.cfg.K, KK = K * K;
-  int64_t b = 0;
-  b += 2 * j.nnz * 8;                               // idx + val, both sides
-  b += (j.M + j.N) * (8 + 4 + 4 * K + 8);           // ptr, perm, X, bins
-  b += 2 * (KK * 8 * 2 + (K + 1) * (K + 1) * 4 + KK * 4 + K * 16);
-  b += 2 * std::max<int64_t>(2LL * num_sms * KK, 16LL * num_sms + 1024) * 8;  // reduction partials (two sets)
-  b += 2 * (6 * KK + 8 * K) * 8;                    // Wishart scratch (two sets)
-  b += std::max(j.M, j.N) * 4;                      // flagged rows
-  b += j.n_test * (4 + 4 + 4 + 8);                  // test set and running sums
-  b += (j.nnz / 2048 + 16) * (K + 8) * (K + 8) * 4; // split-row partial Grams
-  b += j.nnz * 32 + (j.M + j.N) * 16;               // sort and copy buffers of bpmf_init
-  // L^-1 of the other side's rows, where a row with ratings can be in the tiny bin
-  if (j.cfg.path != BPMF_PATH_PLAIN && (j.cfg.tiny_max > 0 || (j.cfg.tiny_max < 0 && j.cfg.autotune)))
-    for (const int64_t n : {j.M, j.N}) b += rank1_pre_floats((int)K, n, j.M + j.N - n, j.nnz) * 4;
-  return b + (8LL << 20);
+  return sampler_bytes(j.M, j.N, j.nnz, j.n_test, j.cfg, num_sms) + (8LL << 20);
 }
 
 double now_s(std::chrono::steady_clock::time_point t0) {
