@@ -507,7 +507,11 @@ int bpmf_init(bpmf_t** out, int64_t M, int64_t N, int64_t nnz, const int32_t* ro
       if (pass == 0) rc = dalloc(&scratch, (int64_t)c.bytes);
     }
     if (rc) break;
-    if ((rc = build_structure(h, d_row, d_col, d_val, ws))) break;
+    if ((rc = build_structure(h, d_row, d_col, d_val, ws))) break;  // waits for its work
+    if (!cfg->autotune) {  // before the bins' own memory is taken
+      dfree(scratch);
+      scratch = nullptr;
+    }
     if ((rc = setup_bins(h, BPMF_USERS))) break;
     if ((rc = setup_bins(h, BPMF_MOVIES))) break;
     if ((rc = launch_init_factors(h, BPMF_USERS))) break;
