@@ -238,8 +238,9 @@ int read_fp64_rows(Handle* h, int s) {
 // the iteration word advances.  The second side's hyperparameter draw reads
 // only that side's factors, which the first side's draw and sweep leave
 // alone, so it runs on aux2 beside them (with its own scratch) and joins
-// before the second sweep: the one-CTA FP64 draws of the two sides overlap,
-// and the second side's reductions fill SMs the first side leaves idle.
+// before the second sweep: the FP64 draws of the two sides, a cluster of 4 to
+// 16 CTAs each, overlap, and the second side's reductions fill SMs the first side
+// leaves idle.
 // Everything that changes from one iteration to the next lives in device
 // memory, so the same launches serve every iteration.
 int step_body(Handle* h) {
