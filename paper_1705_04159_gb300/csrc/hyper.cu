@@ -138,7 +138,11 @@ __global__ void __launch_bounds__(32 * kFinalWarps) colsum_final(
 // behind.  480,189 rows by 64 blocks, K = 64: 552 us with 4 x 4 tiles, a
 // centring pass with a division an element and two barriers a chunk, 287 now
 // (chunks of 32 rows 330, and 361 with 288 threads in 96 registers);
-// by 26 blocks, K = 100: 2,078 (8 x 8 tiles) -> 1,528.  TF32 tensor-core products,
+// by 26 blocks, K = 100: 2,078 (8 x 8 tiles) -> 1,528 (64 and 26 blocks are the
+// allocation-free entry point's, at most one an SM; an iteration's up to 304: both
+// sides' reductions of a 480,189 x 17,770 one, K = 100, 800 -> 520).  Two CTAs share an
+// SM up to K = 112; past it the ring takes 120 KB and more, and the registers are
+// cut for two all the same.  TF32 tensor-core products,
 // split in two and summed in FP32 every eight rows, took 205 us at K = 64 but
 // their truncated sums doubled the error (2.8e-8 rms of the scale, here 1.5e-8).
 constexpr int kScatStages = 4;

@@ -111,7 +111,8 @@ constexpr int kWsMaxCons = 7;
 // K = 72 sides averaging kWsWideRow ratings or more lose (K = 64, 208 a row: 1%).  A
 // row much longer than the others is copied by one SM at the pace of its ring:
 // sides with one of more than kWsWideMax ratings keep eight stages
-// (ChEMBL-shaped, K = 64: 1,320 us against 1,328).
+// (ChEMBL-shaped, K = 64: 1,320 us against 1,328; not measured with such rows at
+// K >= 72, where eight stages leave far fewer consumers).
 constexpr int kWsWideCons = 11, kWsWideK = 64, kWsWideAllK = 72;
 constexpr int64_t kWsWideRow = 128, kWsWideMax = 1024;
 constexpr int kWsRecs = 32;          // row records in flight: >= stages + accumulators + 1
